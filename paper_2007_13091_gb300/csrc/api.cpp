@@ -148,6 +148,7 @@ void layout(const MeshHost& mh, int64_t cap, size_t rs, bool with_e, Carver& c, 
     M.bf_f = c.take<float>(11 * (nbf ? nbf : 1));
     M.lsq_c = c.take<double>(12 * nc);
     M.lsq_dxf = c.take<double>(12 * nc);
+    M.f_dx = c.take<double>(6 * nf);
     M.eps2 = c.take<double>(nc);
     M.f_lk = c.take<int32_t>(nf);
     M.f_own = c.take<int32_t>(nf);
@@ -184,8 +185,7 @@ void layout(const MeshHost& mh, int64_t cap, size_t rs, bool with_e, Carver& c, 
     S.wacc = c.take<int64_t>(5 * nc);
     S.mom = c.take<double>(5 * nc);
     S.F = c.take<double>(5 * nf);
-    S.gradW = c.take<double>(15 * nc);
-    S.gradH = c.take<double>(3 * nc);
+    S.rec = c.take<double>(REC_N * nc);
     S.bsum = c.take<int2>((size_t)scan_blocks(mh.nc) + 1);
     S.t = c.take<double>(1);
     S.dt = c.take<double>(1);
@@ -453,7 +453,7 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
     // image of the centroid; grad = sum_k c_k (v_k - v_i) with
     // c_k = A^-1 w_k dx_k, A = sum_k w_k dx_k dx_k^T.  Also the centroid-to-face
     // vectors and epsilon^2 = (K |Omega|^(1/3))^3 of Venkatakrishnan's limiter.
-    std::vector<double> lsq_c(12 * (size_t)nc), lsq_dxf(12 * (size_t)nc), eps2(nc);
+    std::vector<double> lsq_c(12 * (size_t)nc), lsq_dxf(12 * (size_t)nc), eps2(nc), fdx(6 * (size_t)nf, 0.0);
     std::vector<int32_t> flk(nf, 0);
     for (int i = 0; i < nc; ++i) {
         double xi[3] = {0.0, 0.0, 0.0};
@@ -465,7 +465,10 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
             const int f = mh.cf[4 * (size_t)i + k];
             const bool own = mh.cf_sign[4 * (size_t)i + k] > 0;
             const double* xf = &mh.f_c[3 * (size_t)f];
-            for (int d = 0; d < 3; ++d) lsq_dxf[(size_t)(3 * k + d) * nc + i] = xf[d] - xi[d];
+            for (int d = 0; d < 3; ++d) {
+                lsq_dxf[(size_t)(3 * k + d) * nc + i] = xf[d] - xi[d];
+                fdx[(size_t)((own ? 0 : 3) + d) * nf + f] = xf[d] - xi[d];
+            }
             const int j = own ? mh.f_nbr[f] : mh.f_own[f];
             if (j >= 0) {
                 for (int d = 0; d < 3; ++d) {
@@ -639,6 +642,7 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
     UP(s->M.bf_f, bff.data(), bff.size() * sizeof(float));
     UP(s->M.lsq_c, lsq_c.data(), lsq_c.size() * sizeof(double));
     UP(s->M.lsq_dxf, lsq_dxf.data(), lsq_dxf.size() * sizeof(double));
+    UP(s->M.f_dx, fdx.data(), fdx.size() * sizeof(double));
     UP(s->M.eps2, eps2.data(), eps2.size() * sizeof(double));
     UP(s->M.f_lk, flk.data(), flk.size() * sizeof(int32_t));
     UP(s->M.f_own, mh.f_own.data(), nf * sizeof(int32_t));
@@ -834,7 +838,10 @@ int enqueue_gks_step(ugkwp_sim* s, int32_t mode) {
     if (P.order == 2)
         timed(s, UGKWP_K_GRADIENTS, 1, q, [&] { launch_gradients(s->M, s->S, P, q); });
     if (P.order == 2)
-        timed(s, UGKWP_K_FLUX_O2, 1, q, [&] { launch_face_flux_o2(s->M, s->S, P, s->lc.wave_blocks, q); });
+        // nothing runs beside the flux in these steps: as many blocks as fit
+        timed(s, UGKWP_K_FLUX_O2, 1, q, [&] {
+            launch_face_flux_o2(s->M, s->S, P, std::max(s->lc.wave_blocks, 2 * sm_count()), q);
+        });
     else
         timed(s, UGKWP_K_FLUX, 1, q, [&] { launch_face_flux(s->M, s->S, P, 0, 0, q); });
     timed(s, UGKWP_K_UPDATE, 1, q, [&] { launch_cell_update(s->M, s->S, P, nullptr, q); });
@@ -1342,8 +1349,14 @@ int ugkwp_last(ugkwp_sim* s, int32_t which, void* host_out) {
         case 9:
         case 10:
             if (s->P.order != 2) return fail(UGKWP_E_ARG, "gradients exist only at order 2");
-            if (which == 9) CU(get(s->S.gradW, 15 * nc * 8));
-            else CU(get(s->S.gradH, 3 * nc * 8));
+            {
+                // the gradients sit in the cells' rows after W and rho^h
+                std::vector<double> v(REC_N * nc);
+                CU(cudaMemcpy(v.data(), s->S.rec, REC_N * nc * 8, cudaMemcpyDeviceToHost));
+                const size_t first = which == 9 ? 6 : 21, n = which == 9 ? 15 : 3;
+                for (size_t j = 0; j < n; ++j)
+                    for (size_t i = 0; i < nc; ++i) ((double*)host_out)[j * nc + i] = v[REC_N * i + first + j];
+            }
             break;
         default: return fail(UGKWP_E_ARG, "unknown diagnostic");
     }
@@ -1694,18 +1707,18 @@ int enqueue_chunk_step(FusedChunk& ch, const std::vector<ugkwp_sim*>& sims) {
     c.n = (int32_t)ch.idx.size();
     const LaunchCfg lc = sims[ch.idx[0]]->lc;
     const int sms = sm_count();
-    std::vector<long long> w6(c.n), wf(c.n);
+    std::vector<long long> wc(c.n), wf(c.n);
     std::vector<int> need_grad(c.n), need_o2(c.n), need_o1(c.n);
     for (int i = 0; i < c.n; ++i) {
         ugkwp_sim* s = sims[ch.idx[i]];
         c.mem[i] = BatchMember{s->M, s->S, s->P, s->A, s->B, s->Mv};
-        w6[i] = 6LL * s->M.nc;
+        wc[i] = s->M.nc;
         wf[i] = s->M.nf;
-        need_grad[i] = (int)((6LL * s->M.nc + gradient_threads() - 1) / gradient_threads());
+        need_grad[i] = (s->M.nc + gradient_threads() - 1) / gradient_threads();
         need_o2[i] = (s->M.nf + wave_threads() - 1) / wave_threads();
         need_o1[i] = (s->M.nf + 255) / 256;
     }
-    const std::vector<int> b_grad = split_blocks(4 * sms, w6, need_grad);
+    const std::vector<int> b_grad = split_blocks(gradient_blocks_per_sm() * sms, wc, need_grad);
     const std::vector<int> b_o2 = split_blocks(lc.wave_blocks, wf, need_o2);
     const std::vector<int> b_o1 = split_blocks(lc.wave_blocks, wf, need_o1);
     for (int k = 0; k < BCL_N; ++k) c.off[k][0] = 0;

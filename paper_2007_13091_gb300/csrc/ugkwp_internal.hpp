@@ -57,6 +57,9 @@ enum : int {
 // Tiles taken from the tile counter per atomic.
 constexpr int TILE_GRAB = 4;
 
+// Values of a cell's row in DevState::rec.
+constexpr int REC_N = 24;
+
 struct DevBc {
     int32_t type;
     int32_t pad;
@@ -123,6 +126,7 @@ struct DevMesh {
     // second-order reconstruction (order 2)
     const double* lsq_c;     // [12][nc]: gradient = sum_k c_k (v_k - v_i), c_k at [(3k+d) nc + i]
     const double* lsq_dxf;   // [12][nc]: face centroid minus cell centroid for local face k
+    const double* f_dx;      // [6][nf] face centroid minus the owner's, the neighbour's centroid
     const double* eps2;      // [nc] Venkatakrishnan epsilon^2 = (K h)^3
     const int32_t* f_lk;     // [nf] owner's local face | neighbour's local face << 2
     const int32_t* face_order;  // [nf] interior faces, then boundary faces grouped by type
@@ -184,8 +188,8 @@ struct DevState {
     int64_t* wacc;        // [5][nc] fixed-point scratch for W^p
     double* mom;          // [5][nc] staging of moments copied to the host
     double* F;            // [5][nf]
-    double* gradW;        // [15][nc] limited gradients of W, [(3q+d) nc + i] (order 2)
-    double* gradH;        // [3][nc] limited gradient of rho^h (order 2)
+    double* rec;          // [nc][REC_N] order 2: what a face reads of a cell: W (5), rho^h, the limited
+                          // gradients of W [3q + d] (15) and of rho^h (3)
     int2* bsum;           // [n_scan_blocks] block sums of (count, N_sam)
     double* t;            // [1]
     double* dt;           // [1]
@@ -319,7 +323,8 @@ static_assert(sizeof(BatchChunk) <= 32764, "a chunk must fit a launch's paramete
 int blocks_reset(int nc);        // grid of one simulation's reset launch
 int blocks_cells(int nc);        // one thread per cell, 256 per block
 int blocks_gp_coef(int nc);      // one thread per cell, 128 per block
-int gradient_threads();          // threads per block of the gradient kernel
+int gradient_threads();          // threads per block of the gradient kernel (one per cell)
+int gradient_blocks_per_sm();    // its persistent grid
 void launch_reset_batch(const BatchChunk& c, int blocks, cudaStream_t st);
 void launch_cell_prep_batch(const BatchChunk& c, int blocks, cudaStream_t st);
 void launch_sample_count_batch(const BatchChunk& c, int blocks, cudaStream_t st);
