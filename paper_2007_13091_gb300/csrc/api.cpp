@@ -1364,31 +1364,30 @@ int ugkwp_last(ugkwp_sim* s, int32_t which, void* host_out) {
 }
 
 // Device scratch of the adjoint for K steps: checkpoints of W (K + 1), the
-// recorded rho^p (K) and particle fluxes (5 K), time steps, fluxes, face
-// terms, two adjoint states, face products and per-step sums.
+// recorded rho^p (K) and particle fluxes (5 K), time steps, fluxes, boundary
+// faces' terms, two adjoint states, the faces' rows of products and per-step sums.
 static void adjoint_layout(const ugkwp_sim* s, int K, Carver& c, double** ck, double** rp, double** pf, double** dt,
-                           double** F, double** jf, double** lam0, double** lam1, double** wbar, double** thbar,
+                           double** F, double** jf, double** lam0, double** lam1, double** fb, double** thbar,
                            double** sums, double** theta, AdjO2* o2) {
-    const size_t nc = s->M.nc, nf = s->M.nf;
+    // (terms of boundary faces: at least one slot, a mesh without any is not excluded)
+    const size_t nc = s->M.nc, nf = s->M.nf, nbf = std::max(s->M.nbf, 1);
     std::memset(o2, 0, sizeof(*o2));
     if (s->P.order == 2) {  // limiter values of every step, and scratch
         o2->phi = c.take<double>((size_t)K * 6 * nc);
-        o2->gW = c.take<double>(15 * nc);
-        o2->gH = c.take<double>(3 * nc);
-        o2->gbar = c.take<double>(36 * nf);
+        o2->rec = c.take<double>(REC_N * nc);
         o2->gg = c.take<double>(18 * nc);
-        o2->thc = c.take<double>(3 * nc);
+        o2->thc = c.take<double>(3 * nbf);
     }
     *ck = c.take<double>((size_t)(K + 1) * 5 * nc);
     *rp = c.take<double>((size_t)K * nc);
     *pf = c.take<double>((size_t)K * 5 * nc);
     *dt = c.take<double>((size_t)K);
     *F = c.take<double>(5 * nf);
-    *jf = c.take<double>(nf);
+    *jf = c.take<double>(nbf);
     *lam0 = c.take<double>(5 * nc);
     *lam1 = c.take<double>(5 * nc);
-    *wbar = c.take<double>(10 * nf);
-    *thbar = c.take<double>(3 * nf);
+    *fb = c.take<double>(2 * adjoint_face_row(s->P.order) * nf);
+    *thbar = c.take<double>(3 * nbf);
     *sums = c.take<double>((size_t)4 * K);
     *theta = c.take<double>(3);
 }
@@ -1449,9 +1448,9 @@ int ugkwp_adjoint_wave(ugkwp_sim* s, const ugkwp_adjoint_req* r, double* out) {
     const double th_h[3] = {r->theta ? r->theta[0] : theta0[0], r->theta ? r->theta[1] : theta0[1],
                             r->theta ? r->theta[2] : theta0[2]};
     Carver c(r->d_workspace);
-    double *ck, *rp, *pf, *dtv, *F, *jf, *lam0, *lam1, *wbar, *thbar, *sums, *theta;
+    double *ck, *rp, *pf, *dtv, *F, *jf, *lam0, *lam1, *fb, *thbar, *sums, *theta;
     AdjO2 o2;
-    adjoint_layout(s, K, c, &ck, &rp, &pf, &dtv, &F, &jf, &lam0, &lam1, &wbar, &thbar, &sums, &theta, &o2);
+    adjoint_layout(s, K, c, &ck, &rp, &pf, &dtv, &F, &jf, &lam0, &lam1, &fb, &thbar, &sums, &theta, &o2);
     auto step_o2 = [&](int n) {
         AdjO2 t = o2;
         if (t.phi) t.phi += (size_t)n * 6 * (size_t)s->M.nc;
@@ -1483,7 +1482,7 @@ int ugkwp_adjoint_wave(ugkwp_sim* s, const ugkwp_adjoint_req* r, double* out) {
     double* cur = lam0;
     for (int n = K - 1; n >= 0; --n) {
         launch_adj_reverse(s->M, s->P, ap, ck + (size_t)n * 5 * nc, rp + (size_t)n * nc, dth[n], theta, step_o2(n), next,
-                           cur, wbar, thbar, sums + K + 3 * (size_t)n, q);
+                           cur, fb, thbar, sums + K + 3 * (size_t)n, q);
         std::swap(next, cur);
     }
     CU(cudaGetLastError());

@@ -1,5 +1,5 @@
-// Adjoint of the wave part of the step with the particle part frozen (first
-// order; Sec. 2.1, 2.3, 2.4 (d), (e)).
+// Adjoint of the wave part of the step with the particle part frozen (Sec. 2.1,
+// 2.3, 2.4 (d), (e)).
 //
 // Frozen map: with the recorded time steps dt^n, particle densities rho^p_n
 // (rho^h = rho - rho^p) and particle fluxes pf^n of K real steps,
@@ -10,474 +10,26 @@
 // equal to the first one (density, speed along its direction, its own
 // temperature) and the temperature of the listed diffuse walls.
 //
-// Reverse sweep (hand-written adjoint): lambda^K = 0 and for n = K-1..0
+// Reverse sweep: lambda^K = 0 and for n = K-1..0
 //   g_f      = -|S_f|/|Omega_o| lambda^{n+1}_o + |S_f|/|Omega_nb| lambda^{n+1}_nb
 //              + |S_f| e_c  (listed boundary faces),
 //   lambda^n = lambda^{n+1} + sum_f (dF_f/dW^n)^T g_f,
 //   dJ/dtheta += sum_f (dF_f/dtheta)^T g_f.
-// Face states are recomputed from the checkpointed W^n; each face's local
-// vector-Jacobian products come from evaluating its flux on dual numbers
-// seeded on the owner's W, the neighbour's W and theta in turn.  Per-face
-// products are gathered per cell in the fixed order of the cell's faces.
-#include "dual.cuh"
+// Face states are recomputed from the checkpointed W^n; each face's products
+// with its local Jacobians come from the hand-written reverse pass of the face's
+// flux (wave_math.cuh), one evaluation for all inputs, where forward-mode duals
+// took two (first order) or ten (second order) evaluations of five directions
+// each.  A face writes the products of each side as one row; a cell gathers its
+// faces' rows in their fixed order.
+//
+// Bound by the binary64 pipe.  Measured per step (channels of 40,500 and 20,736
+// tets): first order @O1@, second order @O2@.
+#include "recon.cuh"
 #include "ugkwp_internal.hpp"
 
 namespace ugkwp {
 
 namespace {
-
-using ad::Dual;
-constexpr double PI = 3.14159265358979323846;
-
-// generic elementary functions: binary64 or dual
-__device__ __forceinline__ double sqrt_(double x) { return ::sqrt(x); }
-__device__ __forceinline__ double exp_(double x) { return ::exp(x); }
-__device__ __forceinline__ double log_(double x) { return ::log(x); }
-__device__ __forceinline__ double expm1_(double x) { return ::expm1(x); }
-__device__ __forceinline__ double erfc_(double x) { return ::erfc(x); }
-__device__ __forceinline__ double fabs_(double x) { return ::fabs(x); }
-template <int N> __device__ __forceinline__ Dual<N> sqrt_(const Dual<N>& x) { return ad::sqrt(x); }
-template <int N> __device__ __forceinline__ Dual<N> exp_(const Dual<N>& x) { return ad::exp(x); }
-template <int N> __device__ __forceinline__ Dual<N> log_(const Dual<N>& x) { return ad::log(x); }
-template <int N> __device__ __forceinline__ Dual<N> expm1_(const Dual<N>& x) { return ad::expm1(x); }
-template <int N> __device__ __forceinline__ Dual<N> erfc_(const Dual<N>& x) { return ad::erfc(x); }
-template <int N> __device__ __forceinline__ Dual<N> fabs_(const Dual<N>& x) { return ad::fabs(x); }
-
-template <class S> struct Prim { S rho, U[3], p, T, lam; };
-
-template <class S> __device__ Prim<S> prim_of(const S* W, double R) {
-    Prim<S> s;
-    s.rho = W[0];
-    const S ir = 1.0 / W[0];
-    for (int d = 0; d < 3; ++d) s.U[d] = W[1 + d] * ir;
-    const S U2 = s.U[0] * s.U[0] + s.U[1] * s.U[1] + s.U[2] * s.U[2];
-    s.p = (W[4] - 0.5 * (s.rho * U2)) * (2.0 / 3.0);
-    s.T = s.p / (s.rho * R);
-    s.lam = s.rho / (2.0 * s.p);
-    return s;
-}
-
-// mu(T)/p with mu = mu_ref (T/T_ref)^omega
-template <class S> __device__ S tau_of(const S& T, const S& p, const DevParams& P) {
-    return P.mu_ref * exp_(P.omega * log_(T * (1.0 / P.T_ref))) / p;
-}
-
-// q1, q4 and a4 = q4 - dt e^{-dt/tau}
-template <class S> __device__ void coeffs(double dt, const S& tau, S& q1, S& q4, S& a4) {
-    const S x = dt / tau;
-    if (ad::val(x) < 1.0) {
-        S s1 = 0.0, s4 = 0.0, sa = 0.0, term = 1.0;
-        for (int k = 1; k <= 30; ++k) {
-            term = term * x * (1.0 / (double)k);
-            const double sg = (k & 1) ? -1.0 : 1.0;
-            if (k >= 2) s1 = s1 + sg * term;
-            s4 = s4 - sg * term;
-            if (k >= 2) sa = sa + (sg * (double)(k - 1)) * term;
-        }
-        q1 = tau * s1;
-        q4 = tau * s4;
-        a4 = tau * sa;
-    } else {
-        const S em1 = expm1_(-x);
-        q4 = -(tau * em1);
-        q1 = dt - q4;
-        a4 = q4 - dt * (em1 + 1.0);
-    }
-}
-
-// unit-density half-space (half = +1/-1) or full (0) moments <psi>, <u_n psi>
-template <class S> __device__ void moments(const S& Un, const S* Ut, const double* n, const S& lam, int half, S H[5],
-                                           S G[5]) {
-    S M[5];
-    if (half == 0) {
-        M[0] = 1.0;
-        M[1] = Un;
-    } else {
-        const S a = sqrt_(lam) * Un;
-        const S edge = 0.5 * exp_(-(lam * Un * Un)) / sqrt_(PI * lam);
-        if (half > 0) { M[0] = 0.5 * erfc_(-a); M[1] = Un * M[0] + edge; }
-        else          { M[0] = 0.5 * erfc_(a);  M[1] = Un * M[0] - edge; }
-    }
-    const S h = 0.5 / lam;
-    for (int k = 0; k < 3; ++k) M[k + 2] = Un * M[k + 1] + (double)(k + 1) * h * M[k];
-    const S tv = Ut[0] * Ut[0] + Ut[1] * Ut[1] + Ut[2] * Ut[2] + 2.0 * h;
-    H[0] = M[0];
-    G[0] = M[1];
-    for (int d = 0; d < 3; ++d) {
-        H[1 + d] = M[1] * n[d] + M[0] * Ut[d];
-        G[1 + d] = M[2] * n[d] + M[1] * Ut[d];
-    }
-    H[4] = 0.5 * (M[2] + M[0] * tv);
-    G[4] = 0.5 * (M[3] + M[1] * tv);
-}
-
-template <class S> struct Side { S rho, rhoh, Un, Ut[3], lam, p, T; };
-
-template <class S> __device__ Side<S> side_of(const S* W, const S& rhoh, const double* n, double R) {
-    const Prim<S> s = prim_of(W, R);
-    Side<S> f;
-    f.rho = s.rho; f.rhoh = rhoh; f.lam = s.lam; f.p = s.p; f.T = s.T;
-    f.Un = s.U[0] * n[0] + s.U[1] * n[1] + s.U[2] * n[2];
-    for (int d = 0; d < 3; ++d) f.Ut[d] = s.U[d] - f.Un * n[d];
-    return f;
-}
-
-// F = q1 <u_n psi>_{g0} + a4 (upwind hydrodynamic halves); a ghost that
-// emits no particles carries q4 on its incoming half
-template <class S> __device__ void interior(const Side<S>& L, const Side<S>& R, bool ghost, const double* n, double dt,
-                                            const DevParams& P, S F[5]) {
-    S HL[5], GL[5], HR[5], GR[5];
-    moments(L.Un, L.Ut, n, L.lam, +1, HL, GL);
-    moments(R.Un, R.Ut, n, R.lam, -1, HR, GR);
-    S W0[5];
-    for (int q = 0; q < 5; ++q) W0[q] = L.rho * HL[q] + R.rho * HR[q];
-    const Prim<S> s0 = prim_of(W0, P.R);
-    S tau = tau_of(s0.T, s0.p, P);
-    if (P.C2 > 0.0) tau = tau + P.C2 * fabs_(L.p - R.p) / fabs_(L.p + R.p) * dt;
-    S q1, q4, a4;
-    coeffs(dt, tau, q1, q4, a4);
-    const S Un0 = s0.U[0] * n[0] + s0.U[1] * n[1] + s0.U[2] * n[2];
-    S Ut0[3];
-    for (int d = 0; d < 3; ++d) Ut0[d] = s0.U[d] - Un0 * n[d];
-    S H0[5], G0[5];
-    moments(Un0, Ut0, n, s0.lam, 0, H0, G0);
-    const S cR = ghost ? q4 : a4;
-    for (int k = 0; k < 5; ++k) F[k] = q1 * (s0.rho * G0[k]) + a4 * (L.rhoh * GL[k]) + cR * (R.rhoh * GR[k]);
-}
-
-// Flux of face f from the owner's W (and the neighbour's, or the boundary
-// condition parameterised by theta).
-template <class S> __device__ void face_flux(const DevMesh& m, const DevParams& P, const AdjParams& ap, int f,
-                                             const S* WL, double rpL, const S* WR, double rpR, const S* th, double dt,
-                                             S F[5]) {
-    const int nf = m.nf;
-    const double n[3] = {m.f_n[f], m.f_n[nf + f], m.f_n[2 * nf + f]};
-    const S rhohL = WL[0] - rpL;
-    const Side<S> L = side_of(WL, rhohL, n, P.R);
-    const int nb = m.f_nbr[f];
-    if (nb >= 0) {
-        const S rhohR = WR[0] - rpR;
-        const Side<S> R = side_of(WR, rhohR, n, P.R);
-        interior(L, R, false, n, dt, P, F);
-        return;
-    }
-    const int tag = m.bf_tag[-1 - nb];
-    const DevBc& bc = P.bc[tag];
-    const AdjBc& ab = ap.b[tag];
-    if (bc.type == UGKWP_BC_DIFFUSE_WALL) {
-        const S tauL = tau_of(L.T, L.p, P);
-        S q1, q4, a4;
-        coeffs(dt, tauL, q1, q4, a4);
-        S HL[5], GL[5];
-        moments(L.Un, L.Ut, n, L.lam, +1, HL, GL);
-        S Gin[5];
-        for (int k = 0; k < 5; ++k) Gin[k] = q1 * (L.rho * GL[k]) + a4 * (L.rhoh * GL[k]);
-        const S Tw = ab.param_wall ? th[2] : S(bc.T_w);
-        const S lamw = 1.0 / (2.0 * P.R * Tw);
-        const double Uwn = bc.U_w[0] * n[0] + bc.U_w[1] * n[1] + bc.U_w[2] * n[2];
-        S Uwt[3];
-        for (int d = 0; d < 3; ++d) Uwt[d] = bc.U_w[d] - Uwn * n[d];
-        S Hw[5], Gw[5];
-        moments(S(Uwn), Uwt, n, lamw, -1, Hw, Gw);
-        const S rhow = -Gin[0] / (dt * Gw[0]);
-        for (int k = 0; k < 5; ++k) F[k] = Gin[k] + dt * rhow * Gw[k];
-        return;
-    }
-    if (bc.type == UGKWP_BC_SPECULAR) {
-        Side<S> R = L;
-        R.Un = -L.Un;
-        S Ff[5];
-        interior(L, R, false, n, dt, P, Ff);
-        const S fn = Ff[1] * n[0] + Ff[2] * n[1] + Ff[3] * n[2];
-        F[0] = 0.0;
-        F[4] = 0.0;
-        for (int d = 0; d < 3; ++d) F[1 + d] = fn * n[d];
-        return;
-    }
-    Side<S> R = L;
-    if (bc.type == UGKWP_BC_FARFIELD) {
-        S Win[5];
-        if (ab.param_ff) {
-            Win[0] = th[0];
-            for (int d = 0; d < 3; ++d) Win[1 + d] = th[0] * th[1] * ab.e[d];
-            Win[4] = th[0] * (0.5 * th[1] * th[1] + 1.5 * ab.RT);
-        } else {
-            for (int q = 0; q < 5; ++q) Win[q] = bc.W_in[q];
-        }
-        R = side_of(Win, Win[0], n, P.R);
-    }
-    R.rhoh = R.rho;
-    interior(L, R, true, n, dt, P, F);
-}
-
-// ---- second order, generic (Sec. 2.1, 2.3): interior faces of a step whose
-// limited least-squares gradients are given (their limiter values frozen),
-// in the closed forms of the second-order kernel, on binary64 or duals.
-template <class S> struct TabS { S n[7], v[7], w[7]; };
-
-template <class S> __device__ void gauss_mom_s(const S& mean, const S& h, S* M) {
-    M[0] = S(1.0);
-    M[1] = mean;
-    for (int k = 0; k < 5; ++k) M[k + 2] = mean * M[k + 1] + ((double)(k + 1) * h) * M[k];
-}
-
-template <class S> __device__ void make_tab_s(const S* U, const S& lam, int half, TabS<S>& T) {
-    const S h = 0.5 / lam;
-    if (half == 0) {
-        gauss_mom_s(U[0], h, T.n);
-    } else {
-        const S a = sqrt_(lam) * U[0];
-        const S edge = (0.5 * exp_(-(a * a))) / sqrt_(PI * lam);
-        T.n[0] = half > 0 ? 0.5 * erfc_(-a) : 0.5 * erfc_(a);
-        T.n[1] = U[0] * T.n[0] + (half > 0 ? edge : -edge);
-        for (int k = 0; k < 5; ++k) T.n[k + 2] = U[0] * T.n[k + 1] + ((double)(k + 1) * h) * T.n[k];
-    }
-    gauss_mom_s(U[1], h, T.v);
-    gauss_mom_s(U[2], h, T.w);
-}
-
-// <u^AL v^BE w^GA (a.psi) psi_k>, factorised per direction
-template <int AL, int BE, int GA, class S> __device__ void apsi_s(const TabS<S>& T, const S* a, S out[5]) {
-    const S h4 = 0.5 * a[4];
-    S NA[3], VA[3], WA[3];
-    for (int i = 0; i < 3; ++i) {
-        NA[i] = a[0] * T.n[AL + i] + a[1] * T.n[AL + i + 1] + h4 * T.n[AL + i + 2];
-        VA[i] = a[2] * T.v[BE + i + 1] + h4 * T.v[BE + i + 2];
-        WA[i] = a[3] * T.w[GA + i + 1] + h4 * T.w[GA + i + 2];
-    }
-    auto SS = [&](int x, int y, int z) {
-        return NA[x] * T.v[BE + y] * T.w[GA + z] + T.n[AL + x] * (VA[y] * T.w[GA + z] + T.v[BE + y] * WA[z]);
-    };
-    out[0] = SS(0, 0, 0);
-    out[1] = SS(1, 0, 0);
-    out[2] = SS(0, 1, 0);
-    out[3] = SS(0, 0, 1);
-    out[4] = 0.5 * (SS(2, 0, 0) + SS(0, 2, 0) + SS(0, 0, 2));
-}
-
-template <int AL, class S> __device__ void psi_mom_s(const TabS<S>& T, S out[5]) {
-    out[0] = T.n[AL];
-    out[1] = T.n[AL + 1];
-    out[2] = T.n[AL] * T.v[1];
-    out[3] = T.n[AL] * T.w[1];
-    out[4] = 0.5 * (T.n[AL + 2] + T.n[AL] * (T.v[2] + T.w[2]));
-}
-
-template <class S> __device__ void slope_mom_s(const TabS<S>& T, int d, const S* a, S out[5]) {
-    if (d == 0) apsi_s<2, 0, 0>(T, a, out);
-    else if (d == 1) apsi_s<1, 1, 0>(T, a, out);
-    else apsi_s<1, 0, 1>(T, a, out);
-}
-
-// <psi psi^T> a = b for the unit Maxwellian (U, lambda), closed form
-template <class S> __device__ void micro_s(const S* U, const S& lam, const S& th, const S* b, S* a) {
-    const S R1 = b[1] - U[0] * b[0], R2 = b[2] - U[1] * b[0], R3 = b[3] - U[2] * b[0];
-    const S U2 = U[0] * U[0] + U[1] * U[1] + U[2] * U[2];
-    const S R4 = 2.0 * b[4] - (U2 + 3.0 * th) * b[0];
-    a[4] = (4.0 / 3.0) * lam * lam * (R4 - 2.0 * (U[0] * R1 + U[1] * R2 + U[2] * R3));
-    a[1] = 2.0 * lam * R1 - U[0] * a[4];
-    a[2] = 2.0 * lam * R2 - U[1] * a[4];
-    a[3] = 2.0 * lam * R3 - U[2] * a[4];
-    a[0] = b[0] - (U[0] * a[1] + U[1] * a[2] + U[2] * a[3]) - 0.5 * a[4] * (U2 + 3.0 * th);
-}
-
-// derivatives of the Maxwellian moments along a conservative slope b
-template <class S> struct DPrimS { S dr, dU[3], dth, UdU; };
-template <class S> __device__ DPrimS<S> dprim_s(const S* U, const S& th, const S& U2, const S* b) {
-    DPrimS<S> q;
-    q.dr = b[0];
-    for (int j = 0; j < 3; ++j) q.dU[j] = b[1 + j] - U[j] * b[0];
-    q.UdU = U[0] * q.dU[0] + U[1] * q.dU[1] + U[2] * q.dU[2];
-    q.dth = ((2.0 * b[4] - (U2 + 3.0 * th) * b[0]) - 2.0 * q.UdU) * (1.0 / 3.0);
-    return q;
-}
-template <int D, class S>
-__device__ void euler_jac_s(const S* U, const S& th, const S& U2, const S* b, const DPrimS<S>& q, S out[5]) {
-    out[0] = b[1 + D];
-    for (int j = 0; j < 3; ++j) {
-        S v = q.dr * (U[D] * U[j]) + q.dU[D] * U[j] + U[D] * q.dU[j];
-        if (j == D) v = v + q.dr * th + q.dth;
-        out[1 + j] = v;
-    }
-    out[4] = b[1 + D] * (0.5 * U2 + 2.5 * th) + U[D] * (q.UdU + 2.5 * q.dth);
-}
-template <int D, class S> __device__ void q_jac_s(const S* U, const S& th, const S& U2, const DPrimS<S>& q, S out[5]) {
-    const S un_ud = U[0] * U[D];
-    const S d_un_ud = q.dU[0] * U[D] + U[0] * q.dU[D];
-    out[0] = q.dr * un_ud + d_un_ud;
-    if (D == 0) out[0] = out[0] + q.dr * th + q.dth;
-    for (int j = 0; j < 3; ++j) {
-        S sv = S(0.0), ds = S(0.0);
-        if (D == j) { sv = sv + U[0]; ds = ds + q.dU[0]; }
-        if (j == 0) { sv = sv + U[D]; ds = ds + q.dU[D]; }
-        if (D == 0) { sv = sv + U[j]; ds = ds + q.dU[j]; }
-        out[1 + j] = q.dr * (un_ud * U[j] + th * sv) + d_un_ud * U[j] + un_ud * q.dU[j] + q.dth * sv + th * ds;
-    }
-    const S A = U2 + 7.0 * th;
-    S v = q.dr * (0.5 * un_ud * A) + 0.5 * (d_un_ud * A + un_ud * (2.0 * q.UdU + 7.0 * q.dth));
-    if (D == 0) {
-        const S Bq = U2 + 5.0 * th;
-        v = v + q.dr * (0.5 * th * Bq) + 0.5 * (q.dth * Bq + th * (2.0 * q.UdU + 5.0 * q.dth));
-    }
-    out[4] = v;
-}
-
-template <class S> struct QCS { S q1, q2, q3, q4, q5, a4, a5; };
-template <class S> __device__ QCS<S> time_coeffs_s(double dt, const S& tau) {
-    QCS<S> c;
-    const S em1 = expm1_(-(dt / tau));
-    const S e = 1.0 + em1;
-    const S tdt = tau * dt;
-    c.q4 = -(tau * em1);
-    c.q1 = dt - c.q4;
-    c.a4 = c.q4 - dt * e;
-    c.q2 = 2.0 * tau * c.q4 - tdt - tdt * e;
-    c.q3 = 0.5 * dt * dt - tdt + tau * c.q4;
-    c.q5 = tdt * e - tau * c.q4;
-    c.a5 = c.q5 + 0.5 * dt * dt * e;
-    return c;
-}
-
-__device__ void face_frame_d(const double* n, double R[3][3]) {
-    int ax = 0;
-    if (::fabs(n[1]) < ::fabs(n[ax])) ax = 1;
-    if (::fabs(n[2]) < ::fabs(n[ax])) ax = 2;
-    double t1[3];
-    t1[0] = ax == 0 ? 0.0 : (ax == 1 ? n[2] : -n[1]);
-    t1[1] = ax == 1 ? 0.0 : (ax == 0 ? -n[2] : n[0]);
-    t1[2] = ax == 2 ? 0.0 : (ax == 0 ? n[1] : -n[0]);
-    const double il = rsqrt(t1[0] * t1[0] + t1[1] * t1[1] + t1[2] * t1[2]);
-    for (int d = 0; d < 3; ++d) t1[d] *= il;
-    R[0][0] = n[0]; R[0][1] = n[1]; R[0][2] = n[2];
-    R[1][0] = t1[0]; R[1][1] = t1[1]; R[1][2] = t1[2];
-    R[2][0] = n[1] * t1[2] - n[2] * t1[1];
-    R[2][1] = n[2] * t1[0] - n[0] * t1[2];
-    R[2][2] = n[0] * t1[1] - n[1] * t1[0];
-}
-
-template <class S> struct SideS { S rho, rhoh, p, H[5], G[5], S5[5]; };
-
-// One side at second order in the face frame: W, rho^h and their lab
-// gradients gW [3q + d], gH [d] reconstructed at the face (first order if the
-// reconstruction is not positive); B accumulates half of the frame slopes.
-template <class S>
-__device__ SideS<S> side_o2_s(const S* Wc, const S& rhohc, const S* gW, const S* gH, const double* dx,
-                              const double R[3][3], int half, S B[3][5], bool first) {
-    S Wf[5];
-    for (int q = 0; q < 5; ++q) Wf[q] = Wc[q] + gW[3 * q] * dx[0] + gW[3 * q + 1] * dx[1] + gW[3 * q + 2] * dx[2];
-    S rh = rhohc + gH[0] * dx[0] + gH[1] * dx[1] + gH[2] * dx[2];
-    S pr = (Wf[4] - 0.5 * (Wf[1] * Wf[1] + Wf[2] * Wf[2] + Wf[3] * Wf[3]) / Wf[0]) * (2.0 / 3.0);
-    const bool o2 = ad::val(Wf[0]) > 0.0 && ad::val(pr) > 0.0;
-    if (!o2) {
-        for (int q = 0; q < 5; ++q) Wf[q] = Wc[q];
-        rh = rhohc;
-        pr = (Wf[4] - 0.5 * (Wf[1] * Wf[1] + Wf[2] * Wf[2] + Wf[3] * Wf[3]) / Wf[0]) * (2.0 / 3.0);
-    }
-    SideS<S> o;
-    S W[5];
-    W[0] = Wf[0];
-    for (int j = 0; j < 3; ++j) W[1 + j] = R[j][0] * Wf[1] + R[j][1] * Wf[2] + R[j][2] * Wf[3];
-    W[4] = Wf[4];
-    o.rho = W[0];
-    o.rhoh = rh;
-    o.p = pr;
-    const S ir = 1.0 / W[0];
-    const S U[3] = {W[1] * ir, W[2] * ir, W[3] * ir};
-    const S lam = 0.5 * W[0] / pr;
-    const S th = 0.5 / lam;
-    TabS<S> T;
-    make_tab_s(U, lam, half, T);
-    psi_mom_s<0>(T, o.H);
-    psi_mom_s<1>(T, o.G);
-    for (int k = 0; k < 5; ++k) o.S5[k] = S(0.0);
-    if (!o2) {
-        if (first)
-            for (int dd = 0; dd < 3; ++dd)
-                for (int q = 0; q < 5; ++q) B[dd][q] = S(0.0);
-        return o;
-    }
-    const S ratio = rh * ir;
-    for (int dd = 0; dd < 3; ++dd) {
-        S g[5], dW[5], b[5], a[5], sm[5];
-        for (int q = 0; q < 5; ++q) g[q] = gW[3 * q] * R[dd][0] + gW[3 * q + 1] * R[dd][1] + gW[3 * q + 2] * R[dd][2];
-        dW[0] = g[0];
-        for (int j = 0; j < 3; ++j) dW[1 + j] = R[j][0] * g[1] + R[j][1] * g[2] + R[j][2] * g[3];
-        dW[4] = g[4];
-        for (int q = 0; q < 5; ++q) B[dd][q] = first ? 0.5 * dW[q] : B[dd][q] + 0.5 * dW[q];
-        const S gh = gH[0] * R[dd][0] + gH[1] * R[dd][1] + gH[2] * R[dd][2];
-        const S gr = (gh - ratio * dW[0]) * ir;
-        for (int q = 0; q < 5; ++q) b[q] = ratio * dW[q] + W[q] * gr;
-        micro_s(U, lam, th, b, a);
-        slope_mom_s(T, dd, a, sm);
-        for (int k = 0; k < 5; ++k) o.S5[k] = o.S5[k] + sm[k];
-    }
-    return o;
-}
-
-// Second-order flux of an interior face (lab frame, per unit area).
-template <class S>
-__device__ void interior_o2_s(const S* WL, const S& rhL, const S* gWL, const S* gHL, const double* dxL, const S* WR,
-                              const S& rhR, const S* gWR, const S* gHR, const double* dxR, const double* n, double dt,
-                              const DevParams& P, S F[5]) {
-    double R[3][3];
-    face_frame_d(n, R);
-    S B[3][5];
-    const SideS<S> L = side_o2_s(WL, rhL, gWL, gHL, dxL, R, +1, B, true);
-    const SideS<S> Rs = side_o2_s(WR, rhR, gWR, gHR, dxR, R, -1, B, false);
-    S W0[5];
-    for (int k = 0; k < 5; ++k) W0[k] = L.rho * L.H[k] + Rs.rho * Rs.H[k];
-    const S rho0 = W0[0], ir0 = 1.0 / rho0;
-    const S U0[3] = {W0[1] * ir0, W0[2] * ir0, W0[3] * ir0};
-    const S U20 = U0[0] * U0[0] + U0[1] * U0[1] + U0[2] * U0[2];
-    const S p0 = (W0[4] - 0.5 * rho0 * U20) * (2.0 / 3.0);
-    const S T0 = p0 * ir0 / P.R;
-    S tau = tau_of(T0, p0, P);
-    if (P.C2 > 0.0) tau = tau + P.C2 * fabs_(L.p - Rs.p) / fabs_(L.p + Rs.p) * dt;
-    const QCS<S> qc = time_coeffs_s(dt, tau);
-    for (int k = 0; k < 5; ++k) F[k] = qc.a4 * (L.rhoh * L.G[k] + Rs.rhoh * Rs.G[k]) + qc.a5 * (L.S5[k] + Rs.S5[k]);
-    const S th0 = p0 * ir0;
-    S Fe[5];
-    Fe[0] = qc.q1 * W0[1];
-    for (int j = 0; j < 3; ++j) Fe[1 + j] = qc.q1 * (W0[1] * U0[j]) + (j == 0 ? qc.q1 * p0 : S(0.0));
-    Fe[4] = qc.q1 * U0[0] * (W0[4] + p0);
-    S Wt[5], t5[5];
-    {
-        const DPrimS<S> q = dprim_s(U0, th0, U20, B[0]);
-        q_jac_s<0>(U0, th0, U20, q, t5);
-        for (int k = 0; k < 5; ++k) Fe[k] = Fe[k] + qc.q2 * t5[k];
-        euler_jac_s<0>(U0, th0, U20, B[0], q, t5);
-        for (int k = 0; k < 5; ++k) Wt[k] = -t5[k];
-    }
-    {
-        const DPrimS<S> q = dprim_s(U0, th0, U20, B[1]);
-        q_jac_s<1>(U0, th0, U20, q, t5);
-        for (int k = 0; k < 5; ++k) Fe[k] = Fe[k] + qc.q2 * t5[k];
-        euler_jac_s<1>(U0, th0, U20, B[1], q, t5);
-        for (int k = 0; k < 5; ++k) Wt[k] = Wt[k] - t5[k];
-    }
-    {
-        const DPrimS<S> q = dprim_s(U0, th0, U20, B[2]);
-        q_jac_s<2>(U0, th0, U20, q, t5);
-        for (int k = 0; k < 5; ++k) Fe[k] = Fe[k] + qc.q2 * t5[k];
-        euler_jac_s<2>(U0, th0, U20, B[2], q, t5);
-        for (int k = 0; k < 5; ++k) Wt[k] = Wt[k] - t5[k];
-    }
-    {
-        const DPrimS<S> q = dprim_s(U0, th0, U20, Wt);
-        euler_jac_s<0>(U0, th0, U20, Wt, q, t5);
-        for (int k = 0; k < 5; ++k) Fe[k] = Fe[k] + qc.q3 * t5[k];
-    }
-    if (P.pr_fix != 0.0) {
-        S mo[5];
-        for (int k = 0; k < 5; ++k) mo[k] = qc.q1 * W0[k] + (qc.q3 - qc.q2) * Wt[k];
-        const S qf = (Fe[4] - ((U0[0] * Fe[1] + U0[1] * Fe[2]) + U0[2] * Fe[3])) + 0.5 * U20 * Fe[0];
-        const S qm = (mo[4] - ((U0[0] * mo[1] + U0[1] * mo[2]) + U0[2] * mo[3])) + 0.5 * U20 * mo[0];
-        Fe[4] = Fe[4] + P.pr_fix * (qf - U0[0] * qm);
-    }
-    for (int k = 0; k < 5; ++k) F[k] = F[k] + Fe[k];
-    const S Fm[3] = {F[1], F[2], F[3]};
-    for (int d = 0; d < 3; ++d) F[1 + d] = Fm[0] * R[0][d] + Fm[1] * R[1][d] + Fm[2] * R[2][d];
-}
 
 __device__ __forceinline__ bool listed_face(const DevMesh& m, const AdjParams& ap, int f) {
     const int nb = m.f_nbr[f];
@@ -498,119 +50,203 @@ __device__ __forceinline__ void farfield_state(const DevParams& P, const AdjPara
     }
 }
 
-// Limited least-squares gradients of W and rho^h = rho - rho^p (second order):
-// one thread per (quantity, cell), as in the step; with record the limiter
-// values are computed and stored in phi [6][nc], otherwise phi is used as
-// given (the limiter frozen at theta).  Far-field ghosts hold the state at theta.
+// The Maxwellian re-emitted by a diffuse wall (unit density).
+__device__ __forceinline__ wm::Prim wall_state(const DevBc& bc, double R, double T_w) {
+    wm::Prim w;
+    w.rho = w.ir = 1.0;
+    for (int d = 0; d < 3; ++d) w.U[d] = bc.U_w[d];
+    w.U2 = wm::dot(w.U, w.U);
+    w.th = w.p = R * T_w;
+    return w;
+}
+
+// First-order flux of a face from the owner's state (and the neighbour's, or the
+// boundary condition at theta).
+__device__ __forceinline__ void face_o1(const DevMesh& m, const DevParams& P, const AdjParams& ap, int nb,
+                                        const wm::Prim& L, double rhL, const double* WR, double rpR, const double* th,
+                                        const double* n, double dt, const wm::FaceGas& fg, double F[5]) {
+    if (nb >= 0) {
+        wm::flux_o1(L, rhL, wm::prim_of(WR, fg.gas), WR[0] - rpR, false, false, n, dt, fg, F);
+        return;
+    }
+    const int tag = m.bf_tag[-1 - nb];
+    const DevBc& bc = P.bc[tag];
+    if (bc.type == UGKWP_BC_DIFFUSE_WALL) {
+        const wm::QC1 c = wm::time_coeffs(dt, wm::face_tau0(L, fg));
+        const double c1 = c.q1 * L.rho + c.a4 * rhL;
+        const wm::PrimGrad none{};
+        const double z[3] = {0.0, 0.0, 0.0};
+        const wm::Prim w = wall_state(bc, P.R, ap.b[tag].param_wall ? th[2] : bc.T_w);
+        const wm::SideFlux a = wm::side_flux<false>(L, none, 0.0, z, n, 1.0, fg.gas);
+        const wm::SideFlux b = wm::side_flux<false>(w, none, 0.0, z, n, -1.0, fg.gas);
+        const double r = a.G[0] / b.G[0];
+        F[0] = 0.0;
+        for (int k = 1; k < 5; ++k) F[k] = c1 * (a.G[k] - r * b.G[k]);
+        return;
+    }
+    wm::Prim R = L;
+    double rhR = rhL;
+    if (bc.type == UGKWP_BC_SPECULAR) {
+        const double Un = wm::dot(L.U, n);
+        for (int d = 0; d < 3; ++d) R.U[d] = L.U[d] - 2.0 * Un * n[d];
+    } else {
+        if (bc.type == UGKWP_BC_FARFIELD) {
+            double Win[5];
+            farfield_state(P, ap, tag, th, Win);
+            R = wm::prim_of(Win, fg.gas);
+        }
+        rhR = R.rho;
+    }
+    wm::flux_o1(L, rhL, R, rhR, bc.type != UGKWP_BC_SPECULAR, false, n, dt, fg, F);
+    if (bc.type == UGKWP_BC_SPECULAR) {
+        const double fn = wm::dot(F + 1, n);
+        F[0] = 0.0;
+        F[4] = 0.0;
+        for (int d = 0; d < 3; ++d) F[1 + d] = fn * n[d];
+    }
+}
+
+// The adjoint of face_o1 along g: Lb, Rb (of the conservative states; of the
+// neighbour's only for an interior face) and thb of theta (boundary faces), all
+// added to.
+__device__ __forceinline__ void face_o1_adj(const DevMesh& m, const DevParams& P, const AdjParams& ap, int nb,
+                                            const wm::Prim& L, double rhL, const double* WR, double rpR,
+                                            const double* th, const double* n, double dt, const wm::FaceGas& fg,
+                                            const double* g, double* Lb, double* Rb, double* thb) {
+    wm::PrimAdj aL = wm::prim_adj_zero(), aR = wm::prim_adj_zero();
+    double rhLb = 0.0, rhRb = 0.0;
+    if (nb >= 0) {
+        const wm::Prim R = wm::prim_of(WR, fg.gas);
+        wm::flux_o1_adj(L, rhL, R, WR[0] - rpR, false, n, dt, fg, g, aL, rhLb, aR, rhRb);
+        aR.rho += rhRb;  // rho^h = rho - rho^p
+        wm::prim_adj(R, aR, fg.gas, Rb);
+    } else {
+        const int tag = m.bf_tag[-1 - nb];
+        const DevBc& bc = P.bc[tag];
+        const AdjBc& ab = ap.b[tag];
+        if (bc.type == UGKWP_BC_DIFFUSE_WALL) {
+            // F_k = c1 (a_k - r b_k), r = a_0 / b_0, c1 = q1 rho + a4 rho^h (F_0 = 0)
+            const double tau = wm::face_tau0(L, fg);
+            const wm::QC1 c = wm::time_coeffs(dt, tau);
+            const double c1 = c.q1 * L.rho + c.a4 * rhL;
+            const wm::PrimGrad none{};
+            const double z[3] = {0.0, 0.0, 0.0};
+            const wm::Prim w = wall_state(bc, P.R, ab.param_wall ? th[2] : bc.T_w);
+            const wm::SideFlux a = wm::side_flux<false>(L, none, 0.0, z, n, 1.0, fg.gas);
+            const wm::SideFlux b = wm::side_flux<false>(w, none, 0.0, z, n, -1.0, fg.gas);
+            const double ib = 1.0 / b.G[0], r = a.G[0] * ib;
+            double c1b = 0.0, rb = 0.0, ab_[5], bb[5], Hb[5] = {}, Sb[5] = {};
+            for (int k = 1; k < 5; ++k) {
+                c1b += g[k] * (a.G[k] - r * b.G[k]);
+                rb -= c1 * g[k] * b.G[k];
+                ab_[k] = c1 * g[k];
+                bb[k] = -c1 * r * g[k];
+            }
+            ab_[0] = rb * ib;
+            bb[0] = -rb * r * ib;
+            double u1 = 0.0, u3[3] = {0.0, 0.0, 0.0};
+            wm::PrimGrad ub{};
+            wm::side_flux_adj<false>(L, none, 0.0, z, n, 1.0, fg.gas, Hb, ab_, Sb, aL, ub, u1, u3);
+            aL.rho += c1b * c.q1;
+            rhLb += c1b * c.a4;
+            const double taub = wm::time_coeffs_adj1(c, dt, tau, c1b * L.rho, 0.0, c1b * rhL);
+            aL.th += taub * fg.omega * tau / L.th;
+            aL.p -= taub * tau / L.p;
+            if (ab.param_wall) {
+                wm::side_flux_adj<false>(w, none, 0.0, z, n, -1.0, fg.gas, Hb, bb, Sb, aR, ub, u1, u3);
+                thb[2] += aR.th * P.R;
+            }
+        } else if (bc.type == UGKWP_BC_SPECULAR) {
+            wm::Prim R = L;
+            const double Un = wm::dot(L.U, n), gn = g[1] * n[0] + g[2] * n[1] + g[3] * n[2];
+            for (int d = 0; d < 3; ++d) R.U[d] = L.U[d] - 2.0 * Un * n[d];
+            const double gs[5] = {0.0, gn * n[0], gn * n[1], gn * n[2], 0.0};
+            wm::flux_o1_adj(L, rhL, R, rhL, false, n, dt, fg, gs, aL, rhLb, aR, rhRb);
+            const double rn = wm::dot(aR.U, n);
+            for (int d = 0; d < 3; ++d) aL.U[d] += aR.U[d] - 2.0 * rn * n[d];
+            aL.th += aR.th;
+            aL.rho += aR.rho;
+            aL.p += aR.p;
+            rhLb += rhRb;
+        } else {
+            wm::Prim R = L;
+            double Win[5];
+            if (bc.type == UGKWP_BC_FARFIELD) {
+                farfield_state(P, ap, tag, th, Win);
+                R = wm::prim_of(Win, fg.gas);
+            }
+            wm::flux_o1_adj(L, rhL, R, R.rho, true, n, dt, fg, g, aL, rhLb, aR, rhRb);
+            aR.rho += rhRb;  // all of the ghost is hydrodynamic
+            if (bc.type == UGKWP_BC_OUTFLOW) {
+                for (int d = 0; d < 3; ++d) aL.U[d] += aR.U[d];
+                aL.th += aR.th;
+                aL.rho += aR.rho;
+                aL.p += aR.p;
+            } else if (ab.param_ff) {
+                double b[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+                wm::prim_adj(R, aR, fg.gas, b);
+                const double be = b[1] * ab.e[0] + b[2] * ab.e[1] + b[3] * ab.e[2];
+                thb[0] += b[0] + th[1] * be + b[4] * (0.5 * th[1] * th[1] + 1.5 * ab.RT);
+                thb[1] += th[0] * (be + b[4] * th[1]);
+            }
+        }
+    }
+    aL.rho += rhLb;
+    wm::prim_adj(L, aL, fg.gas, Lb);
+}
+
+// Limited least-squares gradients of W and rho^h = rho - rho^p as rows (second
+// order); with record the limiter values are stored in phi [6][nc], otherwise
+// phi is used as given (the limiter frozen at theta).  Far-field ghosts hold the
+// state at theta.
 __global__ void __launch_bounds__(128) k_adj_grad(DevMesh m, DevParams P, AdjParams ap, const double* W,
                                                   const double* rho_p, const double* theta, double* phi, int record,
-                                                  double* gW, double* gH) {
+                                                  double* rec) {
     const int nc = m.nc;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nc) return;
     const double th[3] = {theta[0], theta[1], theta[2]};
-    const long long n = 6LL * nc;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-        const int q = (int)(t / nc);
-        const int i = (int)(t - (long long)q * nc);
-        const int own = m.cfs[i];
-        const double self = q < 5 ? W[(size_t)q * nc + i] : W[i] - rho_p[i];
-        double val[4];
-        for (int k = 0; k < 4; ++k) {
-            const int f = m.cf[k * nc + i];
-            const int other = ((own >> k) & 1) ? m.f_nbr[f] : m.f_own[f];
-            if (other >= 0) {
-                val[k] = q < 5 ? W[(size_t)q * nc + other] : W[other] - rho_p[other];
-            } else {
-                const int b = -1 - other;
-                const int tag = m.bf_tag[b];
-                const DevBc& bc = P.bc[tag];
-                val[k] = self;
-                if (bc.type == UGKWP_BC_SPECULAR && q >= 1 && q <= 3) {
-                    const int nbf = m.nbf;
-                    double nn[3];
-                    for (int d = 0; d < 3; ++d) nn[d] = m.bf_n[(size_t)d * nbf + b];
-                    const double mn = W[(size_t)nc + i] * nn[0] + W[(size_t)2 * nc + i] * nn[1] + W[(size_t)3 * nc + i] * nn[2];
-                    val[k] = self - 2.0 * mn * nn[q - 1];
-                } else if (bc.type == UGKWP_BC_FARFIELD) {
-                    double Win[5];
-                    farfield_state(P, ap, tag, th, Win);
-                    val[k] = q < 5 ? Win[q] : Win[0];
-                }
-            }
-        }
-        double g[3] = {0.0, 0.0, 0.0};
-        for (int k = 0; k < 4; ++k)
-            for (int d = 0; d < 3; ++d) g[d] += m.lsq_c[(size_t)(3 * k + d) * nc + i] * (val[k] - self);
-        double ph;
-        if (record) {
-            double vmax = self, vmin = self;
-            for (int k = 0; k < 4; ++k) { vmax = fmax(vmax, val[k]); vmin = fmin(vmin, val[k]); }
-            const double eps2 = m.eps2[i];
-            double bn = 1.0, bd = 1.0;
-            for (int k = 0; k < 4; ++k) {
-                const double d2 = g[0] * m.lsq_dxf[(size_t)(3 * k) * nc + i] + g[1] * m.lsq_dxf[(size_t)(3 * k + 1) * nc + i] +
-                                  g[2] * m.lsq_dxf[(size_t)(3 * k + 2) * nc + i];
-                if (d2 == 0.0) continue;
-                const double d1 = d2 > 0.0 ? vmax - self : vmin - self;
-                double num = (d1 * d1 + eps2) * d2 + 2.0 * d2 * d2 * d1;
-                double den = d2 * (d1 * d1 + 2.0 * d2 * d2 + d1 * d2 + eps2);
-                if (den < 0.0) { num = -num; den = -den; }
-                if (num * bd < bn * den) { bn = num; bd = den; }
-            }
-            ph = bn / bd;
-            phi[(size_t)q * nc + i] = ph;
-        } else {
-            ph = phi[(size_t)q * nc + i];
-        }
-        for (int d = 0; d < 3; ++d) {
-            if (q < 5) gW[(size_t)(3 * q + d) * nc + i] = ph * g[d];
-            else gH[(size_t)d * nc + i] = ph * g[d];
-        }
-    }
+    limited_row(
+        m, P, i, [&](int q, int j) { return q < 5 ? W[(size_t)q * nc + j] : W[j] - rho_p[j]; },
+        [&](int tag, int q) {
+            double Win[5];
+            farfield_state(P, ap, tag, th, Win);
+            return Win[q < 5 ? q : 0];
+        },
+        [&](int q, double ph) {
+            double& v = phi[(size_t)q * nc + i];
+            if (record) v = ph;
+            return record ? ph : v;
+        },
+        rec + (size_t)REC_N * i);
 }
 
-__device__ __forceinline__ void load_grad(const double* gW, const double* gH, int nc, int c, double* gw, double* gh) {
-    for (int j = 0; j < 15; ++j) gw[j] = gW[(size_t)j * nc + c];
-    for (int d = 0; d < 3; ++d) gh[d] = gH[(size_t)d * nc + c];
-}
-
-// the owner's and the neighbour's centroid-to-face vectors of an interior face
-__device__ __forceinline__ void face_dx(const DevMesh& m, int f, int o, int nb, double* dxL, double* dxR) {
-    const int nc = m.nc;
-    const int lk = m.f_lk[f];
-    for (int d = 0; d < 3; ++d) {
-        dxL[d] = m.lsq_dxf[(size_t)(3 * (lk & 3) + d) * nc + o];
-        dxR[d] = m.lsq_dxf[(size_t)(3 * ((lk >> 2) & 3) + d) * nc + nb];
-    }
-}
-
-// ---- forward: fluxes and the functional's face terms at theta
+// ---- forward: fluxes and the functional's terms (boundary faces) at theta
 template <bool O2>
 __global__ void __launch_bounds__(128) k_adj_fwd_flux(DevMesh m, DevParams P, AdjParams ap, const double* W,
                                                       const double* rho_p, double dt, const double* theta,
-                                                      const double* gW, const double* gH, double* F, double* jf) {
+                                                      const double* rec, double* F, double* jf) {
     const int nc = m.nc, nf = m.nf;
-    const double th[3] = {theta[0], theta[1], theta[2]};
-    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
-        const int o = m.f_own[f], nb = m.f_nbr[f];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nf) return;
+    const int f = m.face_order[t];  // interior faces first
+    const double n[3] = {m.f_n[f], m.f_n[nf + f], m.f_n[2 * nf + f]};
+    const int o = m.f_own[f], nb = m.f_nbr[f];
+    double Fv[5];
+    if (O2 && nb >= 0) {
+        interior_flux_o2(m, rec, P, f, o, nb, n, dt, Fv);
+    } else {
+        const double th[3] = {theta[0], theta[1], theta[2]};
+        const wm::FaceGas fg = face_gas(P);
         double WL[5], WR[5];
         for (int q = 0; q < 5; ++q) {
             WL[q] = W[(size_t)q * nc + o];
             WR[q] = nb >= 0 ? W[(size_t)q * nc + nb] : 0.0;
         }
-        double Fv[5];
-        if (O2 && nb >= 0) {
-            double gwl[15], ghl[3], gwr[15], ghr[3], dxL[3], dxR[3];
-            load_grad(gW, gH, nc, o, gwl, ghl);
-            load_grad(gW, gH, nc, nb, gwr, ghr);
-            face_dx(m, f, o, nb, dxL, dxR);
-            const double n[3] = {m.f_n[f], m.f_n[nf + f], m.f_n[2 * nf + f]};
-            interior_o2_s<double>(WL, WL[0] - rho_p[o], gwl, ghl, dxL, WR, WR[0] - rho_p[nb], gwr, ghr, dxR, n, dt, P, Fv);
-        } else {
-            face_flux<double>(m, P, ap, f, WL, rho_p[o], WR, nb >= 0 ? rho_p[nb] : 0.0, th, dt, Fv);
-        }
-        for (int q = 0; q < 5; ++q) F[(size_t)q * nf + f] = Fv[q];
-        jf[f] = listed_face(m, ap, f) ? Fv[ap.comp] * m.f_area[f] : 0.0;
+        face_o1(m, P, ap, nb, wm::prim_of(WL, fg.gas), WL[0] - rho_p[o], WR, nb >= 0 ? rho_p[nb] : 0.0, th, n, dt, fg, Fv);
     }
+    for (int q = 0; q < 5; ++q) F[(size_t)q * nf + f] = Fv[q];
+    if (nb < 0) jf[-1 - nb] = listed_face(m, ap, f) ? Fv[ap.comp] * m.f_area[f] : 0.0;
 }
 
 __global__ void k_adj_update(DevMesh m, const double* W, const double* F, const double* pf, double* Wn) {
@@ -618,247 +254,325 @@ __global__ void k_adj_update(DevMesh m, const double* W, const double* F, const 
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nc) return;
     const int own = m.cfs[i];
+    const double ivol = m.ivol[i];
+    int f[4];
+    double s[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        f[k] = m.cf[k * nc + i];
+        s[k] = ((own >> k) & 1) ? m.f_area[f[k]] : -m.f_area[f[k]];
+    }
+#pragma unroll
     for (int q = 0; q < 5; ++q) {
         double acc = 0.0;
-        for (int k = 0; k < 4; ++k) {
-            const int f = m.cf[k * nc + i];
-            const double v = F[(size_t)q * nf + f] * m.f_area[f];
-            acc += ((own >> k) & 1) ? v : -v;
-        }
-        Wn[(size_t)q * nc + i] = (W[(size_t)q * nc + i] - acc / m.vol[i]) + pf[(size_t)q * nc + i] / m.vol[i];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc += F[(size_t)q * nf + f[k]] * s[k];
+        Wn[(size_t)q * nc + i] = (W[(size_t)q * nc + i] - acc * ivol) + pf[(size_t)q * nc + i] * ivol;
     }
 }
 
-// out[c] (+)= sum_j x[c n + j] for c < ncomp (one block, fixed order per thread)
-__global__ void k_adj_sum(const double* x, int n, int ncomp, double* out, int accumulate) {
+// out[c] = sum_j x[c n + j] (+ y[c n + j]), c < ncomp: one block per component,
+// fixed order.  The summands are one per boundary face, so that a block of 256
+// threads is enough.
+__global__ void __launch_bounds__(256) k_adj_sum(const double* x, const double* y, int n, double* out) {
     __shared__ double sh[256];
-    for (int c = 0; c < ncomp; ++c) {
-        double a = 0.0;
-        for (int j = threadIdx.x; j < n; j += blockDim.x) a += x[(size_t)c * n + j];
-        sh[threadIdx.x] = a;
+    const size_t at = (size_t)blockIdx.x * n;
+    double a = 0.0;
+    for (int j = threadIdx.x; j < n; j += 256) a += y ? x[at + j] + y[at + j] : x[at + j];
+    sh[threadIdx.x] = a;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
         __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
+    }
+    if (threadIdx.x == 0) out[blockIdx.x] = sh[0];
+}
+
+// The reverse pass of an interior face at second order: the products of g with
+// the Jacobians with respect to both cells' rows, written as rows of the same
+// shape (place 5 unused: rho^h's product is added to rho's).
+__device__ __forceinline__ void store_row(double* out, const double* Wb, const double gb[5][3], const double* ghb) {
+    double v[REC_N];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        v[q] = Wb[q];
+        for (int d = 0; d < 3; ++d) v[6 + 3 * q + d] = gb[q][d];
+    }
+    v[5] = 0.0;
+    for (int d = 0; d < 3; ++d) v[21 + d] = ghb[d];
+    double2* o = reinterpret_cast<double2*>(out);
+#pragma unroll
+    for (int j = 0; j < REC_N / 2; ++j) o[j] = make_double2(v[2 * j], v[2 * j + 1]);
+}
+
+__device__ __forceinline__ void side_o2_adj(const double* rec, int c, const double* dx, const double* n, double sgn,
+                                            const wm::Gas& gas, const double* g, const double* W0b, double c4,
+                                            double c5, double gG, double WH, double p_b, const double Bb[5][3],
+                                            double* out) {
+    const Row r = load_row(rec, c, dx);
+    const wm::Prim s = wm::prim_of(r.W, gas);
+    const wm::PrimGrad pg = wm::prim_grad(s, r.g, 1.0, gas);
+    double Hb[5], Gb[5], Sb[5];
+    for (int k = 0; k < 5; ++k) {
+        Hb[k] = s.rho * W0b[k];
+        Gb[k] = c4 * r.rh * g[k];
+        Sb[k] = c5 * g[k];
+    }
+    wm::PrimAdj a = wm::prim_adj_zero();
+    wm::PrimGrad pgb{};
+    double rhb = c4 * gG, ghb[3] = {0.0, 0.0, 0.0}, gb[5][3], Wb[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int q = 0; q < 5; ++q)
+        for (int d = 0; d < 3; ++d) gb[q][d] = Bb[q][d];
+    a.rho = WH;
+    a.p = p_b;
+    wm::side_flux_adj<true>(s, pg, r.rh, r.gh, n, sgn, gas, Hb, Gb, Sb, a, pgb, rhb, ghb);
+    wm::prim_grad_adj(s, r.g, 1.0, pg, pgb, gas, gb, a);
+    wm::prim_adj(s, a, gas, Wb);
+    // the reconstruction: W = W_c + grad W dx, rho^h = rho^h_c + grad rho^h dx;
+    // a side that fell back to its cell values does not depend on its slopes
+    if (r.o2) {
+        for (int d = 0; d < 3; ++d) {
+            for (int q = 0; q < 5; ++q) gb[q][d] += Wb[q] * dx[d];
+            ghb[d] += rhb * dx[d];
         }
-        if (threadIdx.x == 0) out[c] = accumulate ? out[c] + sh[0] : sh[0];
-        __syncthreads();
+    } else {
+        for (int d = 0; d < 3; ++d) {
+            for (int q = 0; q < 5; ++q) gb[q][d] = 0.0;
+            ghb[d] = 0.0;
+        }
+    }
+    Wb[0] += rhb;  // rho^h = rho - rho^p
+    store_row(out, Wb, gb, ghb);
+}
+
+__device__ __forceinline__ void interior_o2_adj(const DevMesh& m, const double* rec, const DevParams& p, int f, int o,
+                                                int nb, const double* n, double dt, const double* g, double* out) {
+    const int nf = m.nf;
+    double dx[6];
+#pragma unroll
+    for (int d = 0; d < 6; ++d) dx[d] = m.f_dx[(size_t)d * nf + f];
+    const wm::FaceGas fg = face_gas(p);
+    const wm::Gas& gas = fg.gas;
+    double B[5][3], W0[5], H[2][5], gG[2], c4b = 0.0, c5b = 0.0, ps[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const Row r = load_row(rec, e == 0 ? o : nb, dx + 3 * e);
+        const wm::Prim c = wm::prim_of(r.W, gas);
+        const wm::SideFlux h =
+            wm::side_flux<true>(c, wm::prim_grad(c, r.g, 1.0, gas), r.rh, r.gh, n, e == 0 ? 1.0 : -1.0, gas);
+        double t = 0.0;
+        for (int k = 0; k < 5; ++k) {
+            W0[k] = e == 0 ? c.rho * h.H[k] : W0[k] + c.rho * h.H[k];
+            H[e][k] = h.H[k];
+            t += g[k] * h.G[k];
+            c5b += g[k] * h.S[k];
+            for (int d = 0; d < 3; ++d) B[k][d] = e == 0 ? r.g[k][d] : B[k][d] + r.g[k][d];
+        }
+        gG[e] = t;
+        c4b += r.rh * t;
+        ps[e] = c.p;
+    }
+    const wm::Prim c0 = wm::prim_of(W0, gas);
+    const double tau0 = wm::face_tau0(c0, fg);
+    double tau = tau0, rD = 0.0;
+    const double D = ps[0] - ps[1], iS = 1.0 / fabs(ps[0] + ps[1]);
+    if (fg.C2 > 0.0) {
+        rD = fabs(D) * iS;
+        tau += fg.C2 * rD * dt;
+    }
+    const wm::QC qc = wm::time_coeffs_all(dt, tau);
+    double qb[3] = {0.0, 0.0, 0.0}, Bb[5][3] = {}, W0b[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, Eb = 0.0;
+    wm::PrimAdj a = wm::prim_adj_zero();
+    wm::equilibrium_flux_adj(W0, c0, B, 0.5, n, qc, p.pr_fix, gas, g, a, Eb, Bb, qb);
+    const double taub = wm::time_coeffs_adj(qc, dt, tau, qb[0], qb[1], qb[2], 0.0, c4b, c5b);
+    a.th += taub * fg.omega * tau0 / c0.th;
+    a.p -= taub * tau0 / c0.p;
+    wm::prim_adj(c0, a, gas, W0b);
+    W0b[4] += Eb;
+    double pb[2] = {0.0, 0.0};
+    if (fg.C2 > 0.0) {
+        const double t = taub * fg.C2 * dt * iS, sg = D > 0.0 ? 1.0 : D < 0.0 ? -1.0 : 0.0;
+        pb[0] = t * (sg - rD);
+        pb[1] = -t * (sg + rD);
+    }
+#pragma unroll 1
+    for (int e = 0; e < 2; ++e) {
+        double WH = 0.0;
+        for (int k = 0; k < 5; ++k) WH += W0b[k] * (e == 0 ? H[0][k] : H[1][k]);
+        side_o2_adj(rec, e == 0 ? o : nb, e == 0 ? dx : dx + 3, n, e == 0 ? 1.0 : -1.0, gas, g, W0b, qc.a4, qc.a5,
+                    e == 0 ? gG[0] : gG[1], WH, e == 0 ? pb[0] : pb[1], Bb, out + e * REC_N);
     }
 }
 
-// ---- reverse: per face, g_f and its products with the local Jacobians
+// Row of a side of a face at first order (the fifth value pads it to 48 bytes).
+constexpr int ROW1 = 6;
+
+// ---- reverse: per face, g_f and its products with the local Jacobians, as one
+// row per side (second order: REC_N values, first order: ROW1) at
+// fb[(2 f + side) row]; the products with theta of a boundary face at
+// thbar[3][nbf].
 template <bool O2>
 __global__ void __launch_bounds__(128) k_adj_face(DevMesh m, DevParams P, AdjParams ap, const double* W,
                                                   const double* rho_p, double dt, const double* theta,
-                                                  const double* gW, const double* gH, const double* lam_next,
-                                                  double* wbar, double* gbar, double* thbar) {
+                                                  const double* rec, const double* lam_next, double* fb,
+                                                  double* thbar) {
+    constexpr int ROW = O2 ? REC_N : ROW1;
     const int nc = m.nc, nf = m.nf;
-    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
-        const int o = m.f_own[f], nb = m.f_nbr[f];
-        const double area = m.f_area[f];
-        double g[5];
-        for (int q = 0; q < 5; ++q) {
-            g[q] = -area / m.vol[o] * lam_next[(size_t)q * nc + o];
-            if (nb >= 0) g[q] += area / m.vol[nb] * lam_next[(size_t)q * nc + nb];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nf) return;
+    const int f = m.face_order[t];  // interior faces first
+    const int o = m.f_own[f], nb = m.f_nbr[f];
+    const double n[3] = {m.f_n[f], m.f_n[nf + f], m.f_n[2 * nf + f]};
+    const double area = m.f_area[f];
+    const double so = area * m.ivol[o], sn = nb >= 0 ? area * m.ivol[nb] : 0.0;
+    double g[5];
+    for (int q = 0; q < 5; ++q) {
+        g[q] = -so * lam_next[(size_t)q * nc + o];
+        if (nb >= 0) g[q] += sn * lam_next[(size_t)q * nc + nb];
+    }
+    if (listed_face(m, ap, f)) g[ap.comp] += area;
+    double* out = fb + (size_t)(2 * ROW) * f;
+    if (O2 && nb >= 0) {
+        interior_o2_adj(m, rec, P, f, o, nb, n, dt, g, out);
+        return;
+    }
+    const double th[3] = {theta[0], theta[1], theta[2]};
+    const wm::FaceGas fg = face_gas(P);
+    double WL[5], WR[5], Lb[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, Rb[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, tb[3] = {0.0, 0.0, 0.0};
+    for (int q = 0; q < 5; ++q) {
+        WL[q] = W[(size_t)q * nc + o];
+        WR[q] = nb >= 0 ? W[(size_t)q * nc + nb] : 0.0;
+    }
+    face_o1_adj(m, P, ap, nb, wm::prim_of(WL, fg.gas), WL[0] - rho_p[o], WR, nb >= 0 ? rho_p[nb] : 0.0, th, n, dt, fg, g,
+                Lb, Rb, tb);
+    if (O2) {  // a boundary face at second order: first order, no products with slopes
+        const double z5[5][3] = {}, z3[3] = {0.0, 0.0, 0.0};
+        store_row(out, Lb, z5, z3);
+    } else {
+        double2* r = reinterpret_cast<double2*>(out);
+        r[0] = make_double2(Lb[0], Lb[1]);
+        r[1] = make_double2(Lb[2], Lb[3]);
+        r[2] = make_double2(Lb[4], 0.0);
+        if (nb >= 0) {
+            r[3] = make_double2(Rb[0], Rb[1]);
+            r[4] = make_double2(Rb[2], Rb[3]);
+            r[5] = make_double2(Rb[4], 0.0);
         }
-        if (listed_face(m, ap, f)) g[ap.comp] += area;
-        const double rpL = rho_p[o], rpR = nb >= 0 ? rho_p[nb] : 0.0;
-        if (O2 && nb >= 0) {
-            // second order: products with the face's Jacobians with respect to
-            // both cells' W and limited gradients, five directions at a time
-            double gw[2][15], gh[2][3], dxL[3], dxR[3], Wc[2][5];
-            load_grad(gW, gH, nc, o, gw[0], gh[0]);
-            load_grad(gW, gH, nc, nb, gw[1], gh[1]);
-            face_dx(m, f, o, nb, dxL, dxR);
-            for (int q = 0; q < 5; ++q) {
-                Wc[0][q] = W[(size_t)q * nc + o];
-                Wc[1][q] = W[(size_t)q * nc + nb];
+    }
+    if (nb < 0)
+        for (int k = 0; k < 3; ++k) thbar[(size_t)k * m.nbf - 1 - nb] = tb[k];
+}
+
+// lambda^n = lambda^{n+1} + the products of the cell's faces with its W; second
+// order: also gg = phi * (the sum of the products with its limited gradients)
+// as a row [18] per cell, 3q + d (q = 5: rho^h).
+template <bool O2>
+__global__ void __launch_bounds__(128) k_adj_gather(DevMesh m, const double* lam_next, const double* fb,
+                                                    const double* phi, double* lam, double* gg) {
+    constexpr int ROW = O2 ? REC_N : ROW1;
+    const int nc = m.nc;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nc) return;
+    const int own = m.cfs[i];
+    double a[ROW];
+#pragma unroll
+    for (int j = 0; j < ROW; ++j) a[j] = j < 5 ? lam_next[(size_t)j * nc + i] : 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int f = m.cf[k * nc + i];
+        const double2* r = reinterpret_cast<const double2*>(fb + ((size_t)2 * f + (((own >> k) & 1) ? 0 : 1)) * ROW);
+#pragma unroll
+        for (int j = 0; j < ROW / 2; ++j) {
+            const double2 v = r[j];
+            a[2 * j] += v.x;
+            a[2 * j + 1] += v.y;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q) lam[(size_t)q * nc + i] = a[q];
+    if constexpr (O2) {
+        double2* o = reinterpret_cast<double2*>(gg + (size_t)18 * i);
+        double ph[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) ph[q] = phi[(size_t)q * nc + i];
+#pragma unroll
+        for (int j = 0; j < 9; ++j) o[j] = make_double2(ph[2 * j / 3] * a[6 + 2 * j], ph[(2 * j + 1) / 3] * a[7 + 2 * j]);
+    }
+}
+
+// Second order: the gradients' dependence on the cells' W, added to lambda^n:
+// gradient_c,q = phi sum_k c_k (val_k - self_q) is linear in the cell's own value
+// (-c_k), in its neighbours' values (+c_k at the neighbour's side) and in the
+// ghost values (specular: mirrored momentum; far field: the state at theta, whose
+// theta products go to thc [3][nbf]).
+__global__ void __launch_bounds__(128) k_adj_cell(DevMesh m, DevParams P, AdjParams ap, const double* theta,
+                                                  const double* gg, double* lam, double* thc) {
+    const int nc = m.nc, nbf = m.nbf;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nc) return;
+    const int4 nbv = m.trk_f ? m.trk_f[i].nb : m.trk_d[i].nb;
+    const int code[4] = {nbv.x, nbv.y, nbv.z, nbv.w};
+    double l[5], own[18];
+    for (int q = 0; q < 5; ++q) l[q] = lam[(size_t)q * nc + i];
+    {
+        const double2* r = reinterpret_cast<const double2*>(gg + (size_t)18 * i);
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            const double2 v = r[j];
+            own[2 * j] = v.x;
+            own[2 * j + 1] = v.y;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        double c[3];
+        for (int d = 0; d < 3; ++d) c[d] = m.lsq_c[(size_t)(3 * k + d) * nc + i];
+        if (code[k] >= 0) {
+            const int other = code[k] >> 2, ko = code[k] & 3;
+            double co[3], t[18];
+            for (int d = 0; d < 3; ++d) co[d] = m.lsq_c[(size_t)(3 * ko + d) * nc + other];
+            const double2* r = reinterpret_cast<const double2*>(gg + (size_t)18 * other);
+#pragma unroll
+            for (int j = 0; j < 9; ++j) {
+                const double2 v = r[j];
+                t[2 * j] = v.x;
+                t[2 * j + 1] = v.y;
             }
-            const double n[3] = {m.f_n[f], m.f_n[nf + f], m.f_n[2 * nf + f]};
-            // pass: 0/1 W of owner/neighbour, 2..4 / 5..7 gradients of W along
-            // x, y, z of owner/neighbour, 8/9 gradient of rho^h of owner/neighbour
-            for (int pass = 0; pass < 10; ++pass) {
-                Dual<5> WL[5], WR[5], GWL[15], GWR[15], GHL[3], GHR[3], F[5];
-                for (int q = 0; q < 5; ++q) {
-                    WL[q] = Dual<5>(Wc[0][q]);
-                    WR[q] = Dual<5>(Wc[1][q]);
-                }
-                for (int j = 0; j < 15; ++j) {
-                    GWL[j] = Dual<5>(gw[0][j]);
-                    GWR[j] = Dual<5>(gw[1][j]);
-                }
-                for (int d = 0; d < 3; ++d) {
-                    GHL[d] = Dual<5>(gh[0][d]);
-                    GHR[d] = Dual<5>(gh[1][d]);
-                }
-                int nseed = 5;
-                if (pass == 0) for (int q = 0; q < 5; ++q) WL[q].d[q] = 1.0;
-                else if (pass == 1) for (int q = 0; q < 5; ++q) WR[q].d[q] = 1.0;
-                else if (pass <= 4) for (int q = 0; q < 5; ++q) GWL[3 * q + (pass - 2)].d[q] = 1.0;
-                else if (pass <= 7) for (int q = 0; q < 5; ++q) GWR[3 * q + (pass - 5)].d[q] = 1.0;
-                else if (pass == 8) { for (int d = 0; d < 3; ++d) GHL[d].d[d] = 1.0; nseed = 3; }
-                else { for (int d = 0; d < 3; ++d) GHR[d].d[d] = 1.0; nseed = 3; }
-                interior_o2_s<Dual<5>>(WL, WL[0] - rpL, GWL, GHL, dxL, WR, WR[0] - rpR, GWR, GHR, dxR, n, dt, P, F);
-                for (int j = 0; j < nseed; ++j) {
-                    double a = 0.0;
-                    for (int q = 0; q < 5; ++q) a += g[q] * F[q].d[j];
-                    // gbar rows: side s (0 owner, 1 neighbour) x (3q + d for W, 15 + d for rho^h)
-                    if (pass == 0) wbar[(size_t)j * nf + f] = a;
-                    else if (pass == 1) wbar[(size_t)(5 + j) * nf + f] = a;
-                    else if (pass <= 4) gbar[(size_t)(3 * j + (pass - 2)) * nf + f] = a;
-                    else if (pass <= 7) gbar[(size_t)(18 + 3 * j + (pass - 5)) * nf + f] = a;
-                    else if (pass == 8) gbar[(size_t)(15 + j) * nf + f] = a;
-                    else gbar[(size_t)(18 + 15 + j) * nf + f] = a;
-                }
-            }
-            for (int k = 0; k < 3; ++k) thbar[(size_t)k * nf + f] = 0.0;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) l[q < 5 ? q : 0] += wm::dot(t + 3 * q, co) - wm::dot(own + 3 * q, c);
             continue;
         }
-        if (O2)  // a boundary face at second order: first order, no gradient products
-            for (int j = 0; j < 36; ++j) gbar[(size_t)j * nf + f] = 0.0;
-        // owner's W
-        {
-            Dual<5> WL[5], WR[5], th[3], F[5];
-            for (int q = 0; q < 5; ++q) {
-                WL[q] = Dual<5>(W[(size_t)q * nc + o]);
-                WL[q].d[q] = 1.0;
-                WR[q] = Dual<5>(nb >= 0 ? W[(size_t)q * nc + nb] : 0.0);
-            }
-            for (int k = 0; k < 3; ++k) th[k] = Dual<5>(theta[k]);
-            face_flux<Dual<5>>(m, P, ap, f, WL, rpL, WR, rpR, th, dt, F);
-            for (int j = 0; j < 5; ++j) {
-                double a = 0.0;
-                for (int q = 0; q < 5; ++q) a += g[q] * F[q].d[j];
-                wbar[(size_t)j * nf + f] = a;
-            }
-        }
-        if (nb >= 0) {
-            Dual<5> WL[5], WR[5], th[3], F[5];
-            for (int q = 0; q < 5; ++q) {
-                WL[q] = Dual<5>(W[(size_t)q * nc + o]);
-                WR[q] = Dual<5>(W[(size_t)q * nc + nb]);
-                WR[q].d[q] = 1.0;
-            }
-            for (int k = 0; k < 3; ++k) th[k] = Dual<5>(theta[k]);
-            face_flux<Dual<5>>(m, P, ap, f, WL, rpL, WR, rpR, th, dt, F);
-            for (int j = 0; j < 5; ++j) {
-                double a = 0.0;
-                for (int q = 0; q < 5; ++q) a += g[q] * F[q].d[j];
-                wbar[(size_t)(5 + j) * nf + f] = a;
-            }
-            for (int k = 0; k < 3; ++k) thbar[(size_t)k * nf + f] = 0.0;
-        } else {
-            for (int j = 0; j < 5; ++j) wbar[(size_t)(5 + j) * nf + f] = 0.0;
-            const AdjBc& ab = ap.b[m.bf_tag[-1 - nb]];
-            if (ab.param_ff || ab.param_wall) {
-                Dual<3> WL[5], WR[5], th[3], F[5];
-                for (int q = 0; q < 5; ++q) {
-                    WL[q] = Dual<3>(W[(size_t)q * nc + o]);
-                    WR[q] = Dual<3>(0.0);
-                }
-                for (int k = 0; k < 3; ++k) {
-                    th[k] = Dual<3>(theta[k]);
-                    th[k].d[k] = 1.0;
-                }
-                face_flux<Dual<3>>(m, P, ap, f, WL, rpL, WR, rpR, th, dt, F);
-                for (int k = 0; k < 3; ++k) {
-                    double a = 0.0;
-                    for (int q = 0; q < 5; ++q) a += g[q] * F[q].d[k];
-                    thbar[(size_t)k * nf + f] = a;
-                }
-            } else {
-                for (int k = 0; k < 3; ++k) thbar[(size_t)k * nf + f] = 0.0;
-            }
-        }
-    }
-}
-
-// Second order: gg = phi * (sum over the cell's faces of the products with
-// its limited gradients) [18][nc], row 3q + d (q = 5: rho^h).
-__global__ void k_adj_gg(DevMesh m, const double* phi, const double* gbar, double* gg) {
-    const int nc = m.nc, nf = m.nf;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nc) return;
-    const int own = m.cfs[i];
-    for (int j = 0; j < 18; ++j) {
-        double a = 0.0;
-        for (int k = 0; k < 4; ++k) {
-            const int f = m.cf[k * nc + i];
-            a += gbar[(size_t)((((own >> k) & 1) ? 0 : 18) + j) * nf + f];
-        }
-        gg[(size_t)j * nc + i] = phi[(size_t)(j / 3) * nc + i] * a;
-    }
-}
-
-// lambda^n = lambda^{n+1} + the products of the cell's faces; at second order
-// also the gradients' dependence on the cell's W: gradient_c,q = phi sum_k
-// c_k (val_k - self_q) is linear in the cell's own value (-c_k), in its
-// neighbours' values (+c_k at the neighbour's side) and in the ghost values
-// (specular: mirrored momentum; far field: the state at theta, whose theta
-// products go to thc [3][nc]).
-__global__ void k_adj_cell(DevMesh m, DevParams P, AdjParams ap, const double* W, const double* theta,
-                           const double* lam_next, const double* wbar, const double* gg, double* lam, double* thc) {
-    const int nc = m.nc, nf = m.nf;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nc) return;
-    const int own = m.cfs[i];
-    double l[5];
-    for (int q = 0; q < 5; ++q) {
-        double a = lam_next[(size_t)q * nc + i];
-        for (int k = 0; k < 4; ++k) {
-            const int f = m.cf[k * nc + i];
-            a += wbar[(size_t)(((own >> k) & 1) ? q : 5 + q) * nf + f];
-        }
-        l[q] = a;
-    }
-    double tc[3] = {0.0, 0.0, 0.0};
-    if (P.order == 2) {
-        const double th[3] = {theta[0], theta[1], theta[2]};
-        for (int k = 0; k < 4; ++k) {
-            const int f = m.cf[k * nc + i];
-            const bool is_own = (own >> k) & 1;
-            const int other = is_own ? m.f_nbr[f] : m.f_own[f];
+        const int b = -1 - code[k];
+        const int tag = m.bf_tag[b];
+        const int type = P.bc[tag].type;
+        double tc[2] = {0.0, 0.0};
+        if (type == UGKWP_BC_SPECULAR) {
+            double nn[3], sn = 0.0;
+            for (int d = 0; d < 3; ++d) nn[d] = m.bf_n[(size_t)d * nbf + b];
+            for (int q = 1; q < 4; ++q) sn += wm::dot(own + 3 * q, c) * nn[q - 1];
+            for (int d = 0; d < 3; ++d) l[1 + d] -= 2.0 * sn * nn[d];
+        } else if (type == UGKWP_BC_FARFIELD) {
+            const AdjBc& ab = ap.b[tag];
+            const double th0 = theta[0], th1 = theta[1];
             for (int q = 0; q < 6; ++q) {
-                const int dq = q < 5 ? q : 0;  // rho^h = rho - rho^p
-                double sself = 0.0;
-                for (int d = 0; d < 3; ++d) sself += gg[(size_t)(3 * q + d) * nc + i] * m.lsq_c[(size_t)(3 * k + d) * nc + i];
-                if (other >= 0) {
-                    const int lk = m.f_lk[f];
-                    const int ko = is_own ? ((lk >> 2) & 3) : (lk & 3);
-                    double snb = 0.0;
-                    for (int d = 0; d < 3; ++d)
-                        snb += gg[(size_t)(3 * q + d) * nc + other] * m.lsq_c[(size_t)(3 * ko + d) * nc + other];
-                    l[dq] += snb - sself;
-                    continue;
-                }
-                const int b = -1 - other;
-                const int tag = m.bf_tag[b];
-                const DevBc& bc = P.bc[tag];
-                if (bc.type == UGKWP_BC_SPECULAR && q >= 1 && q <= 3) {
-                    const int nbf = m.nbf;
-                    double nn[3];
-                    for (int d = 0; d < 3; ++d) nn[d] = m.bf_n[(size_t)d * nbf + b];
-                    for (int jj = 0; jj < 3; ++jj) l[1 + jj] += sself * (-2.0 * nn[q - 1] * nn[jj]);
-                } else if (bc.type == UGKWP_BC_FARFIELD) {
-                    l[dq] -= sself;
-                    const AdjBc& ab = ap.b[tag];
-                    if (ab.param_ff) {
-                        // d W_in / d theta: rho = th0, m = th0 th1 e, E = th0 (th1^2/2 + 3/2 RT)
-                        const int qq = q < 5 ? q : 0;
-                        double d0, d1;
-                        if (qq == 0) { d0 = 1.0; d1 = 0.0; }
-                        else if (qq <= 3) { d0 = th[1] * ab.e[qq - 1]; d1 = th[0] * ab.e[qq - 1]; }
-                        else { d0 = 0.5 * th[1] * th[1] + 1.5 * ab.RT; d1 = th[0] * th[1]; }
-                        tc[0] += sself * d0;
-                        tc[1] += sself * d1;
-                    }
-                }
+                const double s = wm::dot(own + 3 * q, c);
+                const int qq = q < 5 ? q : 0;  // rho^h = rho - rho^p
+                l[qq] -= s;
+                if (!ab.param_ff) continue;
+                // d W_in / d theta: rho = th0, m = th0 th1 e, E = th0 (th1^2/2 + 3/2 RT)
+                double d0, d1;
+                if (qq == 0) { d0 = 1.0; d1 = 0.0; }
+                else if (qq <= 3) { d0 = th1 * ab.e[qq - 1]; d1 = th0 * ab.e[qq - 1]; }
+                else { d0 = 0.5 * th1 * th1 + 1.5 * ab.RT; d1 = th0 * th1; }
+                tc[0] += s * d0;
+                tc[1] += s * d1;
             }
         }
+        thc[b] = tc[0];
+        thc[(size_t)nbf + b] = tc[1];
+        thc[2 * (size_t)nbf + b] = 0.0;
     }
     for (int q = 0; q < 5; ++q) lam[(size_t)q * nc + i] = l[q];
-    if (thc)
-        for (int k = 0; k < 3; ++k) thc[(size_t)k * nc + i] = tc[k];
 }
 
 // recorded particle data of the step just taken
@@ -872,37 +586,41 @@ __global__ void k_adj_record(DevMesh m, DevState s, DevParams P, double* rho_p, 
 
 }  // namespace
 
+size_t adjoint_face_row(int order) { return order == 2 ? REC_N : ROW1; }
+
 void launch_adj_record(const DevMesh& m, const DevState& s, const DevParams& p, double* rho_p, double* pf,
                        cudaStream_t st) {
     k_adj_record<<<(m.nc + 255) / 256, 256, 0, st>>>(m, s, p, rho_p, pf);
 }
 
-static int grad_grid(const DevMesh& m) { return (int)((6LL * m.nc + 127) / 128); }
-
 void launch_adj_forward(const DevMesh& m, const DevParams& p, const AdjParams& ap, const double* W, const double* rho_p,
                         const double* pf, double dt, const double* theta, const AdjO2& o2, double* F, double* jf,
                         double* Jn, double* Wn, cudaStream_t st) {
-    const int g = (m.nf + 127) / 128;
-    if (p.order == 2) k_adj_grad<<<grad_grid(m), 128, 0, st>>>(m, p, ap, W, rho_p, theta, o2.phi, 1, o2.gW, o2.gH);
-    if (p.order == 2) k_adj_fwd_flux<true><<<g, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, o2.gW, o2.gH, F, jf);
-    else k_adj_fwd_flux<false><<<g, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, o2.gW, o2.gH, F, jf);
-    k_adj_sum<<<1, 256, 0, st>>>(jf, m.nf, 1, Jn, 0);
-    k_adj_update<<<(m.nc + 255) / 256, 256, 0, st>>>(m, W, F, pf, Wn);
+    const int gf = (m.nf + 127) / 128, gc = (m.nc + 127) / 128;
+    if (p.order == 2) {
+        k_adj_grad<<<gc, 128, 0, st>>>(m, p, ap, W, rho_p, theta, o2.phi, 1, o2.rec);
+        k_adj_fwd_flux<true><<<gf, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, o2.rec, F, jf);
+    } else {
+        k_adj_fwd_flux<false><<<gf, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, nullptr, F, jf);
+    }
+    k_adj_sum<<<1, 256, 0, st>>>(jf, nullptr, m.nbf, Jn);
+    k_adj_update<<<gc, 128, 0, st>>>(m, W, F, pf, Wn);
 }
 
 void launch_adj_reverse(const DevMesh& m, const DevParams& p, const AdjParams& ap, const double* W,
                         const double* rho_p, double dt, const double* theta, const AdjO2& o2, const double* lam_next,
-                        double* lam, double* wbar, double* thbar, double* th_out, cudaStream_t st) {
-    const int g = (m.nf + 127) / 128;
-    if (p.order == 2) k_adj_grad<<<grad_grid(m), 128, 0, st>>>(m, p, ap, W, rho_p, theta, o2.phi, 0, o2.gW, o2.gH);
-    if (p.order == 2)
-        k_adj_face<true><<<g, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, o2.gW, o2.gH, lam_next, wbar, o2.gbar, thbar);
-    else
-        k_adj_face<false><<<g, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, o2.gW, o2.gH, lam_next, wbar, o2.gbar, thbar);
-    if (p.order == 2) k_adj_gg<<<(m.nc + 255) / 256, 256, 0, st>>>(m, o2.phi, o2.gbar, o2.gg);
-    k_adj_cell<<<(m.nc + 255) / 256, 256, 0, st>>>(m, p, ap, W, theta, lam_next, wbar, o2.gg, lam, o2.thc);
-    k_adj_sum<<<1, 256, 0, st>>>(thbar, m.nf, 3, th_out, 0);
-    if (p.order == 2) k_adj_sum<<<1, 256, 0, st>>>(o2.thc, m.nc, 3, th_out, 1);
+                        double* lam, double* fb, double* thbar, double* th_out, cudaStream_t st) {
+    const int gf = (m.nf + 127) / 128, gc = (m.nc + 127) / 128;
+    if (p.order == 2) {
+        k_adj_grad<<<gc, 128, 0, st>>>(m, p, ap, W, rho_p, theta, o2.phi, 0, o2.rec);
+        k_adj_face<true><<<gf, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, o2.rec, lam_next, fb, thbar);
+        k_adj_gather<true><<<gc, 128, 0, st>>>(m, lam_next, fb, o2.phi, lam, o2.gg);
+        k_adj_cell<<<gc, 128, 0, st>>>(m, p, ap, theta, o2.gg, lam, o2.thc);
+    } else {
+        k_adj_face<false><<<gf, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, nullptr, lam_next, fb, thbar);
+        k_adj_gather<false><<<gc, 128, 0, st>>>(m, lam_next, fb, nullptr, lam, nullptr);
+    }
+    k_adj_sum<<<3, 256, 0, st>>>(thbar, p.order == 2 ? o2.thc : nullptr, m.nbf, th_out);
 }
 
 }  // namespace ugkwp

@@ -341,7 +341,7 @@ void launch_track_batch(const BatchChunk& c, int precision, bool ke, const Track
                         cudaStream_t st);
 void launch_movers_batch(const BatchChunk& c, int blocks, int precision, cudaStream_t st);
 
-// ---- adjoint of the frozen-particle wave map (first order)
+// ---- adjoint of the frozen-particle wave map
 struct AdjBc {
     int32_t param_ff;    // far-field state replaced by theta (rho_inf, U_inf)
     int32_t param_wall;  // diffuse-wall temperature replaced by theta[2]
@@ -358,17 +358,17 @@ struct AdjParams {
 void launch_adj_record(const DevMesh& m, const DevState& s, const DevParams& p, double* rho_p, double* pf,
                        cudaStream_t st);
 // Second order: the step's limiter values phi [6][nc] (recorded by the forward
-// pass, used by the reverse one) and scratch: limited gradients gW [15][nc],
-// gH [3][nc], the faces' products with both cells' gradients gbar [36][nf],
-// phi times their per-cell sums gg [18][nc], far-field ghost products thc [3][nc].
+// pass, used by the reverse one) and scratch: the cells' rows rec [nc][REC_N],
+// phi times the per-cell sums of the products with the gradients gg [nc][18],
+// far-field ghost products thc [3][nbf].
 struct AdjO2 {
     double* phi;
-    double* gW;
-    double* gH;
-    double* gbar;
+    double* rec;
     double* gg;
     double* thc;
 };
+// Values per side of a face in the reverse sweep's face rows.
+size_t adjoint_face_row(int order);
 // Fluxes at theta, the step's functional term Jn[0] and the next state Wn.
 void launch_adj_forward(const DevMesh& m, const DevParams& p, const AdjParams& ap, const double* W, const double* rho_p,
                         const double* pf, double dt, const double* theta, const AdjO2& o2, double* F, double* jf,
@@ -376,7 +376,7 @@ void launch_adj_forward(const DevMesh& m, const DevParams& p, const AdjParams& a
 // lambda^n from lambda^{n+1} and this step's dJ/dtheta terms th_out[3].
 void launch_adj_reverse(const DevMesh& m, const DevParams& p, const AdjParams& ap, const double* W,
                         const double* rho_p, double dt, const double* theta, const AdjO2& o2, const double* lam_next,
-                        double* lam, double* wbar, double* thbar, double* th_out, cudaStream_t st);
+                        double* lam, double* fb, double* thbar, double* th_out, cudaStream_t st);
 
 int sm_count();       // multiprocessors of the current device
 int particle_grid();  // default grid of particle kernels (8 blocks per SM)
