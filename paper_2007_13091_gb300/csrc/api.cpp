@@ -1713,7 +1713,7 @@ int enqueue_chunk_step(FusedChunk& ch, const std::vector<ugkwp_sim*>& sims) {
         c.mem[i] = BatchMember{s->M, s->S, s->P, s->A, s->B, s->Mv};
         wc[i] = s->M.nc;
         wf[i] = s->M.nf;
-        need_grad[i] = (s->M.nc + gradient_threads() - 1) / gradient_threads();
+        need_grad[i] = (3 * s->M.nc + gradient_threads() - 1) / gradient_threads();
         need_o2[i] = (s->M.nf + wave_threads() - 1) / wave_threads();
         need_o1[i] = (s->M.nf + 255) / 256;
     }

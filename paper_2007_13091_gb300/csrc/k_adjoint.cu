@@ -22,8 +22,10 @@
 // each.  A face writes the products of each side as one row; a cell gathers its
 // faces' rows in their fixed order.
 //
-// Bound by the binary64 pipe.  Measured per step (channels of 40,500 and 20,736
-// tets): first order @O1@, second order @O2@.
+// Bound by the binary64 pipe.  The face kernel per step: first order, channel of
+// 40,500 tets, 0.19 ms (duals: 1.97 ms); second order, 20,736 tets, 0.32 ms
+// (duals: 21.8 ms).  The sums over faces run over the boundary faces alone (0.006
+// ms; over all faces 0.16-0.47 ms).
 #include "recon.cuh"
 #include "ugkwp_internal.hpp"
 
@@ -203,11 +205,12 @@ __global__ void __launch_bounds__(128) k_adj_grad(DevMesh m, DevParams P, AdjPar
                                                   const double* rho_p, const double* theta, double* phi, int record,
                                                   double* rec) {
     const int nc = m.nc;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nc) return;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 3 * nc) return;
+    const int pair = t >= 2 * nc ? 2 : t >= nc ? 1 : 0, i = t - pair * nc;
     const double th[3] = {theta[0], theta[1], theta[2]};
-    limited_row(
-        m, P, i, [&](int q, int j) { return q < 5 ? W[(size_t)q * nc + j] : W[j] - rho_p[j]; },
+    limited_pair(
+        m, P, i, pair, [&](int q, int j) { return q < 5 ? W[(size_t)q * nc + j] : W[j] - rho_p[j]; },
         [&](int tag, int q) {
             double Win[5];
             farfield_state(P, ap, tag, th, Win);
@@ -598,7 +601,7 @@ void launch_adj_forward(const DevMesh& m, const DevParams& p, const AdjParams& a
                         double* Jn, double* Wn, cudaStream_t st) {
     const int gf = (m.nf + 127) / 128, gc = (m.nc + 127) / 128;
     if (p.order == 2) {
-        k_adj_grad<<<gc, 128, 0, st>>>(m, p, ap, W, rho_p, theta, o2.phi, 1, o2.rec);
+        k_adj_grad<<<(3 * m.nc + 127) / 128, 128, 0, st>>>(m, p, ap, W, rho_p, theta, o2.phi, 1, o2.rec);
         k_adj_fwd_flux<true><<<gf, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, o2.rec, F, jf);
     } else {
         k_adj_fwd_flux<false><<<gf, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, nullptr, F, jf);
@@ -612,7 +615,7 @@ void launch_adj_reverse(const DevMesh& m, const DevParams& p, const AdjParams& a
                         double* lam, double* fb, double* thbar, double* th_out, cudaStream_t st) {
     const int gf = (m.nf + 127) / 128, gc = (m.nc + 127) / 128;
     if (p.order == 2) {
-        k_adj_grad<<<gc, 128, 0, st>>>(m, p, ap, W, rho_p, theta, o2.phi, 0, o2.rec);
+        k_adj_grad<<<(3 * m.nc + 127) / 128, 128, 0, st>>>(m, p, ap, W, rho_p, theta, o2.phi, 0, o2.rec);
         k_adj_face<true><<<gf, 128, 0, st>>>(m, p, ap, W, rho_p, dt, theta, o2.rec, lam_next, fb, thbar);
         k_adj_gather<true><<<gc, 128, 0, st>>>(m, lam_next, fb, o2.phi, lam, o2.gg);
         k_adj_cell<<<gc, 128, 0, st>>>(m, p, ap, theta, o2.gg, lam, o2.thc);

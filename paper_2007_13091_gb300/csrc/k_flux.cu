@@ -19,8 +19,7 @@
 // one).  Second order: 963 binary64 instructions per interior face against 1,595
 // with moment tables and micro slopes in a face frame; alone on the 24^3 cavity
 // (165,888 faces) 0.35 ms against 0.54 ms.  First order (channel of 393,216
-// tets, 790,528 faces): 0.63 ms against 0.78 ms.  The gradients (24^3 cavity):
-// 0.093 ms against 0.107 ms with one thread per quantity and cell.
+// tets, 790,528 faces): 0.63 ms against 0.78 ms.
 #include "ugkwp_internal.hpp"
 #include "recon.cuh"
 
@@ -39,12 +38,12 @@ namespace ugkwp {
 
 namespace {
 
-// Gradient kernel: one thread per cell, a persistent grid.  Two blocks per SM
+// Gradient kernel: three threads per cell, a persistent grid.  Two blocks per SM
 // leave room for the sampling kernel and the first half of the tracking grid,
 // which then spreads evenly over the SMs and leaves each its room for a block
-// of the wave flux: two steps of the settled 24^3 cavity take 2.20 ms in a row
-// and 2.28 ms on their own, against 2.24 and 2.58 with four blocks per SM
-// (2.22 and 3.45 with three).
+// of the wave flux: two steps of the settled 24^3 cavity take 2.22 ms in a row
+// and 2.26 ms on their own, against 2.19 and 2.57 with three blocks per SM and
+// 2.24 and 2.57 with four.
 constexpr int GRAD_THREADS = 128, GRAD_BLOCKS_PER_SM = 2;
 
 // Constants of K internal degrees of freedom (rho E = rho |U|^2/2 + (3+K)/2 p,
@@ -75,11 +74,14 @@ __device__ __forceinline__ double dot3(const double* a, const double* b) { retur
 
 __device__ __forceinline__ void gradients_body(const DevMesh& m, const DevState& s, const DevParams& p, Blk bk) {
     const int nc = m.nc;
-    for (int i = bk.id * blockDim.x + threadIdx.x; i < nc; i += bk.n * blockDim.x)
-        limited_row(
-            m, p, i, [&](int q, int j) { return q < 5 ? s.W[(size_t)q * nc + j] : s.rhoh[j]; },
+    // pair-major, so that neighbouring threads read neighbouring cells of one array
+    for (int t = bk.id * blockDim.x + threadIdx.x; t < 3 * nc; t += bk.n * blockDim.x) {
+        const int pair = t >= 2 * nc ? 2 : t >= nc ? 1 : 0, i = t - pair * nc;
+        limited_pair(
+            m, p, i, pair, [&](int q, int j) { return q < 5 ? s.W[(size_t)q * nc + j] : s.rhoh[j]; },
             [&](int tag, int q) { return p.bc[tag].W_in[q < 5 ? q : 0]; }, [](int, double phi) { return phi; },
             s.rec + (size_t)REC_N * i);
+    }
 }
 __global__ void __launch_bounds__(GRAD_THREADS) k_gradients(DevMesh m, DevState s, DevParams p) {
     gradients_body(m, s, p, Blk{(int)blockIdx.x, (int)gridDim.x});
@@ -362,7 +364,7 @@ static int wave_grid(int n, int blocks) {
 // A persistent grid of GRAD_BLOCKS_PER_SM blocks per SM, which leaves room
 // beside it for the first half of the tracking grid.
 void launch_gradients(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
-    const int need = (m.nc + GRAD_THREADS - 1) / GRAD_THREADS, cap = GRAD_BLOCKS_PER_SM * sm_count();
+    const int need = (3 * m.nc + GRAD_THREADS - 1) / GRAD_THREADS, cap = GRAD_BLOCKS_PER_SM * sm_count();
     k_gradients<<<need < cap ? need : cap, GRAD_THREADS, 0, st>>>(m, s, p);
 }
 

@@ -11,11 +11,13 @@ __device__ __forceinline__ wm::FaceGas face_gas(const DevParams& p) {
     return wm::FaceGas{wm::gas_of(p.K), p.mu_ref, p.omega, 1.0 / (p.R * p.T_ref), p.C2};
 }
 
-// Limited gradients of the six quantities of cell i (W and rho^h), written with
-// the values themselves as the cell's flux record (REC_N values in a row, see
-// DevState::rec).  One thread per cell: the reconstruction weights, the
-// centroid-to-face vectors and the neighbour codes are read once for all
-// quantities, and the flux kernel reads each side of a face as one row.
+// Limited gradients of two of the six quantities (0..4: W, 5: rho^h) of cell i,
+// quantities 2 pair and 2 pair + 1, written with the values themselves into the
+// cell's row (REC_N values, see DevState::rec), which the flux kernel reads whole
+// for each side of a face.  One thread per pair and cell: a thread's two
+// quantities share the reconstruction weights, the centroid-to-face vectors and
+// the neighbour codes and fill whole 16-byte pieces of the row, and three
+// threads per cell keep enough of them in flight on small meshes.
 // Venkatakrishnan's function of the allowed difference d1 and the extrapolated
 // difference d2 (same sign, d2 != 0), divided through by d2:
 // num/den = (A + 2 s) / (A + s + 2 d2^2), A = d1^2 + eps^2, s = d1 d2 >= 0.
@@ -27,7 +29,7 @@ __device__ __forceinline__ wm::FaceGas face_gas(const DevParams& p) {
 // boundary condition; lim(q, phi): the limiter value to use, given the computed
 // one (an adjoint pass records or replaces it).
 template <class Val, class Far, class Lim>
-__device__ __forceinline__ void limited_row(const DevMesh& m, const DevParams& p, int i, Val&& val, Far&& far, Lim&& lim,
+__device__ __forceinline__ void limited_pair(const DevMesh& m, const DevParams& p, int i, int pair, Val&& val, Far&& far, Lim&& lim,
                                             double* row_of_i) {
     const int nc = m.nc;
     const int4 nbv = m.trk_f ? m.trk_f[i].nb : m.trk_d[i].nb;
@@ -42,7 +44,8 @@ __device__ __forceinline__ void limited_row(const DevMesh& m, const DevParams& p
     double2* row = reinterpret_cast<double2*>(row_of_i);
     double out[4];  // values waiting for a whole pair
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
+    for (int e = 0; e < 2; ++e) {
+        const int q = 2 * pair + e;
         const double self = val(q, i);
         double v[4];
 #pragma unroll
@@ -94,12 +97,12 @@ __device__ __forceinline__ void limited_row(const DevMesh& m, const DevParams& p
         // the row: W (5), rho^h, grad W [3 q + d], grad rho^h; three gradient
         // values per quantity from an even place on: two quantities make three pairs
         const double v3[3] = {phi * g[0], phi * g[1], phi * g[2]};
-        if ((q & 1) == 0) {
+        if (e == 0) {
             out[0] = self;
             out[1] = v3[0]; out[2] = v3[1]; out[3] = v3[2];
         } else {
-            row[q / 2] = make_double2(out[0], self);
-            const int at = 3 + 3 * (q / 2);
+            row[pair] = make_double2(out[0], self);
+            const int at = 3 + 3 * pair;
             row[at] = make_double2(out[1], out[2]);
             row[at + 1] = make_double2(out[3], v3[0]);
             row[at + 2] = make_double2(v3[1], v3[2]);
