@@ -330,8 +330,9 @@ int ugkwp_last(ugkwp_sim* s, int32_t which, void* host_out);
 enum {
     UGKWP_K_RESET = 0, UGKWP_K_CELL_PREP, UGKWP_K_SAMPLE_COUNT, UGKWP_K_SCAN,
     UGKWP_K_SCATTER, /* no kernel launches in this class: the tracking kernel compacts the survivors */
-    UGKWP_K_SAMPLE, UGKWP_K_TRACK, UGKWP_K_FLUX, UGKWP_K_UPDATE, UGKWP_K_MOVERS, UGKWP_K_GRADIENTS,
-    UGKWP_K_FLUX_O2, UGKWP_N_KERNELS
+    UGKWP_K_SAMPLE, UGKWP_K_TRACK, UGKWP_K_FLUX, UGKWP_K_UPDATE,
+    UGKWP_K_MOVERS,  /* no kernel launches in this class: the tracking kernel adds the counting flux */
+    UGKWP_K_GRADIENTS, UGKWP_K_FLUX_O2, UGKWP_N_KERNELS
 };
 
 /* ---- launch configuration and autotuning -------------------------------
@@ -340,9 +341,9 @@ enum {
  * counter-based stream and every sum over particles is fixed point), only the
  * speed does. */
 typedef struct {
-    int32_t particle_blocks;     /* blocks of the sampling, tracking and movers kernels (> 0) */
+    int32_t particle_blocks;     /* blocks of the sampling and tracking kernels (> 0) */
     int32_t wave_blocks;         /* blocks of the persistent second-order wave kernels (> 0) */
-    int32_t track_threads;       /* particles per tracking tile, one per thread of a block: 128 or 256 */
+    int32_t track_threads;       /* threads per block of the tracking kernel: 128 or 256 */
     int32_t smem_carveout;       /* preferred shared-memory carveout of the step's kernels, percent of
                                   * the largest (0..100), or -1 for the driver's choice (default 58).
                                   * A kernel attribute: it holds for every simulation of the process */

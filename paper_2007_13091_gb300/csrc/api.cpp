@@ -33,7 +33,6 @@ struct ugkwp_sim {
     DevMesh M;
     DevState S;
     PartBufRaw A, B;   // A: the current particles (between steps: the survivors); B: the next survivors
-    PartBufRaw Mv;     // the step's movers (particles whose counting flux is non-zero)
     std::vector<double> anchor;  // [3*nc] anchors of the tets (mixed mode; 0 in binary64)
     cudaStream_t stream = nullptr;
     // device staging of ugkwp_import_state in mixed mode (the tets' anchors
@@ -130,7 +129,7 @@ struct Carver {
 };
 
 void layout(const MeshHost& mh, int64_t cap, size_t rs, bool with_e, Carver& c, DevMesh& M, DevState& S,
-            PartBufRaw& A, PartBufRaw& B, PartBufRaw& Mv) {
+            PartBufRaw& A, PartBufRaw& B) {
     const size_t nc = mh.nc, nf = mh.nf, nbf = mh.nbf;
     M.nc = mh.nc; M.nf = mh.nf; M.nbf = mh.nbf; M.nif = mh.nf - mh.nbf;
     M.vol = c.take<double>(nc);
@@ -143,6 +142,8 @@ void layout(const MeshHost& mh, int64_t cap, size_t rs, bool with_e, Carver& c, 
     M.trk_d = nullptr;
     if (rs == 4) M.trk_f = c.take<TrkF>(nc);
     else M.trk_d = c.take<TrkD>(nc);
+    M.pln_f = rs == 8 ? c.take<float4>(4 * nc) : nullptr;
+    M.margin = c.take<float>(nc);
     M.face_order = c.take<int32_t>(nf);
     M.smp_f = c.take<float>(24 * nc);
     M.bf_f = c.take<float>(11 * (nbf ? nbf : 1));
@@ -181,6 +182,8 @@ void layout(const MeshHost& mh, int64_t cap, size_t rs, bool with_e, Carver& c, 
     S.soff = c.take<int32_t>(nc);
     S.wcap = c.take<int32_t>(nc);
     S.woff = c.take<int32_t>(nc);
+    S.cinfo = c.take<int4>(nc);
+    S.cthr = c.take<uint32_t>(nc);
     S.pflux = c.take<int64_t>(5 * nc);
     S.wacc = c.take<int64_t>(5 * nc);
     S.mom = c.take<double>(5 * nc);
@@ -190,18 +193,17 @@ void layout(const MeshHost& mh, int64_t cap, size_t rs, bool with_e, Carver& c, 
     S.t = c.take<double>(1);
     S.dt = c.take<double>(1);
     S.cnt64 = c.take<int64_t>(CNT_SLOTS);
-    // each particle array holds the capacity rounded up to whole tiles of the
-    // tracking kernel (TRACK_TILE_MAX particles), so that a tile's loads of
-    // its whole slots stay inside the array
+    // each particle array holds the capacity rounded up to a multiple of
+    // TRACK_TILE_MAX slots, so that a tracking warp's loads of whole tiles stay
+    // inside the array
     const size_t capt = ((size_t)cap + TRACK_TILE_MAX - 1) / TRACK_TILE_MAX * TRACK_TILE_MAX;
-    for (PartBufRaw* pb : {&A, &B, &Mv}) {
+    for (PartBufRaw* pb : {&A, &B}) {
         for (int d = 0; d < 3; ++d) pb->x[d] = c.take<char>(rs * capt);
         for (int d = 0; d < 3; ++d) pb->u[d] = c.take<char>(rs * capt);
         pb->m = c.take<double>(capt);
         pb->cell = c.take<int32_t>(capt);
         pb->id = c.take<uint64_t>(capt);
         pb->e = with_e ? (void*)c.take<char>(rs * capt) : nullptr;
-        pb->e2 = (with_e && pb == &Mv) ? (void*)c.take<char>(rs * capt) : nullptr;
     }
 }
 
@@ -369,8 +371,7 @@ int ugkwp_query_sizes(const ugkwp_mesh* m, const ugkwp_params* p, ugkwp_sizes* o
     DevState S{};
     PartBufRaw A{}, B{};
     Carver c(nullptr);
-    PartBufRaw Mv{};
-    layout(m->h, p->particle_capacity, p->precision == UGKWP_MIXED ? 4 : 8, p->K > 0, c, M, S, A, B, Mv);
+    layout(m->h, p->particle_capacity, p->precision == UGKWP_MIXED ? 4 : 8, p->K > 0, c, M, S, A, B);
     out->workspace_bytes = (c.off + 255) & ~(size_t)255;
     out->n_cells = m->h.nc;
     out->n_faces = m->h.nf;
@@ -407,7 +408,7 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
     s->capacity = p->particle_capacity;
     s->n_bc = p->n_bc;
     Carver c(d_workspace);
-    layout(mh, p->particle_capacity, s->real_size, p->K > 0, c, s->M, s->S, s->A, s->B, s->Mv);
+    layout(mh, p->particle_capacity, s->real_size, p->K > 0, c, s->M, s->S, s->A, s->B);
     // parameters
     DevParams& P = s->P;
     std::memset(&P, 0, sizeof(P));
@@ -615,6 +616,42 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
             td[i].nb = nb4;
         }
     }
+    // Inside test of the tracking (k_track): the planes in binary32 and the margin.
+    // A point counts as inside when d - n.x, evaluated in binary32, exceeds the
+    // margin.  Mixed mode: n, x0, u, d are the walk's own binary32 values in the
+    // tet's frame; with H bounding |x|_1 of the tet's points and |d| there, the
+    // roundings of the test (x = x0 + u t: 2^-23 H per unit of |n|; the three-term
+    // products and d: 4 2^-23 H) and those of the walk's exit time
+    // (d - n.x0)/(u.n) against t (|x0|_1 and |u t|_1 up to 3 H: at most 16 2^-23 H)
+    // stay below 2^-18 H = 32 2^-23 H.  Binary64: the test's own roundings (x, n and
+    // d to binary32: 3 2^-24 X each; its arithmetic as above), X bounding |x|_1 of
+    // the domain, stay below the same multiple of X, and the walk's are 2^-29 of that.
+    std::vector<float> margin(nc);
+    std::vector<float4> plnf(s->real_size == 8 ? 4 * (size_t)nc : 0);
+    {
+        double X = 0.0;
+        for (size_t v = 0; v < mh.xyz.size() / 3; ++v)
+            X = std::max(X, std::fabs(mh.xyz[3 * v]) + std::fabs(mh.xyz[3 * v + 1]) + std::fabs(mh.xyz[3 * v + 2]));
+        for (int i = 0; i < nc; ++i) {
+            double H = X;
+            if (s->real_size == 4) {
+                H = 0.0;
+                for (int k = 0; k < 4; ++k) {
+                    double a = 0.0;
+                    for (int d = 0; d < 3; ++d)
+                        a += std::fabs(mh.xyz[3 * (size_t)mh.tet[4 * (size_t)i + k] + d] - s->anchor[3 * (size_t)i + d]);
+                    H = std::max(H, a);
+                }
+                for (int k = 0; k < 4; ++k) H = std::max(H, (double)std::fabs(tf[i].pl[k].w));
+            } else {
+                for (int k = 0; k < 4; ++k) {
+                    const Dbl4& v = td[i].pl[k];
+                    plnf[4 * (size_t)i + k] = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
+                }
+            }
+            margin[i] = (float)std::ldexp(H, -18);
+        }
+    }
     cudaStream_t st = s->stream;
     auto up = [&](const void* dst, const void* src, size_t bytes) {
         return cudaMemcpyAsync(const_cast<void*>(dst), src, bytes, cudaMemcpyHostToDevice, st);
@@ -637,6 +674,8 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
     } else {
         UP(s->M.trk_d, td.data(), td.size() * sizeof(TrkD));
     }
+    if (s->real_size == 8) UP(s->M.pln_f, plnf.data(), plnf.size() * sizeof(float4));
+    UP(s->M.margin, margin.data(), margin.size() * sizeof(float));
     UP(s->M.face_order, forder.data(), nf * sizeof(int32_t));
     UP(s->M.smp_f, smpf.data(), smpf.size() * sizeof(float));
     UP(s->M.bf_f, bff.data(), bff.size() * sizeof(float));
@@ -804,17 +843,16 @@ int enqueue_step(ugkwp_sim* s) {
         const int first_half = (s->lc.particle_blocks + 1) / 2;
         timed(s, UGKWP_K_TRACK, s->lc.particle_blocks > first_half ? 2 : 1, q, [&] {
             ce = cudaEventRecord(s->sampled, q);
-            launch_track(s->M, s->S, s->P, s->A, s->B, s->Mv, s->lc.track, first_half, q);
+            launch_track(s->M, s->S, s->P, s->A, s->B, s->lc.track, first_half, q);
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(s->aux, s->sampled, 0);
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(s->aux, s->join, 0);
             if (s->lc.particle_blocks > first_half)
-                launch_track(s->M, s->S, s->P, s->A, s->B, s->Mv, s->lc.track, s->lc.particle_blocks - first_half,
+                launch_track(s->M, s->S, s->P, s->A, s->B, s->lc.track, s->lc.particle_blocks - first_half,
                              s->aux);
             if (ce == cudaSuccess) ce = cudaEventRecord(s->tracked, s->aux);
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(q, s->tracked, 0);
         });
         if (ce != cudaSuccess) return cuda_fail(ce, "tracking launch order");
-        timed(s, UGKWP_K_MOVERS, 1, q, [&] { launch_movers(s->M, s->S, s->P, s->Mv, s->lc.particle_blocks, q); });
         CU(cudaStreamWaitEvent(q, s->waved, 0));  // the wave part of the update is done
         timed(s, UGKWP_K_UPDATE, 1, q, [&] { launch_cell_update(s->M, s->S, s->P, s->B.cell, q); });
         std::swap(s->A, s->B);
@@ -931,7 +969,7 @@ int ugkwp_step(ugkwp_sim* s, int32_t n_steps, ugkwp_stats* st) {
         st->n_sampled = h[CNT_SAMPLED]; st->n_collided = h[CNT_COLLIDED]; st->n_exited = h[CNT_EXITED];
         st->n_lost = h[CNT_LOST]; st->n_crossings = h[CNT_CROSSINGS]; st->n_wall_hits = h[CNT_WALL];
         st->n_moves_total = h[CNT_MOVES];
-        st->n_movers = h[CNT_RESV];
+        st->n_movers = h[CNT_MOVERS];
         return read_error(s);
     }
     return UGKWP_OK;
@@ -1710,7 +1748,7 @@ int enqueue_chunk_step(FusedChunk& ch, const std::vector<ugkwp_sim*>& sims) {
     std::vector<int> need_grad(c.n), need_o2(c.n), need_o1(c.n);
     for (int i = 0; i < c.n; ++i) {
         ugkwp_sim* s = sims[ch.idx[i]];
-        c.mem[i] = BatchMember{s->M, s->S, s->P, s->A, s->B, s->Mv};
+        c.mem[i] = BatchMember{s->M, s->S, s->P, s->A, s->B};
         wc[i] = s->M.nc;
         wf[i] = s->M.nf;
         need_grad[i] = (3 * s->M.nc + gradient_threads() - 1) / gradient_threads();
@@ -1758,7 +1796,6 @@ int enqueue_chunk_step(FusedChunk& ch, const std::vector<ugkwp_sim*>& sims) {
         launch_track_batch(c, ch.precision, ch.ke, lc.track, lc.particle_blocks - first_half, ch.aux);
     CU(cudaEventRecord(ch.tracked, ch.aux));
     CU(cudaStreamWaitEvent(q, ch.tracked, 0));
-    launch_movers_batch(c, lc.particle_blocks, ch.precision, q);
     CU(cudaStreamWaitEvent(q, ch.waved, 0));
     launch_cell_update_batch(c, blocks(BCL_CELLS), q);
     for (int i = 0; i < c.n; ++i) {

@@ -1,0 +1,73 @@
+// Fixed-point images of binary64 values (the particle flux and the survivors' mass).
+#pragma once
+
+namespace ugkwp {
+
+// Round-to-nearest-even of v 2^-e for a binary64 v, from the bits of v with
+// integer operations only (v 2^-e is an exact exponent shift, so this equals
+// rounding the scaled binary64 value); false (q = 0) if v is not finite or
+// |v 2^-e| >= 2^62.  Keeps the conversions off the FP64 pipe.
+__device__ __forceinline__ bool fixed_of(double v, int e, long long& q) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+    const int ex = (int)((bits >> 52) & 0x7ff);
+    unsigned long long mant = bits & 0x000fffffffffffffULL;
+    q = 0;
+    if (ex == 0x7ff) return false;
+    int sh;  // |v| 2^-e = mant 2^sh
+    if (ex == 0) {
+        sh = 1 - 1075 - e;
+    } else {
+        mant |= 0x0010000000000000ULL;
+        sh = ex - 1075 - e;
+    }
+    unsigned long long mag;
+    if (sh >= 0) {
+        if (mant == 0) return true;
+        if (sh > 9) return false;  // mant >= 2^52 when nonzero and normal: 2^(52+10) = 2^62
+        mag = mant << sh;
+        if (mag >= (1ULL << 62)) return false;
+    } else {
+        const int r = -sh;
+        if (r > 63) return true;
+        const unsigned long long hi = mant >> r;
+        const unsigned long long rem = mant & ((1ULL << r) - 1ULL);
+        const unsigned long long half = 1ULL << (r - 1);
+        mag = hi + ((rem > half || (rem == half && (hi & 1ULL))) ? 1ULL : 0ULL);
+    }
+    q = (bits >> 63) ? -(long long)mag : (long long)mag;
+    return true;
+}
+
+// round-to-nearest-even of m 2^-e for a finite m >= 0, computed on the bits of
+// m with integer operations only (m 2^-e is an exact exponent shift, so this
+// equals rounding the binary64 product); false if the result is >= 2^62.
+__device__ __forceinline__ bool fixed_of_mass(double m, int e, long long& q) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(m);
+    const int ex = (int)((bits >> 52) & 0x7ff);
+    unsigned long long mant = bits & 0x000fffffffffffffULL;
+    int s;  // value = mant 2^s
+    if (ex == 0) {
+        s = 1 - 1075 - e;
+    } else {
+        mant |= 0x0010000000000000ULL;
+        s = ex - 1075 - e;
+    }
+    if (ex == 0x7ff || (bits >> 63)) { q = 0; return false; }
+    if (s >= 0) {
+        if (mant == 0) { q = 0; return true; }
+        if (s > 9) { q = 0; return false; }  // mant < 2^53: 2^(53+s) > 2^62
+        const unsigned long long v = mant << s;
+        if (v >= (1ULL << 62)) { q = 0; return false; }
+        q = (long long)v;
+        return true;
+    }
+    const int r = -s;
+    if (r > 63) { q = 0; return true; }
+    const unsigned long long hi = mant >> r;
+    const unsigned long long rem = mant & ((1ULL << r) - 1ULL);
+    const unsigned long long half = 1ULL << (r - 1);
+    q = (long long)(hi + ((rem > half || (rem == half && (hi & 1ULL))) ? 1ULL : 0ULL));
+    return true;
+}
+
+}  // namespace ugkwp

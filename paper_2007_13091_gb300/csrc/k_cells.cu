@@ -6,6 +6,7 @@
 #include <cfloat>
 
 #include "dmath.cuh"
+#include "fixed.cuh"
 #include "ugkwp_internal.hpp"
 
 namespace ugkwp {
@@ -47,10 +48,7 @@ __device__ __forceinline__ void reset_body(const DevMesh& m, const DevState& s, 
     const long long stride = (long long)bk.n * blockDim.x;
     for (long long i = (long long)bk.id * blockDim.x + threadIdx.x; i < 5LL * nc; i += stride) {
         s.pflux[i] = 0;
-        if (i < nc) {
-            s.nleft_next[i] = 0;
-            s.smass_next[i] = 0;
-        }
+        if (i < nc) s.nleft_next[i] = 0;
     }
     if (bk.id == 0 && threadIdx.x == 0) {
         s.cnt64[CNT_SAMPLED] = 0;
@@ -59,7 +57,7 @@ __device__ __forceinline__ void reset_body(const DevMesh& m, const DevState& s, 
         s.cnt64[CNT_LOST] = 0;
         s.cnt64[CNT_CROSSINGS] = 0;
         s.cnt64[CNT_WALL] = 0;
-        s.cnt64[CNT_RESV] = 0;
+        s.cnt64[CNT_MOVERS] = 0;
         s.cnt64[CNT_TRACKED] = 0;
         s.cnt64[CNT_DT_BITS] = 0x7ff0000000000000LL;  // +inf
         s.cnt64[CNT_TILE] = 0;
@@ -161,6 +159,17 @@ __device__ __forceinline__ void sample_count_body(const DevMesh& m, const DevSta
                 ms = Mhp / (double)ns;
             }
         }
+        // the survivors' mass of this step starts from every particle of the cell;
+        // the tracking takes out what is removed or leaves and adds what arrives
+        long long qm = 0;
+        if (ns > 0 && !fixed_of_mass(ms, p.exps[0], qm)) set_err(s, ERRB_FIXED_OVERFLOW);
+        s.smass_next[i] = s.smass[i] + ns * qm;
+        // collision threshold on the first 32 random bits of a particle's draw:
+        // -tau ln eta < dt needs eta > e^{-dt/tau} up to the roundings of tau, dt and
+        // of the logarithm in the particle precision (below 3e-7 in eta) and of eta
+        // itself (2^-24); 2^-18 = 3.8e-6 below it no particle collides
+        const double th = (ex - 0x1p-18) * 0x1p32;
+        s.cthr[i] = th > 0.0 ? (uint32_t)th : 0u;
         s.nsam[i] = (int)ns;
         s.msam[i] = ms;
         nsam = (int)ns;
@@ -219,7 +228,9 @@ __device__ __forceinline__ void scan_apply_body(const DevMesh& m, const DevState
     const int2 incl = block_scan_incl2(v, shw);
     if (i < m.nc) {
         s.soff[i] = s.bsum[bk.id].y + incl.y - v.y;
-        s.woff[i] = s.bsum[bk.id].x + incl.x - v.x;
+        const int woff = s.bsum[bk.id].x + incl.x - v.x;
+        s.woff[i] = woff;
+        s.cinfo[i] = make_int4((int)s.cthr[i], woff, v.x, __float_as_int(m.margin[i]));
     }
 }
 __global__ void k_scan_apply(DevMesh m, DevState s) {
@@ -409,7 +420,8 @@ __global__ void k_rebuild(DevMesh m, DevState s, DevParams p, PartBufRaw a) {
         long long q = 0;
         if (i < n) {
             c = cell[i];
-            if (c >= 0) q = __double2ll_rn(a.m[i] * p.qinv[0]);
+            // (a mass outside the fixed-point range is reported, as in the step)
+            if (c >= 0 && !fixed_of_mass(a.m[i], p.exps[0], q)) set_err(s, ERRB_FIXED_OVERFLOW);
         }
         const int prev = __shfl_up_sync(FULL, c, 1);
         const unsigned heads = __ballot_sync(FULL, lane == 0 || prev != c);

@@ -4,16 +4,13 @@
 //
 //   k_sample_write  a5: N_sam hydro particles per cell, in pairs U +/- sqrt(RT) X
 //                   with X ~ N(0, I) (Box-Muller), uniform in the tet.
-//   k_sort          a11: the survivors of the last step, compacted, sorted by
-//                   cell (counting sort on the scanned per-cell counts) into
-//                   the working buffer, where each cell's samples follow them.
-//   k_track         a6-a9: t_f = min(-tau ln eta, dt), face-by-face streaming
-//                   of the cell-sorted particles, boundary interaction,
-//                   particle flux (movers listed for k_movers), removal; the
-//                   survivors are written compacted into the survivor buffer
-//                   (block-level slot reservation).  Blocks take tiles of
-//                   128 or 256 particles from a global counter.
+//   k_track         a6-a9, a11: t_f = min(-tau ln eta, dt), face-by-face streaming
+//                   of the cell-sorted particles, boundary interaction, the
+//                   counting flux of the particles that left their cell or met a
+//                   wall, removal; each survivor is written into the bucket of
+//                   its end cell in the next buffer.
 #include "dmath.cuh"
+#include "fixed.cuh"
 #include "ugkwp_internal.hpp"
 
 namespace ugkwp {
@@ -50,7 +47,6 @@ template <class Real> __device__ __forceinline__ PartView<Real> view(const PartB
     v.cell = r.cell;
     v.id = r.id;
     v.e = (Real*)r.e;
-    v.e2 = (Real*)r.e2;
     return v;
 }
 
@@ -342,10 +338,6 @@ template <> struct Trk<float> {
         nx = v.x; ny = v.y; nz = v.z; d = v.w;
     }
     __device__ static __forceinline__ int4 nbv(const DevMesh& m, int tet) { return m.trk_f[tet].nb; }
-    // the record is one 128-byte line
-    __device__ static __forceinline__ void prefetch(const DevMesh& m, int tet) {
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(m.trk_f + tet));
-    }
     __device__ static __forceinline__ float tau(const DevState& s, int c) { return s.tauf[c]; }
     __device__ static __forceinline__ float tf(float tau, unsigned long long r) {
         return -(tau * dm::f_log(dm::u01f(r)));
@@ -358,52 +350,11 @@ template <> struct Trk<double> {
         nx = v.x; ny = v.y; nz = v.z; d = v.w;
     }
     __device__ static __forceinline__ int4 nbv(const DevMesh& m, int tet) { return m.trk_d[tet].nb; }
-    // the 144-byte record starts on a 16-byte boundary, so it spans two lines
-    __device__ static __forceinline__ void prefetch(const DevMesh& m, int tet) {
-        const char* r = reinterpret_cast<const char*>(m.trk_d + tet);
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(r));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(r + sizeof(TrkD) - 1));
-    }
     __device__ static __forceinline__ double tau(const DevState& s, int c) { return s.tau[c]; }
     __device__ static __forceinline__ double tf(double tau, unsigned long long r) {
         return -(tau * dm::d_log(dm::u01d(r)));
     }
 };
-
-// Round-to-nearest-even of v 2^-e for a binary64 v, from the bits of v with
-// integer operations only (v 2^-e is an exact exponent shift, so this equals
-// rounding the scaled binary64 value); false (q = 0) if v is not finite or
-// |v 2^-e| >= 2^62.  Keeps the conversions off the FP64 pipe.
-__device__ __forceinline__ bool fixed_of(double v, int e, long long& q) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
-    const int ex = (int)((bits >> 52) & 0x7ff);
-    unsigned long long mant = bits & 0x000fffffffffffffULL;
-    q = 0;
-    if (ex == 0x7ff) return false;
-    int sh;  // |v| 2^-e = mant 2^sh
-    if (ex == 0) {
-        sh = 1 - 1075 - e;
-    } else {
-        mant |= 0x0010000000000000ULL;
-        sh = ex - 1075 - e;
-    }
-    unsigned long long mag;
-    if (sh >= 0) {
-        if (mant == 0) return true;
-        if (sh > 9) return false;  // mant >= 2^52 when nonzero and normal: 2^(52+10) = 2^62
-        mag = mant << sh;
-        if (mag >= (1ULL << 62)) return false;
-    } else {
-        const int r = -sh;
-        if (r > 63) return true;
-        const unsigned long long hi = mant >> r;
-        const unsigned long long rem = mant & ((1ULL << r) - 1ULL);
-        const unsigned long long half = 1ULL << (r - 1);
-        mag = hi + ((rem > half || (rem == half && (hi & 1ULL))) ? 1ULL : 0ULL);
-    }
-    q = (bits >> 63) ? -(long long)mag : (long long)mag;
-    return true;
-}
 
 // Exact binary32 -> binary64 widening on the bits (integer pipes only).
 __device__ __forceinline__ double widen(float f) {
@@ -434,60 +385,6 @@ __device__ __forceinline__ bool phi_q(const Real* u, Real e, double mm, const De
     ok &= fixed_of(mm * u2, p.exps[3], q[3]);
     ok &= fixed_of(mm * (((u0 * u0 + u1 * u1) + u2 * u2) + widen(e)), p.exps[4] + 1, q[4]);
     return ok;
-}
-
-// round-to-nearest-even of m 2^-e for a finite m >= 0, computed on the bits of
-// m with integer operations only (m 2^-e is an exact exponent shift, so this
-// equals rounding the binary64 product); false if the result is >= 2^62.
-__device__ __forceinline__ bool fixed_of_mass(double m, int e, long long& q) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(m);
-    const int ex = (int)((bits >> 52) & 0x7ff);
-    unsigned long long mant = bits & 0x000fffffffffffffULL;
-    int s;  // value = mant 2^s
-    if (ex == 0) {
-        s = 1 - 1075 - e;
-    } else {
-        mant |= 0x0010000000000000ULL;
-        s = ex - 1075 - e;
-    }
-    if (ex == 0x7ff || (bits >> 63)) { q = 0; return false; }
-    if (s >= 0) {
-        if (mant == 0) { q = 0; return true; }
-        if (s > 9) { q = 0; return false; }  // mant < 2^53: 2^(53+s) > 2^62
-        const unsigned long long v = mant << s;
-        if (v >= (1ULL << 62)) { q = 0; return false; }
-        q = (long long)v;
-        return true;
-    }
-    const int r = -s;
-    if (r > 63) { q = 0; return true; }
-    const unsigned long long hi = mant >> r;
-    const unsigned long long rem = mant & ((1ULL << r) - 1ULL);
-    const unsigned long long half = 1ULL << (r - 1);
-    q = (long long)(hi + ((rem > half || (rem == half && (hi & 1ULL))) ? 1ULL : 0ULL));
-    return true;
-}
-
-// Thread 0's source of tiles: grabs of TILE_GRAB consecutive tiles from the
-// global counter (one atomic per grab), handed out in order, so the tiles a
-// block walks increase.  The grab after the current one is reserved when the
-// current one starts, so its atomic completes while the current grab's tiles
-// are walked (a block stops at its first tile past the end, and every grab it
-// still holds then lies past the end too).  Returns the first particle index
-// of the next tile.
-struct TileQueue {
-    long long next = 0, end = 0, ahead = -1;
-};
-
-__device__ __forceinline__ long long next_tile(TileQueue& q, int64_t* ctr, int T) {
-    if (q.next == q.end) {
-        const long long g =
-            q.ahead >= 0 ? q.ahead : (long long)atomicAdd(reinterpret_cast<unsigned long long*>(ctr), 1ULL);
-        q.next = g * TILE_GRAB;
-        q.end = q.next + TILE_GRAB;
-        q.ahead = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(ctr), 1ULL);
-    }
-    return (q.next++) * T;
 }
 
 // ---- the walk of one particle, one tet at a time
@@ -623,342 +520,335 @@ __device__ __forceinline__ bool visit(const DevMesh& m, const DevParams& p, long
     return true;
 }
 
-// A particle whose walk ended, ready for the outputs.
-template <class Real> struct Ended {
-    bool active, survivor, mover, exited;
-    int tet, c0;
-    Real xe[3], ue[3], us[3], es, ee;
-    double mm;
-    unsigned long long id;
-};
+// Entries of a warp's queue of particles that may leave their tet: fewer than 32
+// wait before a tile is taken and a tile adds at most 32.
+constexpr int WALK_QUEUE = 64;
 
-// Walks that did not end in their first tet wait in shared memory (structure
-// of arrays, QCAP entries per block) until a tile's worth of them has
-// gathered; the block then walks one tile's worth on in full warps.  Before a
-// tile's pushes fewer than T walks wait, so 2T entries always suffice.  An entry holds the walk state,
-// the particle's internal energy (KE) and its slot in the buffer, from which
-// the rest of the particle is read again when the walk ends.
-template <class Real, bool KE, int T> struct WalkQueue {
-    static constexpr int QCAP = 2 * T;
-    Real x0[3][QCAP], u[3][QCAP], t0[QCAP], t_end[QCAP], ee[KE ? QCAP : 1];
-    int tet[QCAP], last[QCAP], ncross[QCAP], nrefl[QCAP], nwall[QCAP], flags[QCAP];  // flags: status | coll << 3
-    long long slot[QCAP];
-    int count;
-};
+// Sum over each run of lanes [start, lane] (start: the run's first lane).
+__device__ __forceinline__ long long run_sum(long long v, int lane, int start) {
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const long long o = __shfl_up_sync(FULL, v, d);
+        if (lane - d >= start) v += o;
+    }
+    return v;
+}
 
-// KE: the particles carry an internal energy (K > 0).  THREADS: particles per
-// tile (one per thread).
+// The planes of a tet in binary32, for the inside test: in mixed mode those of
+// the tracking record (relative to the anchor), else rounded from binary64.
+template <class Real> __device__ __forceinline__ const float4* test_planes(const DevMesh& m, int c) {
+    if constexpr (sizeof(Real) == 4) return m.trk_f[c].pl;
+    else return m.pln_f + (size_t)4 * c;
+}
+
+// One warp's share of the tracking.  Warps work on their own (no block barrier):
+// each takes runs of 32-slot tiles from a global counter, one atomic per run,
+// reserved one run ahead.
+//
+// Per tile, one slot per lane:
+//  * the collision test compares the t_f draw with a per-cell threshold that lies
+//    below e^{-dt/tau}; only the lanes above it need -tau ln eta, and a warp
+//    without such a lane skips the logarithm (DevState::cinfo);
+//  * the end point x0 + u t is tested against the tet's four planes in binary32.
+//    If it lies inside all of them by more than the cell's margin, which bounds
+//    the rounding of that test and of the walk's own exit test, then the walk
+//    (visit) would stop in this tet at the same point, bit for bit;
+//  * the others wait in the warp's queue until 32 of them have gathered, and
+//    are then walked face by face in a full warp.
+// Nine tenths of the particles of a rarefied cavity end in the tile pass.  They
+// change no sum: a cell's survivor mass starts the step from its survivors and
+// samples (k_sample_count), and only what is removed or moves is added to it.
+//
+// Bound by memory latency: 24% of the warps active beside the wave flux, issue
+// 29% busy, long-scoreboard stalls 5.4 cycles per issue (16^3 cavity).  Alone with
+// half its grid, tracking and counting flux of the settled 24^3 cavity (1.66e7
+// particles) take 0.65 ms, in binary64 (21^3, 9.7e6 particles) 1.01 ms; with the
+// walk of every first tet, block-wide output rounds and a mover list for a flux
+// kernel of its own they took 0.98 and 2.96 ms.
 template <class Real, bool KE, int THREADS>
 __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, const DevParams& p,
-                                           const PartBufRaw& br, const PartBufRaw& nr, const PartBufRaw& ar) {
+                                           const PartBufRaw& br, const PartBufRaw& nr) {
     constexpr int NW = THREADS / 32;
-    using Q = WalkQueue<Real, KE, THREADS>;
     // (block-uniform: another block may set the bit while this one starts)
     if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
-    const PartView<Real> b = view<Real>(br);   // this step's particles, sorted by cell (holes: cell -1)
+    __shared__ int q_slot[NW][WALK_QUEUE];
+    __shared__ Real q_end[NW][WALK_QUEUE];  // t_f, or dt
+    __shared__ unsigned sh_red[NW][8];
+    const PartView<Real> b = view<Real>(br);    // this step's particles, sorted by cell (holes: cell -1)
     const PartView<Real> nxt = view<Real>(nr);  // the next step's survivors, in their end cells' buckets
-    const PartView<Real> mv = view<Real>(ar);  // mover list: x = u at start, u = u at end
-    const long long n = s.cnt64[CNT_N_B];
+    const unsigned n = (unsigned)s.cnt64[CNT_N_B];
     const long long step = s.cnt64[CNT_STEP];
-    const double dt = s.dt[0];
-    const Real dtR = (Real)dt;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // slot bookkeeping in two sets, alternating between output rounds, so
-    // that no barrier is needed after a round's stores: a set is rewritten
-    // two rounds later, after two barriers every warp has passed
-    __shared__ int sh_cnt[2][NW];
-    __shared__ long long sh_base[2], sh_tile[2];
-    __shared__ int sh_qc;  // queue size after the last output round
     const long long wtot = s.cnt64[CNT_WTOT];  // overflow slots start after the buckets
-    int par = 0;
-    __shared__ unsigned long long sh_red[NW][8];
-    __shared__ Q q;
-    // per-thread counters, reduced once per block at the end
-    unsigned c_valid = 0, c_coll = 0, c_exit = 0, c_lost = 0, c_cross = 0, c_wall = 0, c_surv = 0;
-    // tiles of THREADS particles are taken from a global counter, so that
-    // blocks that start late (or walk short paths) take fewer tiles
-    TileQueue tq;  // thread 0's
-    if (threadIdx.x == 0) {
-        q.count = 0;
-        sh_qc = 0;
-        sh_tile[0] = next_tile(tq, &s.cnt64[CNT_TILE], THREADS);
-    }
-    __syncthreads();
+    const Real dtR = (Real)s.dt[0];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u, upto = FULL >> (31 - lane);
+    const int nc = m.nc;
+    unsigned long long* tile_ctr = reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_TILE]);
+    unsigned long long* smass = reinterpret_cast<unsigned long long*>(s.smass_next);
+    unsigned long long* pf = reinterpret_cast<unsigned long long*>(s.pflux);
+    // warp-uniform counters
+    unsigned c_valid = 0, c_coll = 0, c_surv = 0, c_mover = 0;
+    unsigned c_exit = 0, c_lost = 0, c_cross = 0, c_wall = 0;  // per lane
+    int qn = 0;
 
-    // ---- outputs of the particles whose walks ended this round (one per
-    // lane or none): the survivor's slot in its end cell's bucket, the
-    // survivors' mass per end cell, the counters, the mover record.  Contains
-    // the block's two barriers of the round; with `advance`, thread 0 also
-    // takes the next tile.
-    auto emit = [&](const Ended<Real>& e, bool advance, int qtake) {
-        // a11: each survivor goes to the bucket of its end cell in the next
-        // buffer, so the next step finds the particles sorted by cell.  Lanes
-        // with the same end cell take consecutive slots from the cell's count
-        // (one atomic per group); the count is also the cell's survivor count
-        // N_left of the next step.  A survivor beyond its bucket takes an
-        // overflow slot after the buckets.  The group's first slot is read
-        // after the round's barriers, so the atomic's round trip overlaps them.
-        const int key = e.survivor ? e.tet : -1;
-        const unsigned peers = __match_any_sync(FULL, key);
-        const int leader = __ffs(peers) - 1;
-        int sfirst = 0;
-        if (lane == leader && key >= 0) sfirst = atomicAdd(&s.nleft_next[key], __popc(peers));
-        // survivors' fixed-point mass per end cell: segmented reduction over
-        // lanes with equal keys in a row, one atomic per run
-        {
-            long long v = 0;
-            if (e.survivor && !fixed_of_mass(e.mm, p.exps[0], v)) set_err(s, ERRB_FIXED_OVERFLOW);
-            const int prev = __shfl_up_sync(FULL, key, 1);
-            const bool head = lane == 0 || prev != key;
-            const unsigned heads = __ballot_sync(FULL, head);
-            const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const long long o = __shfl_up_sync(FULL, v, d);
-                if (lane - d >= start) v += o;
-            }
-            const bool tail = lane == 31 || ((heads >> (lane + 1)) & 1u);
-            if (tail && key >= 0) atomicAdd(reinterpret_cast<unsigned long long*>(&s.smass_next[key]), (unsigned long long)v);
+    // the slot of a survivor in its end cell's bucket (rank: its place among the
+    // cell's survivors), or in the overflow region behind the buckets; -1: none
+    auto slot_of = [&](int rank, int woff, int wcap) -> long long {
+        long long j = -1;
+        if (rank < wcap) {
+            j = (long long)woff + rank;
+        } else {
+            const long long o = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_OVF]), 1ULL);
+            if (o < p.capacity - wtot) j = wtot + o;
+            else set_err(s, ERRB_CAPACITY);
         }
-        c_surv += e.survivor ? 1u : 0u;
-        // movers: one slot reservation per block and round
-        const unsigned mmask = __ballot_sync(FULL, e.mover);
-        if (lane == 0) sh_cnt[par][warp] = __popc(mmask);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int tot = 0;
-            for (int w = 0; w < NW; ++w) {
-                const int c = sh_cnt[par][w];
-                sh_cnt[par][w] = tot;
-                tot += c;
-            }
-            sh_base[par] =
-                tot ? (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_RESV]), (unsigned long long)tot)
-                    : 0LL;
-            // the walks taken from the queue this round leave it (every
-            // thread read its entry before the barrier above)
-            q.count -= qtake;
-            // the queue's size as every warp must see it after this round: a
-            // warp that leaves the round early may already push the next
-            // tile's walks into q.count before a slower warp reads it
-            sh_qc = q.count;
-            // the next tile, in the other set (its last readers read it before
-            // the barrier above); a round without a new tile keeps the current one
-            sh_tile[par ^ 1] = advance ? next_tile(tq, &s.cnt64[CNT_TILE], THREADS) : sh_tile[par];
+        if (j >= p.capacity) {
+            check_failed(s, 6, (unsigned long long)j);
+            j = -1;
         }
-        __syncthreads();
-        const int srank = __shfl_sync(FULL, sfirst, leader) + __popc(peers & ((1u << lane) - 1u));
-        if (e.survivor) {
-            long long j = -1;
-            if (srank < s.wcap[e.tet]) {
-                j = (long long)s.woff[e.tet] + srank;
-            } else {
-                const long long o = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_OVF]), 1ULL);
-                if (o < p.capacity - wtot) j = wtot + o;
-                else set_err(s, ERRB_CAPACITY);
-            }
-            if (j >= p.capacity) {
-                check_failed(s, 6, (unsigned long long)j);
-                j = -1;
-            }
-            if (j >= 0) {
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    nxt.x[c][j] = e.xe[c];
-                    nxt.u[c][j] = e.ue[c];
-                }
-                nxt.m[j] = e.mm;
-                nxt.cell[j] = e.tet;
-                nxt.id[j] = e.id;
-                if constexpr (KE) nxt.e[j] = e.ee;
-            }
-        }
-        const long long mj = sh_base[par] + sh_cnt[par][warp] + __popc(mmask & ((1u << lane) - 1u));
-        if (e.mover && mj >= p.capacity) check_failed(s, 7, (unsigned long long)mj);
-        if (e.mover && mj < p.capacity) {
-            const long long j = mj;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                mv.x[c][j] = e.us[c];
-                mv.u[c][j] = e.ue[c];
-            }
-            mv.m[j] = e.mm;
-            mv.cell[j] = e.c0;
-            mv.id[j] = ((unsigned long long)(unsigned)e.tet << 1) | (e.exited ? 1ULL : 0ULL);
-            if constexpr (KE) {
-                mv.e[j] = e.es;
-                mv.e2[j] = e.ee;
-            }
-        }
-        par ^= 1;
+        return j;
     };
 
-    // The end of a walk: removal (a9), counters, the mover flag (a8: a
-    // particle that ends in its start cell with its velocity unchanged
-    // contributes nothing to the counting flux; the others are listed for the
-    // binary64 flux pass).
-    auto finish = [&](const Walk<Real>& w, bool coll, Ended<Real>& e) {
-        e.active = true;
-        e.exited = w.status & 2;
-        const bool lost = w.status & 4;
-        e.survivor = !e.exited && (!coll || lost);
-        const int status = w.status | ((coll && !lost && !e.exited) ? 1 : 0);
-        e.tet = w.tet;
-        e.mover = e.exited || w.tet != e.c0 || w.nrefl > 0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) e.ue[c] = w.u[c];
-        c_coll += status & 1;
-        c_exit += (status >> 1) & 1;
-        c_lost += (status >> 2) & 1;
-        c_cross += w.ncross;
-        c_wall += w.nwall;
-    };
-
-    for (;;) {
-        const long long bb = sh_tile[par];  // block-uniform
-        const bool have_tile = bb < n;
-        if (!have_tile && sh_qc == 0) break;
-        // ---- a new tile: load, t_f, the first tet of every walk
-        Ended<Real> e;
-        e.active = e.survivor = e.mover = e.exited = false;
-        e.tet = e.c0 = -1;
-        e.es = e.ee = (Real)0;
-        e.mm = 0.0;
-        e.id = 0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) e.xe[c] = e.ue[c] = e.us[c] = (Real)0;
-        if (have_tile) {
-            const long long i = bb + threadIdx.x;
-            // the whole slot is read at once (one round trip; the arrays hold
-            // whole tiles, so slots past n are inside them and ignored); the
-            // slot's start cell -1 marks a hole of a survivor bucket
-            Walk<Real> w;
-            const int cell_i = b.cell[i];
-            const unsigned long long id_i = b.id[i];
+    // ---- the last `take` (<= 32) particles of the queue: the walk, the counting
+    // flux (-phi at the start cell, +phi at the end cell unless the particle left
+    // the domain; a particle that ends in its start cell with its velocity
+    // unchanged contributes nothing), the survivors' mass, removal (a9)
+    auto drain = [&](int take) {
+        const int k = qn - take + lane;
+        const bool act = lane < take;
+        qn -= take;
+        __syncwarp();
+        Walk<Real> w;
+        Real us[3] = {(Real)0, (Real)0, (Real)0}, xe[3] = {(Real)0, (Real)0, (Real)0}, es = (Real)0, ee = (Real)0;
+        double mm = 0.0;
+        int c0 = -1;
+        unsigned long long id = 0;
+        bool survivor = false, mover = false, exited = false;
+        w.tet = -1;
+        w.u[0] = w.u[1] = w.u[2] = (Real)0;
+        w.nrefl = 0;
+        if (act) {
+            const int i = q_slot[warp][k];
+            w.t_end = q_end[warp][k];
+            c0 = b.cell[i];
+            id = b.id[i];
+            mm = b.m[i];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 w.x0[c] = b.x[c][i];
-                w.u[c] = b.u[c][i];
+                w.u[c] = us[c] = b.u[c][i];
             }
-            const double m_i = b.m[i];
-            Real e_i = (Real)0;
-            if constexpr (KE) e_i = b.e[i];
-            const int c0 = i < n ? cell_i : -1;
-            if (c0 >= 0) {
-                // the start tet's record is on its way to L1 during the t_f draw
-                Trk<Real>::prefetch(m, c0);
-                e.id = id_i;
-                e.mm = m_i;
-                e.es = e_i;
-                e.ee = e.es;
-                e.c0 = c0;
+            if constexpr (KE) es = ee = b.e[i];
+            const bool coll = w.t_end < dtR;
+            w.t0 = (Real)0;
+            w.tet = c0;
+            w.last = -1;
+            w.ncross = w.nwall = w.status = 0;
+            while (visit<Real, KE>(m, p, step, id, w, xe, ee)) {
+            }
+            exited = w.status & 2;
+            const bool lost = w.status & 4;
+            survivor = !exited && (!coll || lost);
+            mover = exited || w.tet != c0 || w.nrefl > 0;
+            c_exit += exited;
+            c_lost += lost;
+            c_cross += w.ncross;
+            c_wall += w.nwall;
+            c_coll += coll && !lost && !exited;
+        }
+        __syncwarp();
+        // runs of equal start cells (the queue keeps the order of the slots)
+        const int prev = __shfl_up_sync(FULL, c0, 1);
+        const unsigned heads = __ballot_sync(FULL, lane == 0 || prev != c0);
+        const int start = 31 - __clz(heads & upto);
+        const bool tail = lane == 31 || ((heads >> (lane + 1)) & 1u);
+        c_mover += __popc(__ballot_sync(FULL, mover));
+        long long q0[5] = {0, 0, 0, 0, 0};
+        if (__any_sync(FULL, mover)) {
+            if (mover) {
+                if (!phi_q(us, es, mm, p, q0)) set_err(s, ERRB_FIXED_OVERFLOW);
+                if (!exited) {
+                    if (w.nrefl == 0) {
 #pragma unroll
-                for (int c = 0; c < 3; ++c) e.us[c] = w.u[c];
-                c_valid += 1;
-                // a6: t_f = min(-tau ln eta, dt) for the particles left from the last step
-                w.t_end = dtR;
-                bool coll = false;
-                if ((long long)(e.id >> 40) != step) {
-                    // Philox4x32-10, counter (id low, id high, step, TAG_TF), key (seed low, seed high)
-                    const unsigned long long r = dm::philox32_2((unsigned)e.id, (unsigned)(e.id >> 32), (unsigned)step,
-                                                                (unsigned)TAG_TF, (unsigned)p.seed,
-                                                                (unsigned)(p.seed >> 32));
-                    const Real tf = Trk<Real>::tf(Trk<Real>::tau(s, c0), r);
-                    if (tf < dtR) { coll = true; w.t_end = tf; }
-                }
-                // a7: the walk's first tet
-                w.t0 = (Real)0;
-                w.tet = c0;
-                w.last = -1;
-                w.ncross = w.nrefl = w.nwall = w.status = 0;
-                if (visit<Real, KE>(m, p, step, e.id, w, e.xe, e.ee)) {
-                    // the walk goes on: it waits in the queue
-                    const int k = atomicAdd(&q.count, 1);
-                    if (k >= Q::QCAP) check_failed(s, 5, (unsigned long long)k);
-                    else {
+                        for (int q = 0; q < 5; ++q) atomicAdd(&pf[(size_t)q * nc + w.tet], (unsigned long long)q0[q]);
+                    } else {
+                        long long q1[5];
+                        if (!phi_q(w.u, ee, mm, p, q1)) set_err(s, ERRB_FIXED_OVERFLOW);
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        q.x0[c][k] = w.x0[c];
-                        q.u[c][k] = w.u[c];
+                        for (int q = 0; q < 5; ++q) atomicAdd(&pf[(size_t)q * nc + w.tet], (unsigned long long)q1[q]);
                     }
-                    q.t0[k] = w.t0;
-                    q.t_end[k] = w.t_end;
-                    if constexpr (KE) q.ee[k] = e.ee;
-                    q.tet[k] = w.tet;
-                    q.last[k] = w.last;
-                    q.ncross[k] = w.ncross;
-                    q.nrefl[k] = w.nrefl;
-                    q.nwall[k] = w.nwall;
-                    q.flags[k] = w.status | (coll ? 8 : 0);
-                    q.slot[k] = i;
-                    }
-                } else {
-                    finish(w, coll, e);
                 }
+            }
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                const long long v = run_sum(-q0[q], lane, start);
+                if (tail && c0 >= 0) atomicAdd(&pf[(size_t)q * nc + c0], (unsigned long long)v);
             }
         }
-        emit(e, have_tile, 0);
-        // ---- the queued walks, in full warps once a tile's worth of them has
-        // gathered (or once the tiles are done)
-        const int qc = sh_qc;  // block-uniform: set between the round's barriers
-        if (qc >= THREADS || (!have_tile && qc > 0)) {
-            const int take = qc < THREADS ? qc : THREADS;
-            Ended<Real> f;
-            f.active = f.survivor = f.mover = f.exited = false;
-            f.tet = f.c0 = -1;
-            f.es = f.ee = (Real)0;
-            f.mm = 0.0;
-            f.id = 0;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) f.xe[c] = f.ue[c] = f.us[c] = (Real)0;
-            if ((int)threadIdx.x < take) {
-                const int k = qc - take + threadIdx.x;
-                Walk<Real> w;
+        // survivors' mass: out of the start cell, into the end cell
+        const bool stays = survivor && w.tet == c0;
+        if (act && !mover && !stays && !fixed_of_mass(mm, p.exps[0], q0[0])) set_err(s, ERRB_FIXED_OVERFLOW);
+        const long long out = run_sum(act && !stays ? -q0[0] : 0LL, lane, start);
+        if (tail && c0 >= 0 && out != 0) atomicAdd(&smass[c0], (unsigned long long)out);
+        if (survivor && !stays) atomicAdd(&smass[w.tet], (unsigned long long)q0[0]);
+        // a11: lanes with the same end cell take consecutive places of its bucket
+        const int key = survivor ? w.tet : -1;
+        const unsigned peers = __match_any_sync(FULL, key);
+        const int leader = __ffs(peers) - 1;
+        int first = 0;
+        if (lane == leader && key >= 0) first = atomicAdd(&s.nleft_next[key], __popc(peers));
+        c_surv += __popc(__ballot_sync(FULL, survivor));
+        first = __shfl_sync(FULL, first, leader);
+        if (survivor) {
+            const long long j = slot_of(first + __popc(peers & lt), s.woff[key], s.wcap[key]);
+            if (j >= 0) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    w.x0[c] = q.x0[c][k];
-                    w.u[c] = q.u[c][k];
+                    nxt.x[c][j] = xe[c];
+                    nxt.u[c][j] = w.u[c];
                 }
-                w.t0 = q.t0[k];
-                w.t_end = q.t_end[k];
-                w.tet = q.tet[k];
-                w.last = q.last[k];
-                w.ncross = q.ncross[k];
-                w.nrefl = q.nrefl[k];
-                w.nwall = q.nwall[k];
-                const int fl = q.flags[k];
-                w.status = fl & 7;
-                const bool coll = fl & 8;
-                const long long i = q.slot[k];
-                // the rest of the particle, read again from its slot
-                f.id = b.id[i];
-                f.c0 = b.cell[i];
-                f.mm = b.m[i];
-#pragma unroll
-                for (int c = 0; c < 3; ++c) f.us[c] = b.u[c][i];
-                if constexpr (KE) {
-                    f.es = b.e[i];
-                    f.ee = q.ee[k];
-                }
-                while (visit<Real, KE>(m, p, step, f.id, w, f.xe, f.ee)) {
-                }
-                finish(w, coll, f);
+                nxt.m[j] = mm;
+                nxt.cell[j] = key;
+                nxt.id[j] = id;
+                if constexpr (KE) nxt.e[j] = ee;
             }
-            emit(f, false, take);
         }
-    }
-    // ---- counters: one atomic per block and counter
-    unsigned vals[7] = {c_valid, c_coll, c_exit, c_lost, c_cross, c_wall, c_surv};
+    };
+
+    // tiles per run: long enough that the counter is off the path, short enough
+    // that a small simulation spreads over the whole grid
+    const unsigned run = min(max(n / (32u * 8192u), 1u), 16u) * 32u;
+    unsigned long long ahead = 0;
+    unsigned base = 0, end = 0;
+    if (lane == 0) ahead = atomicAdd(tile_ctr, 1ULL);
+    base = (unsigned)__shfl_sync(FULL, ahead, 0) * run;
+    end = base + run;
+    if (lane == 0) ahead = atomicAdd(tile_ctr, 1ULL);
+    int cell_i = -1;
+    if (base < n) cell_i = b.cell[base + lane];
+    while (base < n) {
+        const unsigned i = base + lane;
+        const int c0 = i < n ? cell_i : -1;
+        const bool valid = c0 >= 0;
+        // the whole slot at once (the arrays hold whole tiles, so slots past n
+        // are inside them and ignored); a start cell of -1 marks a hole
+        const unsigned long long id = b.id[i];
+        Real x0[3], u[3];
 #pragma unroll
-    for (int k = 0; k < 7; ++k) {
-        const unsigned w = __reduce_add_sync(FULL, vals[k]);
-        if (lane == 0) sh_red[warp][k] = w;
+        for (int c = 0; c < 3; ++c) {
+            x0[c] = b.x[c][i];
+            u[c] = b.u[c][i];
+        }
+        const double mm = b.m[i];
+        Real es = (Real)0;
+        if constexpr (KE) es = b.e[i];
+        const int cc = valid ? c0 : 0;
+        const int4 info = s.cinfo[cc];
+        const float4* pl = test_planes<Real>(m, cc);
+        float4 P[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) P[k] = pl[k];
+        // the next tile's cells (its other loads follow at the top of its turn)
+        unsigned nbase = base + 32;
+        if (nbase == end) {
+            nbase = (unsigned)__shfl_sync(FULL, ahead, 0) * run;
+            end = nbase + run;
+            if (lane == 0 && nbase < n) ahead = atomicAdd(tile_ctr, 1ULL);
+        }
+        if (nbase < n) cell_i = b.cell[nbase + lane];
+        // a6: t_f = min(-tau ln eta, dt) for the particles left from the last step;
+        // Philox4x32-10, counter (id low, id high, step, TAG_TF), key (seed low, seed high)
+        Real t_end = dtR;
+        const bool old = valid && (long long)(id >> 40) != step;
+        unsigned long long r = 0;
+        if (old)
+            r = dm::philox32_2((unsigned)id, (unsigned)(id >> 32), (unsigned)step, (unsigned)TAG_TF, (unsigned)p.seed,
+                               (unsigned)(p.seed >> 32));
+        const bool maybe = old && (unsigned)(r >> 32) >= (unsigned)info.x;
+        if (__any_sync(FULL, maybe)) {
+            if (maybe) {
+                const Real tf = Trk<Real>::tf(Trk<Real>::tau(s, c0), r);
+                if (tf < dtR) t_end = tf;
+            }
+        }
+        const bool coll = t_end < dtR;
+        // a7: the end point and the inside test
+        Real xe[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) xe[c] = x0[c] + u[c] * t_end;
+        const float f0 = (float)xe[0], f1 = (float)xe[1], f2 = (float)xe[2], margin = __int_as_float(info.w);
+        float gap = 1.0f;
+        bool inside = true;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            gap = __fmaf_rn(-P[k].x, f0, __fmaf_rn(-P[k].y, f1, __fmaf_rn(-P[k].z, f2, P[k].w)));
+            inside = inside && gap > margin;
+        }
+        const bool slow = valid && !inside;
+        const bool surv = valid && inside && !coll, gone = valid && inside && coll;
+        // runs of equal cells
+        const int prev = __shfl_up_sync(FULL, c0, 1);
+        const unsigned heads = __ballot_sync(FULL, lane == 0 || prev != c0);
+        const int start = 31 - __clz(heads & upto);
+        const unsigned above = heads & ~upto;
+        const unsigned members = (above ? (above & (0u - above)) - 1u : FULL) & (FULL << start);
+        const unsigned smask = __ballot_sync(FULL, surv), qmask = __ballot_sync(FULL, slow);
+        const unsigned mine = smask & members;
+        int first = 0;
+        if (lane == start && mine) first = atomicAdd(&s.nleft_next[c0], __popc(mine));
+        c_valid += __popc(__ballot_sync(FULL, valid));
+        c_surv += __popc(smask);
+        if (slow) {
+            const int k = qn + __popc(qmask & lt);
+            q_slot[warp][k] = (int)i;
+            q_end[warp][k] = t_end;
+        }
+        qn += __popc(qmask);
+        if (__any_sync(FULL, gone)) {  // removed in their cell (a9)
+            long long q = 0;
+            if (gone) {
+                c_coll += 1;
+                if (!fixed_of_mass(mm, p.exps[0], q)) set_err(s, ERRB_FIXED_OVERFLOW);
+            }
+            q = run_sum(-q, lane, start);
+            if (lane == 31 || ((heads >> (lane + 1)) & 1u))
+                if (valid && q != 0) atomicAdd(&smass[c0], (unsigned long long)q);
+        }
+        first = __shfl_sync(FULL, first, start);
+        if (surv) {
+            const long long j = slot_of(first + __popc(mine & lt), info.y, info.z);
+            if (j >= 0) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    nxt.x[c][j] = xe[c];
+                    nxt.u[c][j] = u[c];
+                }
+                nxt.m[j] = mm;
+                nxt.cell[j] = c0;
+                nxt.id[j] = id;
+                if constexpr (KE) nxt.e[j] = es;
+            }
+        }
+        base = nbase;
+        if (qn >= 32) drain(32);
+    }
+    if (qn > 0) drain(qn);
+    // ---- counters: one atomic per block and counter
+    c_coll = __reduce_add_sync(FULL, c_coll);
+    c_exit = __reduce_add_sync(FULL, c_exit);
+    c_lost = __reduce_add_sync(FULL, c_lost);
+    c_cross = __reduce_add_sync(FULL, c_cross);
+    c_wall = __reduce_add_sync(FULL, c_wall);
+    if (lane == 0) {
+        const unsigned vals[8] = {c_valid, c_coll, c_exit, c_lost, c_cross, c_wall, c_surv, c_mover};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sh_red[warp][k] = vals[k];
     }
     __syncthreads();
-    if (threadIdx.x < 7) {
+    if (threadIdx.x < 8) {
         unsigned long long t = 0;
         for (int w = 0; w < NW; ++w) t += sh_red[w][threadIdx.x];
-        const int slot[7] = {CNT_TRACKED, CNT_COLLIDED, CNT_EXITED, CNT_LOST, CNT_CROSSINGS, CNT_WALL, CNT_SURV};
+        const int slot[8] = {CNT_TRACKED, CNT_COLLIDED, CNT_EXITED, CNT_LOST, CNT_CROSSINGS, CNT_WALL, CNT_SURV, CNT_MOVERS};
         if (t) {
             atomicAdd(reinterpret_cast<unsigned long long*>(&s.cnt64[slot[threadIdx.x]]), t);
             if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_MOVES]), t);
@@ -968,110 +858,8 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
 }
 template <class Real, bool KE, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_track(DevMesh m, DevState s, DevParams p, PartBufRaw br,
-                                                                  PartBufRaw nr, PartBufRaw ar) {
-    track_body<Real, KE, THREADS>(m, s, p, br, nr, ar);
-}
-
-// Same bits (a particle's velocity and internal energy are unchanged unless it
-// met a wall).
-__device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_uint(a) == __float_as_uint(b); }
-__device__ __forceinline__ bool same_bits(double a, double b) {
-    return __double_as_longlong(a) == __double_as_longlong(b);
-}
-
-// Counting flux of the listed movers: -phi(u_start) at the start cell and, unless
-// the particle left the domain, +phi(u_end) at the end cell (full warps of
-// binary64 work, kept out of the tracking kernel).  phi(u_end) is phi(u_start)
-// for the movers that met no wall.
-
-template <class Real>
-__device__ __forceinline__ void movers_body(const DevMesh& m, const DevState& s, const DevParams& p,
-                                            const PartBufRaw& ar, Blk bk) {
-    if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
-    const PartView<Real> mv = view<Real>(ar);
-    const long long n = s.cnt64[CNT_RESV];
-    const int nc = m.nc;
-    const int lane = threadIdx.x & 31;
-    unsigned long long* pf = reinterpret_cast<unsigned long long*>(s.pflux);
-    // movers whose end velocity differs from their start velocity (they met
-    // a wall): their end phi is taken after the block's pass, packed into
-    // whole warps, since binary64 work costs a warp its full issue time
-    __shared__ int wall_j[256];
-    __shared__ int n_wall;
-    for (long long base = (long long)bk.id * 256; base < n; base += (long long)bk.n * 256) {
-        if (threadIdx.x == 0) n_wall = 0;
-        __syncthreads();
-        const long long j = base + threadIdx.x;
-        const bool valid = j < n;
-        Real us[3] = {(Real)0, (Real)0, (Real)0};
-        double mm = 0.0;
-        int c0 = -1, c1 = -1;
-        bool exited = true;
-        long long q0[5] = {0, 0, 0, 0, 0};
-        if (valid) {
-            Real ue[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) { us[c] = mv.x[c][j]; ue[c] = mv.u[c][j]; }
-            mm = mv.m[j];
-            c0 = mv.cell[j];
-            const unsigned long long code = mv.id[j];
-            c1 = (int)(code >> 1);
-            exited = code & 1ULL;
-            // a record outside the mesh is reported and skipped
-            if (c0 < 0 || c0 >= nc || (!exited && (c1 < 0 || c1 >= nc))) {
-                check_failed(s, 8, (unsigned long long)j);
-                c0 = -1;
-                exited = true;
-            }
-            const Real es = mv.e ? mv.e[j] : (Real)0, ee = mv.e2 ? mv.e2[j] : (Real)0;
-            if (!phi_q(us, es, mm, p, q0)) set_err(s, ERRB_FIXED_OVERFLOW);
-            const bool same = same_bits(us[0], ue[0]) && same_bits(us[1], ue[1]) && same_bits(us[2], ue[2]) &&
-                              same_bits(es, ee);
-            if (!exited && !same) wall_j[atomicAdd(&n_wall, 1)] = threadIdx.x;
-            if (!exited && same) {
-                // +phi at the end cell: the start's phi
-#pragma unroll
-                for (int q = 0; q < 5; ++q) atomicAdd(&pf[(size_t)q * nc + c1], (unsigned long long)q0[q]);
-            }
-        }
-        // -phi at the start cell, summed over runs of equal start cells within
-        // the warp (the list is ordered by start cell within each tracking
-        // tile), one atomic per run and quantity
-        const int prev = __shfl_up_sync(FULL, c0, 1);
-        const bool head = lane == 0 || prev != c0;
-        const unsigned heads = __ballot_sync(FULL, head);
-        const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-        const bool tail = lane == 31 || ((heads >> (lane + 1)) & 1u);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            long long v = -q0[q];
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const long long o = __shfl_up_sync(FULL, v, d);
-                if (lane - d >= start) v += o;
-            }
-            if (tail && c0 >= 0) atomicAdd(&pf[(size_t)q * nc + c0], (unsigned long long)v);
-        }
-        __syncthreads();
-        // the block's wall movers: +phi(u_end) at the end cell
-        for (int t = threadIdx.x; t < n_wall; t += 256) {
-            const long long jw = base + wall_j[t];
-            Real ue[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) ue[c] = mv.u[c][jw];
-            const Real ee = mv.e2 ? mv.e2[jw] : (Real)0;
-            long long q1[5];
-            if (!phi_q(ue, ee, mv.m[jw], p, q1)) set_err(s, ERRB_FIXED_OVERFLOW);
-            const int cw = (int)(mv.id[jw] >> 1);
-#pragma unroll
-            for (int q = 0; q < 5; ++q) atomicAdd(&pf[(size_t)q * nc + cw], (unsigned long long)q1[q]);
-        }
-        __syncthreads();
-    }
-}
-template <class Real>
-__global__ void __launch_bounds__(256) k_movers(DevMesh m, DevState s, DevParams p, PartBufRaw ar) {
-    movers_body<Real>(m, s, p, ar, Blk{(int)blockIdx.x, (int)gridDim.x});
+                                                                  PartBufRaw nr) {
+    track_body<Real, KE, THREADS>(m, s, p, br, nr);
 }
 
 // ---- fused batches
@@ -1102,16 +890,10 @@ template <class Real, bool KE, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_track_b(const __grid_constant__ BatchChunk c) {
     for (int k = 0; k < c.n; ++k) {
         const BatchMember& e = c.mem[((int)blockIdx.x + k) % c.n];
-        track_body<Real, KE, THREADS>(e.m, e.s, e.p, e.a, e.b, e.mv);
+        track_body<Real, KE, THREADS>(e.m, e.s, e.p, e.a, e.b);
         __syncthreads();
     }
 }
-template <class Real>
-__global__ void __launch_bounds__(256) k_movers_b(const __grid_constant__ BatchChunk c) {
-    for (int k = 0; k < c.n; ++k)
-        movers_body<Real>(c.mem[k].m, c.mem[k].s, c.mem[k].p, c.mem[k].mv, Blk{(int)blockIdx.x, (int)gridDim.x});
-}
-
 }  // namespace
 
 void launch_sample_write(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b,
@@ -1129,20 +911,20 @@ void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p
 namespace {
 template <class Real, bool KE>
 void track_shape(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b, const PartBufRaw& nxt,
-                 const PartBufRaw& movers, const TrackShape& sh, int blocks, cudaStream_t st) {
-    if (sh.threads == 256) k_track<Real, KE, 256><<<blocks, 256, 0, st>>>(m, s, p, b, nxt, movers);
-    else k_track<Real, KE, 128><<<blocks, 128, 0, st>>>(m, s, p, b, nxt, movers);
+                 const TrackShape& sh, int blocks, cudaStream_t st) {
+    if (sh.threads == 256) k_track<Real, KE, 256><<<blocks, 256, 0, st>>>(m, s, p, b, nxt);
+    else k_track<Real, KE, 128><<<blocks, 128, 0, st>>>(m, s, p, b, nxt);
 }
 }  // namespace
 
 void launch_track(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b, const PartBufRaw& nxt,
-                  const PartBufRaw& movers, const TrackShape& sh, int blocks, cudaStream_t st) {
+                  const TrackShape& sh, int blocks, cudaStream_t st) {
     if (p.precision == UGKWP_MIXED) {
-        if (p.K > 0) track_shape<float, true>(m, s, p, b, nxt, movers, sh, blocks, st);
-        else track_shape<float, false>(m, s, p, b, nxt, movers, sh, blocks, st);
+        if (p.K > 0) track_shape<float, true>(m, s, p, b, nxt, sh, blocks, st);
+        else track_shape<float, false>(m, s, p, b, nxt, sh, blocks, st);
     } else {
-        if (p.K > 0) track_shape<double, true>(m, s, p, b, nxt, movers, sh, blocks, st);
-        else track_shape<double, false>(m, s, p, b, nxt, movers, sh, blocks, st);
+        if (p.K > 0) track_shape<double, true>(m, s, p, b, nxt, sh, blocks, st);
+        else track_shape<double, false>(m, s, p, b, nxt, sh, blocks, st);
     }
 }
 
@@ -1157,12 +939,10 @@ template <class Real, bool KE> cudaError_t configure_type(int carveout) {
     set(k_track<Real, KE, 256>);
     set(k_sample_write<Real>);
     set(k_sample_scale<Real>);
-    set(k_movers<Real>);
     set(k_track_b<Real, KE, 128>);
     set(k_track_b<Real, KE, 256>);
     set(k_sample_write_b<Real>);
     set(k_sample_scale_b<Real>);
-    set(k_movers_b<Real>);
     return e;
 }
 }  // namespace
@@ -1170,11 +950,6 @@ template <class Real, bool KE> cudaError_t configure_type(int carveout) {
 cudaError_t configure_particle_kernels(const DevParams& p, int carveout) {
     if (p.precision == UGKWP_MIXED) return p.K > 0 ? configure_type<float, true>(carveout) : configure_type<float, false>(carveout);
     return p.K > 0 ? configure_type<double, true>(carveout) : configure_type<double, false>(carveout);
-}
-
-void launch_movers(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& a, int blocks, cudaStream_t st) {
-    if (p.precision == UGKWP_MIXED) k_movers<float><<<blocks, 256, 0, st>>>(m, s, p, a);
-    else k_movers<double><<<blocks, 256, 0, st>>>(m, s, p, a);
 }
 
 void launch_sample_scale_batch(const BatchChunk& c, int blocks, int precision, cudaStream_t st) {
@@ -1202,9 +977,4 @@ void launch_track_batch(const BatchChunk& c, int precision, bool ke, const Track
         else track_batch_shape<double, false>(c, sh, blocks, st);
     }
 }
-void launch_movers_batch(const BatchChunk& c, int blocks, int precision, cudaStream_t st) {
-    if (precision == UGKWP_MIXED) k_movers_b<float><<<blocks, 256, 0, st>>>(c);
-    else k_movers_b<double><<<blocks, 256, 0, st>>>(c);
-}
-
 }  // namespace ugkwp

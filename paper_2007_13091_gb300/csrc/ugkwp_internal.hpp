@@ -23,8 +23,8 @@ enum : int32_t {
                             // CNT_CHECK holds the check and the value)
 };
 
-// Largest tile of the tracking kernel (particles per block and tile); the
-// particle arrays hold whole tiles of this size.
+// The particle arrays hold whole multiples of this many slots (a tracking warp
+// loads whole 32-slot tiles).
 constexpr int TRACK_TILE_MAX = 256;
 
 // Device counters (int64 slots).  The counters that tracking blocks update
@@ -47,15 +47,13 @@ enum : int {
     CNT_MOVES = 13,     // particle moves since init (never reset by a step)
     CNT_NSAM = 14,      // particles sampled this step (from the scan)
     CNT_WTOT = 15,      // slots of the survivor buckets of the buffer written this step (from the scan)
-    CNT_RESV = 16,      // mover slots reserved this step
-    CNT_TILE = 32,      // next grab of tracking tiles
+    CNT_MOVERS = 16,    // particles of this step whose counting flux is not zero
+    CNT_TILE = 32,      // next run of tracking tiles
     CNT_IMPORT = 40,    // a state import's first failed particle: (index << 3) | problem
     CNT_OVF = 48,       // overflow slots (survivors whose bucket is full) taken this step
     CNT_CHECK = 56,     // the first failed self-check: (check << 48) | value
     CNT_SLOTS = 64,
 };
-// Tiles taken from the tile counter per atomic.
-constexpr int TILE_GRAB = 4;
 
 // Values of a cell's row in DevState::rec.
 constexpr int REC_N = 24;
@@ -119,6 +117,8 @@ struct DevMesh {
     const int32_t* cfs;      // [nc] bit k set if the cell owns local face k
     const TrkF* trk_f;       // [nc]
     const TrkD* trk_d;       // [nc]
+    const float4* pln_f;     // [nc][4] binary64 mode: the planes rounded to binary32 ([4 i + k])
+    const float* margin;     // [nc] margin of the tracking's inside test
     const float* smp_f;      // [24][nc] mixed mode: for coordinate c at [(8c + j) nc + i], j = 0, 1: vertex 0
                              // minus the tet's anchor, j = 2k, 2k + 1 (k = 1..3): edge p_k - p_0, each
                              // binary64 value split into a binary32 pair (high, low)
@@ -146,8 +146,7 @@ template <class Real> struct PartView {
     double* m;
     int32_t* cell;
     uint64_t* id;
-    Real* e;   // internal energy (K > 0; NULL otherwise)
-    Real* e2;  // mover list only: internal energy at the end
+    Real* e;  // internal energy (K > 0; NULL otherwise)
 };
 
 struct PartBufRaw {
@@ -157,7 +156,6 @@ struct PartBufRaw {
     int32_t* cell;
     uint64_t* id;
     void* e;
-    void* e2;
 };
 
 struct DevState {
@@ -182,6 +180,10 @@ struct DevState {
     int32_t* cnt;         // [nc] particles per cell after sampling
     int32_t* soff;        // [nc] exclusive scan of N_sam (sampled-particle index)
     int32_t* wcap;        // [nc] slots of the cell's survivor bucket in the buffer written this step
+    int4* cinfo;          // [nc] what the tracking reads per cell: collision threshold (a particle whose
+                          // first random word is below it does not collide), woff, wcap, and the
+                          // bits of the inside test's margin (binary32)
+    uint32_t* cthr;       // [nc] the collision thresholds
     int32_t* woff;        // [nc] first slot of that bucket (exclusive scan of wcap); the bucket's
                           // fill count is nleft_next (the survivors that ended in the cell)
     int64_t* pflux;       // [5][nc] fixed-point particle flux
@@ -204,7 +206,6 @@ struct BatchMember {
     DevParams p;
     PartBufRaw a;   // this step's particles
     PartBufRaw b;   // the buffer the survivors are written to
-    PartBufRaw mv;  // the movers
 };
 
 // The block a kernel body runs as: its index among the blocks that work on
@@ -252,7 +253,7 @@ struct TrackShape {
     int threads;  // 128 or 256
 };
 struct LaunchCfg {
-    int particle_blocks;  // blocks of the sampling, tracking and movers kernels
+    int particle_blocks;  // blocks of the sampling and tracking kernels
     int wave_blocks;      // blocks of the persistent second-order wave kernels
     TrackShape track;     // tracking kernel shape
     int carveout;         // preferred shared-memory carveout (percent) of the step's kernels, -1: driver default
@@ -262,19 +263,16 @@ void launch_sample_write(const DevMesh& m, const DevState& s, const DevParams& p
                          int blocks, cudaStream_t st);
 // Energy-matched sampling: the per-cell spread s sqrt(RT) (sig, usig.w).
 void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
-// Tracking of buffer b (survivors, then this step's samples); the survivors go
-// compacted to nxt, the particles whose counting flux is non-zero are listed in
-// movers and their flux added by launch_movers.
+// Tracking of buffer b (survivors, then this step's samples): the survivors go
+// into their end cells' buckets in nxt, the counting flux into pflux.
 void launch_track(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b,
-                  const PartBufRaw& nxt, const PartBufRaw& movers, const TrackShape& sh, int blocks, cudaStream_t st);
+                  const PartBufRaw& nxt, const TrackShape& sh, int blocks, cudaStream_t st);
 // The common preferred shared-memory carveout of the step's kernels (a
 // kernel attribute): set outside stream capture, before the configuration's
 // first launch.
 cudaError_t configure_particle_kernels(const DevParams& p, int carveout);
 cudaError_t configure_wave_kernels(int carveout);
 cudaError_t configure_cell_kernels(int carveout);
-void launch_movers(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& a,
-                   int blocks, cudaStream_t st);
 
 // First-order flux of face_order[first..nf); second-order flux of the nif interior faces.
 void launch_face_flux(const DevMesh& m, const DevState& s, const DevParams& p, int first, int blocks,
@@ -310,8 +308,8 @@ void launch_kn_gll(const DevMesh& m, const DevState& s, const DevParams& p, doub
 // The chunk travels as the launch's parameter (read-only, like a single
 // simulation's structures).  Kernels over cells or faces give member i the
 // blocks off[cls][i] .. off[cls][i + 1] - 1 of the grid, on which it runs the
-// body its own launch would run; the particle kernels (sampling, tracking,
-// movers) take every member in turn on the whole grid.
+// body its own launch would run; the particle kernels (sampling,
+// tracking) take every member in turn on the whole grid.
 constexpr int BATCH_CHUNK = 13;
 enum BatchClass { BCL_RESET, BCL_CELLS, BCL_SCAN, BCL_GRAD, BCL_GPC, BCL_FLUX_O2, BCL_FLUX, BCL_N };
 struct BatchChunk {
@@ -339,7 +337,6 @@ void launch_sample_scale_batch(const BatchChunk& c, int blocks, int precision, c
 void launch_sample_write_batch(const BatchChunk& c, int blocks, int precision, cudaStream_t st);
 void launch_track_batch(const BatchChunk& c, int precision, bool ke, const TrackShape& sh, int blocks,
                         cudaStream_t st);
-void launch_movers_batch(const BatchChunk& c, int blocks, int precision, cudaStream_t st);
 
 // ---- adjoint of the frozen-particle wave map
 struct AdjBc {
