@@ -395,6 +395,71 @@ template <class Real> struct Walk {
     int tet, last, ncross, nrefl, nwall, status;
 };
 
+// Binary32 of a walk's value by truncation, with integer operations only (a
+// conversion would run on the binary64 pipe, which bounds the binary64 mode);
+// values below 2^-126 become 0, values of 2^128 and more, infinities and NaNs
+// become infinity (no test holds for those).
+__device__ __forceinline__ float truncated(float v) { return v; }
+__device__ __forceinline__ float truncated(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), mag = hi & 0x7fffffffu;
+    unsigned f = ((mag - 0x38000000u) << 3) | ((unsigned)__double2loint(v) >> 29);
+    f = mag < 0x38100000u ? 0u : mag >= 0x47f00000u ? 0x7f800000u : f;
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+
+// The exit face of a tet decided in binary32 (binary64 mode): k >= 0 the face, -1
+// the walk stops in the tet, -2 undecided.  un_k = u.n_k and num_k = d_k - n_k.x0
+// carry absolute errors below eu = 2^-20 |u|_1 (truncated u, rounded n, three
+// products: 8 2^-24 |u|_1) and en = the inside test's margin; a comparison counts
+// only beyond these and beyond 2^-20 of its own products, so that it agrees with
+// the binary64 comparison, whose roundings are 2^-29 of that.  About one visit in
+// 300 is undecided (21^3 cavity); one visit in binary64 costs ~70 instructions of
+// the pipe that bounds this mode.
+struct Ray32 {
+    float x[3], u[3], eu;
+};
+template <class Real> __device__ __forceinline__ void ray_start(Ray32& r, const Real* x0, const Real* u) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        r.x[c] = truncated(x0[c]);
+        r.u[c] = truncated(u[c]);
+    }
+    r.eu = (fabsf(r.u[0]) + fabsf(r.u[1]) + fabsf(r.u[2])) * 0x1p-20f;
+}
+__device__ __forceinline__ int exit_face32(const DevMesh& m, const Ray32& r, int tet, int last, float rem) {
+    const float4* pl = m.pln_f + (size_t)4 * tet;
+    const float en = m.margin[tet];
+    float un[4], num[4];
+    bool sure = true;
+    int best = -1;
+    float bn = 0.0f, bu = 1.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 P = pl[k];
+        un[k] = __fmaf_rn(r.u[0], P.x, __fmaf_rn(r.u[1], P.y, r.u[2] * P.z));
+        num[k] = __fmaf_rn(-r.x[0], P.x, __fmaf_rn(-r.x[1], P.y, __fmaf_rn(-r.x[2], P.z, P.w)));
+        if (k == last) un[k] = -1.0f;
+        else sure = sure && fabsf(un[k]) > r.eu;
+        if (un[k] > 0.0f && (best < 0 || num[k] * bu < bn * un[k])) {
+            best = k;
+            bn = num[k];
+            bu = un[k];
+        }
+    }
+    if (!sure) return -2;
+    if (best < 0) return -1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (k == best || un[k] < 0.0f) continue;
+        const float a = num[k] * bu, b = bn * un[k];
+        const float tol = en * (bu + un[k]) + r.eu * (fabsf(num[k]) + fabsf(bn)) + 0x1p-20f * (fabsf(a) + fabsf(b));
+        sure = sure && a - b > tol;
+    }
+    const float t = rem * bu, tol = en + r.eu * rem + 0x1p-20f * (t + fabsf(bn));
+    if (!(sure && fabsf(bn - t) > tol)) return -2;
+    return bn < t ? best : -1;
+}
+
 // One tet of the face-by-face walk (Sec. 2.2 streaming): the exit face is the
 // one with u.n > 0 and the smallest crossing time (d - n.x0)/(u.n), compared
 // by cross products (positive denominators) with one division; ties keep the
@@ -403,7 +468,28 @@ template <class Real> struct Walk {
 // end point), left the domain (status 2) or passed max_crossings (status 4).
 template <class Real, bool KE>
 __device__ __forceinline__ bool visit(const DevMesh& m, const DevParams& p, long long step, unsigned long long id,
-                                      Walk<Real>& w, Real xe[3], Real& ee) {
+                                      Walk<Real>& w, Ray32& ray, Real xe[3], Real& ee) {
+    if constexpr (sizeof(Real) == 8) {
+        // an interior face or an open boundary leaves the ray as it is: the face is
+        // all that is needed, and binary32 decides it
+        const Real rem = w.t_end - w.t0;
+        const int k = exit_face32(m, ray, w.tet, w.last, truncated(rem));
+        if (k == -1) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) xe[c] = w.x0[c] + w.u[c] * rem;
+            return false;
+        }
+        if (k >= 0 && w.ncross < p.max_crossings) {
+            const int4 nbv = Trk<Real>::nbv(m, w.tet);
+            const int code = k == 0 ? nbv.x : k == 1 ? nbv.y : k == 2 ? nbv.z : nbv.w;
+            if (code >= 0) {
+                ++w.ncross;
+                w.tet = code >> 2;
+                w.last = code & 3;
+                return true;
+            }
+        }
+    }
     // the tet's neighbour codes, loaded with its planes (they sit in
     // another sector of the tet's record)
     const int4 nbv = Trk<Real>::nbv(m, w.tet);
@@ -517,22 +603,22 @@ __device__ __forceinline__ bool visit(const DevMesh& m, const DevParams& p, long
     for (int c = 0; c < 3; ++c) w.x0[c] = xh[c];
     w.t0 = w.t0 + sbest;
     w.last = best;
+    if constexpr (sizeof(Real) == 8) ray_start(ray, w.x0, w.u);
     return true;
 }
 
 // Entries of a warp's queue of particles that may leave their tet: fewer than 32
 // wait before a tile is taken and a tile adds at most 32.
 constexpr int WALK_QUEUE = 64;
-
-// Sum over each run of lanes [start, lane] (start: the run's first lane).
-__device__ __forceinline__ long long run_sum(long long v, int lane, int start) {
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const long long o = __shfl_up_sync(FULL, v, d);
-        if (lane - d >= start) v += o;
-    }
-    return v;
-}
+// Lanes of a tile above the collision threshold up to which binary64 defers their
+// logarithm to the queue: two steps of the 21^3 cavity in binary64 2.22 ms with 4,
+// 8 or 16 against 2.52 ms with none.
+constexpr int DEFER_LOG = 8;
+// Threads per SM the tracking kernel is compiled for: 64 registers in mixed mode
+// (80: 1.82 ms against 1.69 ms for two steps of the 24^3 cavity, whose wave flux
+// leaves room for four such blocks per SM), 96 in binary64 (a 20-step run of a tube
+// of 9,600 tets 4.43 ms against 4.71 ms with 64).
+template <class Real> constexpr int TRACK_PER_SM = sizeof(Real) == 4 ? 1024 : 640;
 
 // The planes of a tet in binary32, for the inside test: in mixed mode those of
 // the tracking record (relative to the anchor), else rounded from binary64.
@@ -559,12 +645,16 @@ template <class Real> __device__ __forceinline__ const float4* test_planes(const
 // change no sum: a cell's survivor mass starts the step from its survivors and
 // samples (k_sample_count), and only what is removed or moves is added to it.
 //
-// Bound by memory latency: 24% of the warps active beside the wave flux, issue
-// 29% busy, long-scoreboard stalls 5.4 cycles per issue (16^3 cavity).  Alone with
-// half its grid, tracking and counting flux of the settled 24^3 cavity (1.66e7
-// particles) take 0.65 ms, in binary64 (21^3, 9.7e6 particles) 1.01 ms; with the
-// walk of every first tet, block-wide output rounds and a mover list for a flux
-// kernel of its own they took 0.98 and 2.96 ms.
+// Mixed mode is bound by memory latency: beside the wave flux 15 warps per SM are
+// active and issue is 27% busy, long-scoreboard stalls 6.8 cycles per issue (16^3
+// cavity).  Binary64 is bound by its pipe: what is left there per particle are the
+// end point (6 instructions), and per queued particle the logarithm, the last
+// segment, walls and the counting flux; the exit faces are decided in binary32
+// (exit_face32).  Two steps of the settled 24^3 cavity, mixed, 1.69 ms; of the 21^3
+// cavity in binary64 2.20 ms; with the walk of every first tet, block-wide output
+// rounds and a mover list for a flux kernel of its own 2.20 and 7.33 ms, with
+// every exit face decided in binary64 and no prefetch of the next tile's lines
+// 1.78 and 2.99 ms.
 template <class Real, bool KE, int THREADS>
 __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, const DevParams& p,
                                            const PartBufRaw& br, const PartBufRaw& nr) {
@@ -572,7 +662,7 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
     // (block-uniform: another block may set the bit while this one starts)
     if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
     __shared__ int q_slot[NW][WALK_QUEUE];
-    __shared__ Real q_end[NW][WALK_QUEUE];  // t_f, or dt
+    __shared__ Real q_end[NW][WALK_QUEUE];  // t_f, or dt; -1: not drawn yet
     __shared__ unsigned sh_red[NW][8];
     const PartView<Real> b = view<Real>(br);    // this step's particles, sorted by cell (holes: cell -1)
     const PartView<Real> nxt = view<Real>(nr);  // the next step's survivors, in their end cells' buckets
@@ -593,16 +683,16 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
 
     // the slot of a survivor in its end cell's bucket (rank: its place among the
     // cell's survivors), or in the overflow region behind the buckets; -1: none
-    auto slot_of = [&](int rank, int woff, int wcap) -> long long {
-        long long j = -1;
-        if (rank < wcap) {
-            j = (long long)woff + rank;
-        } else {
+    const int cap = (int)p.capacity;  // < 2^31
+    auto slot_of = [&](int rank, int woff, int wcap) -> int {
+        int j = woff + rank;
+        if (rank >= wcap) {
             const long long o = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_OVF]), 1ULL);
-            if (o < p.capacity - wtot) j = wtot + o;
+            j = -1;
+            if (o < cap - wtot) j = (int)(wtot + o);
             else set_err(s, ERRB_CAPACITY);
         }
-        if (j >= p.capacity) {
+        if (j >= cap) {
             check_failed(s, 6, (unsigned long long)j);
             j = -1;
         }
@@ -639,12 +729,23 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
                 w.u[c] = us[c] = b.u[c][i];
             }
             if constexpr (KE) es = ee = b.e[i];
+            if constexpr (sizeof(Real) == 8) {
+                if (w.t_end < (Real)0) {  // deferred
+                    const unsigned long long r =
+                        dm::philox32_2((unsigned)id, (unsigned)(id >> 32), (unsigned)step, (unsigned)TAG_TF,
+                                       (unsigned)p.seed, (unsigned)(p.seed >> 32));
+                    const Real tf = Trk<Real>::tf(Trk<Real>::tau(s, c0), r);
+                    w.t_end = tf < dtR ? tf : dtR;
+                }
+            }
             const bool coll = w.t_end < dtR;
             w.t0 = (Real)0;
             w.tet = c0;
             w.last = -1;
             w.ncross = w.nwall = w.status = 0;
-            while (visit<Real, KE>(m, p, step, id, w, xe, ee)) {
+            Ray32 ray;
+            if constexpr (sizeof(Real) == 8) ray_start(ray, w.x0, w.u);
+            while (visit<Real, KE>(m, p, step, id, w, ray, xe, ee)) {
             }
             exited = w.status & 2;
             const bool lost = w.status & 4;
@@ -657,11 +758,6 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
             c_coll += coll && !lost && !exited;
         }
         __syncwarp();
-        // runs of equal start cells (the queue keeps the order of the slots)
-        const int prev = __shfl_up_sync(FULL, c0, 1);
-        const unsigned heads = __ballot_sync(FULL, lane == 0 || prev != c0);
-        const int start = 31 - __clz(heads & upto);
-        const bool tail = lane == 31 || ((heads >> (lane + 1)) & 1u);
         c_mover += __popc(__ballot_sync(FULL, mover));
         long long q0[5] = {0, 0, 0, 0, 0};
         if (__any_sync(FULL, mover)) {
@@ -679,17 +775,15 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
                     }
                 }
             }
+            if (mover) {
 #pragma unroll
-            for (int q = 0; q < 5; ++q) {
-                const long long v = run_sum(-q0[q], lane, start);
-                if (tail && c0 >= 0) atomicAdd(&pf[(size_t)q * nc + c0], (unsigned long long)v);
+                for (int q = 0; q < 5; ++q) atomicAdd(&pf[(size_t)q * nc + c0], (unsigned long long)(-q0[q]));
             }
         }
         // survivors' mass: out of the start cell, into the end cell
         const bool stays = survivor && w.tet == c0;
         if (act && !mover && !stays && !fixed_of_mass(mm, p.exps[0], q0[0])) set_err(s, ERRB_FIXED_OVERFLOW);
-        const long long out = run_sum(act && !stays ? -q0[0] : 0LL, lane, start);
-        if (tail && c0 >= 0 && out != 0) atomicAdd(&smass[c0], (unsigned long long)out);
+        if (act && !stays) atomicAdd(&smass[c0], (unsigned long long)(-q0[0]));
         if (survivor && !stays) atomicAdd(&smass[w.tet], (unsigned long long)q0[0]);
         // a11: lanes with the same end cell take consecutive places of its bucket
         const int key = survivor ? w.tet : -1;
@@ -700,7 +794,7 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
         c_surv += __popc(__ballot_sync(FULL, survivor));
         first = __shfl_sync(FULL, first, leader);
         if (survivor) {
-            const long long j = slot_of(first + __popc(peers & lt), s.woff[key], s.wcap[key]);
+            const int j = slot_of(first + __popc(peers & lt), s.woff[key], s.wcap[key]);
             if (j >= 0) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
@@ -724,6 +818,22 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
     base = (unsigned)__shfl_sync(FULL, ahead, 0) * run;
     end = base + run;
     if (lane == 0) ahead = atomicAdd(tile_ctr, 1ULL);
+    // the first lanes prefetch the lines of the next tile's x, u, m and id (its
+    // cells are loaded), one line per lane, with one instruction per tile
+    constexpr int XL = sizeof(Real) / 4;  // lines per coordinate array
+    const char* pptr = nullptr;
+    unsigned pstr = 0;
+    if (lane < 6 * XL) {
+        const int a = lane / XL;
+        pptr = reinterpret_cast<const char*>(a < 3 ? br.x[a] : br.u[a - 3]) + (lane % XL) * 128;
+        pstr = sizeof(Real);
+    } else if (lane < 6 * XL + 2) {
+        pptr = reinterpret_cast<const char*>(br.m) + (lane - 6 * XL) * 128;
+        pstr = 8;
+    } else if (lane < 6 * XL + 4) {
+        pptr = reinterpret_cast<const char*>(br.id) + (lane - 6 * XL - 2) * 128;
+        pstr = 8;
+    }
     int cell_i = -1;
     if (base < n) cell_i = b.cell[base + lane];
     while (base < n) {
@@ -755,7 +865,10 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
             end = nbase + run;
             if (lane == 0 && nbase < n) ahead = atomicAdd(tile_ctr, 1ULL);
         }
-        if (nbase < n) cell_i = b.cell[nbase + lane];
+        if (nbase < n) {
+            cell_i = b.cell[nbase + lane];
+            if (pptr) asm volatile("prefetch.global.L1 [%0];" ::"l"(pptr + (size_t)nbase * pstr));
+        }
         // a6: t_f = min(-tau ln eta, dt) for the particles left from the last step;
         // Philox4x32-10, counter (id low, id high, step, TAG_TF), key (seed low, seed high)
         Real t_end = dtR;
@@ -765,7 +878,11 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
             r = dm::philox32_2((unsigned)id, (unsigned)(id >> 32), (unsigned)step, (unsigned)TAG_TF, (unsigned)p.seed,
                                (unsigned)(p.seed >> 32));
         const bool maybe = old && (unsigned)(r >> 32) >= (unsigned)info.x;
-        if (__any_sync(FULL, maybe)) {
+        // a few lanes: in binary64 they wait for the queue, so that the logarithm
+        // takes the binary64 pipe once per 32 of them
+        const int n_maybe = __popc(__ballot_sync(FULL, maybe));
+        const bool defer = sizeof(Real) == 8 && n_maybe <= DEFER_LOG && maybe;
+        if (n_maybe > (sizeof(Real) == 8 ? DEFER_LOG : 0)) {
             if (maybe) {
                 const Real tf = Trk<Real>::tf(Trk<Real>::tau(s, c0), r);
                 if (tf < dtR) t_end = tf;
@@ -776,7 +893,7 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
         Real xe[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) xe[c] = x0[c] + u[c] * t_end;
-        const float f0 = (float)xe[0], f1 = (float)xe[1], f2 = (float)xe[2], margin = __int_as_float(info.w);
+        const float f0 = truncated(xe[0]), f1 = truncated(xe[1]), f2 = truncated(xe[2]), margin = __int_as_float(info.w);
         float gap = 1.0f;
         bool inside = true;
 #pragma unroll
@@ -784,6 +901,7 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
             gap = __fmaf_rn(-P[k].x, f0, __fmaf_rn(-P[k].y, f1, __fmaf_rn(-P[k].z, f2, P[k].w)));
             inside = inside && gap > margin;
         }
+        inside = inside && !defer;
         const bool slow = valid && !inside;
         const bool surv = valid && inside && !coll, gone = valid && inside && coll;
         // runs of equal cells
@@ -801,22 +919,18 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
         if (slow) {
             const int k = qn + __popc(qmask & lt);
             q_slot[warp][k] = (int)i;
-            q_end[warp][k] = t_end;
+            q_end[warp][k] = defer ? (Real)-1 : t_end;
         }
         qn += __popc(qmask);
-        if (__any_sync(FULL, gone)) {  // removed in their cell (a9)
+        if (gone) {  // removed in its cell (a9)
             long long q = 0;
-            if (gone) {
-                c_coll += 1;
-                if (!fixed_of_mass(mm, p.exps[0], q)) set_err(s, ERRB_FIXED_OVERFLOW);
-            }
-            q = run_sum(-q, lane, start);
-            if (lane == 31 || ((heads >> (lane + 1)) & 1u))
-                if (valid && q != 0) atomicAdd(&smass[c0], (unsigned long long)q);
+            c_coll += 1;
+            if (!fixed_of_mass(mm, p.exps[0], q)) set_err(s, ERRB_FIXED_OVERFLOW);
+            atomicAdd(&smass[c0], (unsigned long long)(-q));
         }
         first = __shfl_sync(FULL, first, start);
         if (surv) {
-            const long long j = slot_of(first + __popc(mine & lt), info.y, info.z);
+            const int j = slot_of(first + __popc(mine & lt), info.y, info.z);
             if (j >= 0) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
@@ -857,7 +971,7 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
     }
 }
 template <class Real, bool KE, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_track(DevMesh m, DevState s, DevParams p, PartBufRaw br,
+__global__ void __launch_bounds__(THREADS, TRACK_PER_SM<Real> / THREADS) k_track(DevMesh m, DevState s, DevParams p, PartBufRaw br,
                                                                   PartBufRaw nr) {
     track_body<Real, KE, THREADS>(m, s, p, br, nr);
 }
@@ -887,7 +1001,7 @@ __global__ void __launch_bounds__(256) k_sample_write_b(const __grid_constant__ 
 // Tiles come from each member's own counter; a block starts at member
 // blockIdx.x mod n, so that the blocks spread over the members' counters.
 template <class Real, bool KE, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_track_b(const __grid_constant__ BatchChunk c) {
+__global__ void __launch_bounds__(THREADS, TRACK_PER_SM<Real> / THREADS) k_track_b(const __grid_constant__ BatchChunk c) {
     for (int k = 0; k < c.n; ++k) {
         const BatchMember& e = c.mem[((int)blockIdx.x + k) % c.n];
         track_body<Real, KE, THREADS>(e.m, e.s, e.p, e.a, e.b);
