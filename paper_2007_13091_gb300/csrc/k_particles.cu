@@ -356,37 +356,6 @@ template <> struct Trk<double> {
     }
 };
 
-// Exact binary32 -> binary64 widening on the bits (integer pipes only).
-__device__ __forceinline__ double widen(float f) {
-    const unsigned b = __float_as_uint(f);
-    const unsigned long long sign = (unsigned long long)(b >> 31) << 63;
-    int ex = (int)((b >> 23) & 0xff);
-    unsigned mant = b & 0x7fffffu;
-    if (ex == 0xff) return __longlong_as_double((long long)(sign | (0x7ffULL << 52) | ((unsigned long long)mant << 29)));
-    if (ex == 0) {
-        if (mant == 0) return __longlong_as_double((long long)sign);
-        const int k = __clz(mant) - 8;  // shift that brings the leading one to bit 23
-        mant = (mant << k) & 0x7fffffu;
-        ex = 1 - k;
-    }
-    return __longlong_as_double(
-        (long long)(sign | ((unsigned long long)(ex - 127 + 1023) << 52) | ((unsigned long long)mant << 29)));
-}
-__device__ __forceinline__ double widen(double d) { return d; }
-
-// Fixed-point image of phi = m (1, u, |u|^2/2); false if a value leaves |v| < 2^62.
-// The factor 1/2 of the energy is applied as an exponent shift.
-template <class Real>
-__device__ __forceinline__ bool phi_q(const Real* u, Real e, double mm, const DevParams& p, long long q[5]) {
-    const double u0 = widen(u[0]), u1 = widen(u[1]), u2 = widen(u[2]);
-    bool ok = fixed_of(mm, p.exps[0], q[0]);
-    ok &= fixed_of(mm * u0, p.exps[1], q[1]);
-    ok &= fixed_of(mm * u1, p.exps[2], q[2]);
-    ok &= fixed_of(mm * u2, p.exps[3], q[3]);
-    ok &= fixed_of(mm * (((u0 * u0 + u1 * u1) + u2 * u2) + widen(e)), p.exps[4] + 1, q[4]);
-    return ok;
-}
-
 // ---- the walk of one particle, one tet at a time
 // Walk state along x0 + u (t - t0): the tet it is in, the face it entered
 // through (or last reflected from, skipped in the exit test), its counters.

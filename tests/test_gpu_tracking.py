@@ -27,3 +27,23 @@ def test_shortcuts_teacher_forced(precision, offset, Kn):
     d = osim.last("counters")
     assert st["n_crossings"] == d["n_crossings"] and st["n_wall_hits"] == d["n_wall_hits"]
     assert st["n_collided"] == d["n_collided"]
+
+
+@pytest.mark.parametrize("precision,K,n", [("fp64", 0, 5), ("fp64", 2, 4), ("mixed", 0, 7), ("mixed", 5, 4)])
+def test_particle_moments_after_steps(precision, K, n):
+    """W^p of a stepped case (buckets with holes, an odd number of slots) against
+    the sums over the exported particles.  Each particle's value is rounded to a
+    quantum of 2^-50 of the largest cell's (about 1e-15 of a cell's W^p), summed
+    over some hundred particles: 1e-12 relative, 1e-12 absolute."""
+    from paper_2007_13091_gb300 import ugkwp
+    cfg = wl.cavity(n=n, N_ref=60, precision=precision, K=K)
+    s = ugkwp.Simulation(cfg["mesh"], cfg["W0"], cfg["params"])
+    s.step(4)
+    st = s.state()
+    nodes, tets = cfg["mesh"]["nodes"], cfg["mesh"]["tets"]
+    vol = np.abs(wl._volumes(nodes, tets))
+    e2 = (st["u"] ** 2).sum(0) + (st["e"] if K else 0.0)
+    phi = np.stack([st["m"], *(st["m"] * st["u"]), 0.5 * st["m"] * e2])
+    WP = np.stack([np.bincount(st["cell"], p, len(tets)) for p in phi]) / vol
+    np.testing.assert_allclose(s.moments(ugkwp.WP), WP, rtol=1e-12, atol=1e-12)
+    np.testing.assert_allclose(s.moments(ugkwp.WH), st["W"] - WP, rtol=1e-11, atol=1e-11)
