@@ -328,7 +328,8 @@ int ugkwp_last(ugkwp_sim* s, int32_t which, void* host_out);
 
 /* Kernel classes of one step, in launch order (for ugkwp_timing_read). */
 enum {
-    UGKWP_K_RESET = 0, UGKWP_K_CELL_PREP, UGKWP_K_SAMPLE_COUNT, UGKWP_K_SCAN,
+    UGKWP_K_RESET = 0, /* no kernel launches in this class: the sums are cleared by the cell kernels */
+    UGKWP_K_CELL_PREP, UGKWP_K_SAMPLE_COUNT, UGKWP_K_SCAN,
     UGKWP_K_SCATTER, /* no kernel launches in this class: the tracking kernel compacts the survivors */
     UGKWP_K_SAMPLE, UGKWP_K_TRACK, UGKWP_K_FLUX, UGKWP_K_UPDATE,
     UGKWP_K_MOVERS,  /* no kernel launches in this class: the tracking kernel adds the counting flux */
@@ -390,8 +391,7 @@ int ugkwp_batch_free(ugkwp_batch* b);
  * synchronises and returns, per kernel class, the summed device time in
  * milliseconds (ms[UGKWP_N_KERNELS]) of the launches timed since the last
  * read, and the number of kernels launched since ugkwp_init
- * (launches[UGKWP_N_KERNELS], counted whether or not timing is enabled; the
- * scan class counts its two kernels); at order 2 the flux class times the
+ * (launches[UGKWP_N_KERNELS], counted whether or not timing is enabled); at order 2 the flux class times the
  * boundary faces and UGKWP_K_FLUX_O2 the interior faces; either pointer may
  * be NULL.  The timed
  * sums are reset by the read. */

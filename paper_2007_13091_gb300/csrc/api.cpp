@@ -697,6 +697,8 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->S.nleft, 0, nc * sizeof(int32_t), st);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->S.smass, 0, nc * sizeof(int64_t), st);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->S.cnt64, 0, CNT_SLOTS * sizeof(int64_t), st);
+    const int64_t none = DT_BITS_NONE;
+    if (ce == cudaSuccess) ce = up(s->S.cnt64 + CNT_DT_BITS, &none, sizeof(none));
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->S.t, 0, sizeof(double), st);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->S.dt, 0, sizeof(double), st);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->S.tsum, 0, sizeof(double), st);
@@ -802,7 +804,6 @@ namespace {
 int enqueue_step(ugkwp_sim* s) {
     cudaStream_t q = s->stream;
     {
-        timed(s, UGKWP_K_RESET, 1, q, [&] { launch_reset(s->M, s->S, q); });
         timed(s, UGKWP_K_CELL_PREP, 1, q, [&] { launch_cell_prep(s->M, s->S, s->P, q); });
         timed(s, UGKWP_K_SAMPLE_COUNT, 1, q, [&] { launch_sample_count(s->M, s->S, s->P, q); });
         // fork: the wave flux needs only W^n, rho^h, tau and dt (ready now) and
@@ -828,7 +829,7 @@ int enqueue_step(ugkwp_sim* s) {
         // beside the tracking; the particle part waits for it
         timed(s, UGKWP_K_UPDATE, 1, s->wave, [&] { launch_wave_update(s->M, s->S, s->wave); });
         CU(cudaEventRecord(s->waved, s->wave));
-        timed(s, UGKWP_K_SCAN, 2, q, [&] { launch_scan(s->M, s->S, s->P, q); });
+        timed(s, UGKWP_K_SCAN, 1, q, [&] { launch_scan(s->M, s->S, s->P, q); });
         if (gp) CU(cudaStreamWaitEvent(q, s->gp_ready, 0));  // the sampler reads the g_p coefficients
         const bool matched = s->P.sampling == UGKWP_SAMPLE_ENERGY_MATCHED;
         timed(s, UGKWP_K_SAMPLE, matched ? 2 : 1, q, [&] {
@@ -870,7 +871,6 @@ int enqueue_gks_step(ugkwp_sim* s, int32_t mode) {
     DevParams P = s->P;
     P.gks = mode;
     P.averaging = 0;
-    timed(s, UGKWP_K_RESET, 1, q, [&] { launch_reset(s->M, s->S, q); });
     timed(s, UGKWP_K_CELL_PREP, 1, q, [&] { launch_cell_prep(s->M, s->S, P, q); });
     timed(s, UGKWP_K_SAMPLE_COUNT, 1, q, [&] { launch_sample_count(s->M, s->S, P, q); });
     if (P.order == 2)
@@ -1177,6 +1177,7 @@ int import_commit(ugkwp_sim* s, int64_t n, int64_t step, double t, const int32_t
     h[CNT_N_A] = n;
     h[CNT_SURV] = n;
     h[CNT_STEP] = step;
+    h[CNT_DT_BITS] = DT_BITS_NONE;
     CU(cudaMemcpyAsync(s->S.cnt64, h, sizeof(h), cudaMemcpyHostToDevice, q));
     CU(cudaMemcpyAsync(s->S.t, &t, sizeof(double), cudaMemcpyHostToDevice, q));
     CU(cudaMemsetAsync(s->S.nleft, 0, nc * sizeof(int32_t), q));
@@ -1761,13 +1762,12 @@ int enqueue_chunk_step(FusedChunk& ch, const std::vector<ugkwp_sim*>& sims) {
     for (int k = 0; k < BCL_N; ++k) c.off[k][0] = 0;
     for (int i = 0; i < c.n; ++i) {
         const int nc = c.mem[i].m.nc;
-        const int per[BCL_N] = {blocks_reset(nc), blocks_cells(nc), scan_blocks(nc), b_grad[i], blocks_gp_coef(nc),
+        const int per[BCL_N] = {blocks_cells(nc), scan_blocks(nc), b_grad[i], blocks_gp_coef(nc),
                                 b_o2[i], b_o1[i]};
         for (int k = 0; k < BCL_N; ++k) c.off[k][i + 1] = c.off[k][i] + per[k];
     }
     auto blocks = [&](int k) { return c.off[k][c.n]; };
     cudaStream_t q = ch.lane;
-    launch_reset_batch(c, blocks(BCL_RESET), q);
     launch_cell_prep_batch(c, blocks(BCL_CELLS), q);
     launch_sample_count_batch(c, blocks(BCL_SCAN), q);
     CU(cudaEventRecord(ch.fork, q));

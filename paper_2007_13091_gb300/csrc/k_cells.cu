@@ -43,32 +43,6 @@ __device__ __forceinline__ int2 block_scan_incl2(int2 v, int2* sh_warp) {
     return v;
 }
 
-__device__ __forceinline__ void reset_body(const DevMesh& m, const DevState& s, Blk bk) {
-    const int nc = m.nc;
-    const long long stride = (long long)bk.n * blockDim.x;
-    for (long long i = (long long)bk.id * blockDim.x + threadIdx.x; i < 5LL * nc; i += stride) {
-        s.pflux[i] = 0;
-        if (i < nc) s.nleft_next[i] = 0;
-    }
-    if (bk.id == 0 && threadIdx.x == 0) {
-        s.cnt64[CNT_SAMPLED] = 0;
-        s.cnt64[CNT_COLLIDED] = 0;
-        s.cnt64[CNT_EXITED] = 0;
-        s.cnt64[CNT_LOST] = 0;
-        s.cnt64[CNT_CROSSINGS] = 0;
-        s.cnt64[CNT_WALL] = 0;
-        s.cnt64[CNT_MOVERS] = 0;
-        s.cnt64[CNT_TRACKED] = 0;
-        s.cnt64[CNT_DT_BITS] = 0x7ff0000000000000LL;  // +inf
-        s.cnt64[CNT_TILE] = 0;
-        s.cnt64[CNT_OVF] = 0;
-        s.cnt64[CNT_SURV] = 0;
-    }
-}
-__global__ void k_reset(DevMesh m, DevState s) {
-    reset_body(m, s, Blk{(int)blockIdx.x, (int)gridDim.x});
-}
-
 // a1 + a2: primitives, tau = mu_ref/p (T/T_ref)^omega, rho^p from the survivors'
 // fixed-point mass, rho^h = rho - rho^p, and min_i |Omega_i| / sum_d Lambda_i^d.
 __device__ __forceinline__ void cell_prep_body(const DevMesh& m, const DevState& s, const DevParams& p, Blk bk) {
@@ -76,6 +50,10 @@ __device__ __forceinline__ void cell_prep_body(const DevMesh& m, const DevState&
     const int i = bk.id * blockDim.x + threadIdx.x;
     double r = __longlong_as_double(0x7ff0000000000000LL);
     if (i < nc) {
+        // the sums this step's tracking adds to
+#pragma unroll
+        for (int q = 0; q < 5; ++q) s.pflux[(size_t)q * nc + i] = 0;
+        s.nleft_next[i] = 0;
         const double rho = s.W[i];
         const double Ux = s.W[nc + i] / rho, Uy = s.W[2 * nc + i] / rho, Uz = s.W[3 * nc + i] / rho;
         const double U2 = (Ux * Ux + Uy * Uy) + Uz * Uz;
@@ -186,55 +164,65 @@ __global__ void k_sample_count(DevMesh m, DevState s, DevParams p) {
     sample_count_body(m, s, p, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
-// Exclusive scan of the block sums (one block): the slots of the survivor
-// buckets of the buffer written this step and the sampled particles (they
-// follow the N_A slots of the current buffer), and the capacity checks.
-__device__ __forceinline__ void scan_bsum_body(const DevState& s, const DevParams& p, int nb) {
+// Offsets of the survivor buckets of the buffer written this step and of the
+// sampled particles (they follow the N_A slots of the current buffer): every
+// block sums the block sums before its own (at most a few per thread) instead of
+// waiting for a scan kernel; the last block has the totals, checks the capacity
+// and clears the counters that the tracking adds to.
+__device__ __forceinline__ void scan_apply_body(const DevMesh& m, const DevState& s, const DevParams& p, Blk bk) {
     __shared__ int2 shw[32];
-    __shared__ long long carry_sh[2];
-    if (threadIdx.x == 0) { carry_sh[0] = 0; carry_sh[1] = 0; }
-    __syncthreads();
-    for (int base = 0; base < nb; base += blockDim.x) {
-        const int j = base + threadIdx.x;
-        const int2 v = j < nb ? s.bsum[j] : make_int2(0, 0);
-        const int2 incl = block_scan_incl2(v, shw);
-        const long long c0 = carry_sh[0], c1 = carry_sh[1];
-        if (j < nb) s.bsum[j] = make_int2((int)(c0 + incl.x - v.x), (int)(c1 + incl.y - v.y));
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) { carry_sh[0] = c0 + incl.x; carry_sh[1] = c1 + incl.y; }
-        __syncthreads();
+    __shared__ long long part[2][32];
+    long long px = 0, py = 0;
+    for (int j = threadIdx.x; j < bk.id; j += blockDim.x) {
+        const int2 v = s.bsum[j];
+        px += v.x;
+        py += v.y;
     }
-    if (threadIdx.x == 0) {
-        const long long total = s.cnt64[CNT_N_A] + carry_sh[1];
-        s.cnt64[CNT_N_B] = total;
-        s.cnt64[CNT_NSAM] = carry_sh[1];
-        s.cnt64[CNT_SAMPLED] = carry_sh[1];
-        s.cnt64[CNT_WTOT] = carry_sh[0];
-        if (total > p.capacity || carry_sh[0] > p.capacity) {
-            set_err(s, ERRB_CAPACITY);
-            s.cnt64[CNT_N_B] = 0;
-            s.cnt64[CNT_NSAM] = 0;
-        }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        px += __shfl_xor_sync(0xffffffffu, px, d);
+        py += __shfl_xor_sync(0xffffffffu, py, d);
     }
-}
-__global__ void k_scan_bsum(DevState s, DevParams p, int nb) {
-    scan_bsum_body(s, p, nb);
-}
-
-__device__ __forceinline__ void scan_apply_body(const DevMesh& m, const DevState& s, Blk bk) {
-    __shared__ int2 shw[32];
+    if ((threadIdx.x & 31) == 0) {
+        part[0][threadIdx.x >> 5] = px;
+        part[1][threadIdx.x >> 5] = py;
+    }
     const int i = bk.id * blockDim.x + threadIdx.x;
     const int2 v = i < m.nc ? make_int2(s.wcap[i], s.nsam[i]) : make_int2(0, 0);
-    const int2 incl = block_scan_incl2(v, shw);
+    const int2 incl = block_scan_incl2(v, shw);  // (its barriers publish part)
+    px = py = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        px += part[0][w];
+        py += part[1][w];
+    }
     if (i < m.nc) {
-        s.soff[i] = s.bsum[bk.id].y + incl.y - v.y;
-        const int woff = s.bsum[bk.id].x + incl.x - v.x;
+        s.soff[i] = (int)py + incl.y - v.y;
+        const int woff = (int)px + incl.x - v.x;
         s.woff[i] = woff;
         s.cinfo[i] = make_int4((int)s.cthr[i], woff, v.x, __float_as_int(m.margin[i]));
     }
+    if (bk.id == bk.n - 1 && threadIdx.x == blockDim.x - 1) {
+        const long long wtot = px + incl.x, nsam = py + incl.y, total = s.cnt64[CNT_N_A] + nsam;
+        const bool fits = total <= p.capacity && wtot <= p.capacity;
+        if (!fits) set_err(s, ERRB_CAPACITY);
+        s.cnt64[CNT_N_B] = fits ? total : 0;
+        s.cnt64[CNT_NSAM] = fits ? nsam : 0;
+        s.cnt64[CNT_SAMPLED] = nsam;
+        s.cnt64[CNT_WTOT] = wtot;
+        s.cnt64[CNT_COLLIDED] = 0;
+        s.cnt64[CNT_EXITED] = 0;
+        s.cnt64[CNT_LOST] = 0;
+        s.cnt64[CNT_CROSSINGS] = 0;
+        s.cnt64[CNT_WALL] = 0;
+        s.cnt64[CNT_MOVERS] = 0;
+        s.cnt64[CNT_TRACKED] = 0;
+        s.cnt64[CNT_TILE] = 0;
+        s.cnt64[CNT_OVF] = 0;
+        s.cnt64[CNT_SURV] = 0;
+    }
 }
-__global__ void k_scan_apply(DevMesh m, DevState s) {
-    scan_apply_body(m, s, Blk{(int)blockIdx.x, (int)gridDim.x});
+__global__ void k_scan_apply(DevMesh m, DevState s, DevParams p) {
+    scan_apply_body(m, s, p, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // a10: W^{n+1} = W^n - 1/|Omega| sum_k (+-F_k |S_k|) + F^{fr,p}/|Omega|, faces
@@ -245,7 +233,10 @@ __device__ __forceinline__ void cell_update_body(const DevMesh& m, const DevStat
     if (p.gks) {
         // GKS step (no particles): W -= sum_k (+-F_k |S_k|) / |Omega|; with local
         // steps F_k holds the flux rate and the cell advances by its own dt
-        if (i == 0 && p.gks == 1) s.t[0] = s.t[0] + s.dt[0];
+        if (i == 0) {
+            if (p.gks == 1) s.t[0] = s.t[0] + s.dt[0];
+            s.cnt64[CNT_DT_BITS] = DT_BITS_NONE;
+        }
         if (i >= nc) return;
         const int own = m.cfs[i];
         const double vol = m.vol[i];
@@ -265,6 +256,7 @@ __device__ __forceinline__ void cell_update_body(const DevMesh& m, const DevStat
         s.t[0] = s.t[0] + s.dt[0];
         if (p.averaging) s.tsum[0] += s.dt[0];
         s.cnt64[CNT_STEP] += 1;
+        s.cnt64[CNT_DT_BITS] = DT_BITS_NONE;  // for the next step's minimum
         // the survivor buckets and the overflow slots become the current buffer
         const long long ovf = s.cnt64[CNT_OVF];
         const long long room = p.capacity - s.cnt64[CNT_WTOT];
@@ -338,10 +330,6 @@ __device__ __forceinline__ Blk member_blk(const int32_t* off, int i) {
     return Blk{(int)blockIdx.x - off[i], off[i + 1] - off[i]};
 }
 
-__global__ void k_reset_b(const __grid_constant__ BatchChunk c) {
-    const int i = member_of(c.off[BCL_RESET], c.n);
-    reset_body(c.mem[i].m, c.mem[i].s, member_blk(c.off[BCL_RESET], i));
-}
 __global__ void k_cell_prep_b(const __grid_constant__ BatchChunk c) {
     const int i = member_of(c.off[BCL_CELLS], c.n);
     cell_prep_body(c.mem[i].m, c.mem[i].s, c.mem[i].p, member_blk(c.off[BCL_CELLS], i));
@@ -350,14 +338,9 @@ __global__ void k_sample_count_b(const __grid_constant__ BatchChunk c) {
     const int i = member_of(c.off[BCL_SCAN], c.n);
     sample_count_body(c.mem[i].m, c.mem[i].s, c.mem[i].p, member_blk(c.off[BCL_SCAN], i));
 }
-// one block per member
-__global__ void k_scan_bsum_b(const __grid_constant__ BatchChunk c) {
-    const BatchMember& e = c.mem[blockIdx.x];
-    scan_bsum_body(e.s, e.p, scan_blocks(e.m.nc));
-}
 __global__ void k_scan_apply_b(const __grid_constant__ BatchChunk c) {
     const int i = member_of(c.off[BCL_SCAN], c.n);
-    scan_apply_body(c.mem[i].m, c.mem[i].s, member_blk(c.off[BCL_SCAN], i));
+    scan_apply_body(c.mem[i].m, c.mem[i].s, c.mem[i].p, member_blk(c.off[BCL_SCAN], i));
 }
 __global__ void k_cell_update_b(const __grid_constant__ BatchChunk c) {
     const int i = member_of(c.off[BCL_CELLS], c.n);
@@ -611,16 +594,12 @@ cudaError_t configure_cell_kernels(int carveout) {
     auto set = [&](auto f) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
     };
-    set(k_reset);
     set(k_cell_prep);
     set(k_sample_count);
-    set(k_scan_bsum);
     set(k_scan_apply);
     set(k_cell_update);
-    set(k_reset_b);
     set(k_cell_prep_b);
     set(k_sample_count_b);
-    set(k_scan_bsum_b);
     set(k_scan_apply_b);
     set(k_cell_update_b);
     set(k_wave_update);
@@ -628,44 +607,37 @@ cudaError_t configure_cell_kernels(int carveout) {
     return e;
 }
 
-void launch_reset(const DevMesh& m, const DevState& s, cudaStream_t st) {
-    k_reset<<<blocks_reset(m.nc), 256, 0, st>>>(m, s);
-}
 void launch_cell_prep(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
-    k_cell_prep<<<cdiv(m.nc, 256), 256, 0, st>>>(m, s, p);
+    k_cell_prep<<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s, p);
 }
 void launch_sample_count(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
     k_sample_count<<<scan_blocks(m.nc), SCAN_BLOCK, 0, st>>>(m, s, p);
 }
 void launch_scan(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
-    k_scan_bsum<<<1, SCAN_SUM_THREADS, 0, st>>>(s, p, scan_blocks(m.nc));
-    k_scan_apply<<<scan_blocks(m.nc), SCAN_BLOCK, 0, st>>>(m, s);
+    k_scan_apply<<<scan_blocks(m.nc), SCAN_BLOCK, 0, st>>>(m, s, p);
 }
 void launch_cell_update(const DevMesh& m, const DevState& s, const DevParams& p, int32_t* wcell, cudaStream_t st) {
-    k_cell_update<<<cdiv(m.nc, 256), 256, 0, st>>>(m, s, p, wcell);
+    k_cell_update<<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s, p, wcell);
 }
 void launch_wave_update(const DevMesh& m, const DevState& s, cudaStream_t st) {
-    k_wave_update<<<cdiv(m.nc, 256), 256, 0, st>>>(m, s);
+    k_wave_update<<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s);
 }
-int blocks_reset(int nc) { return cdiv(5LL * nc, 256) < 4096 ? cdiv(5LL * nc, 256) : 4096; }
-int blocks_cells(int nc) { return cdiv(nc, 256); }
+int blocks_cells(int nc) { return cdiv(nc, CELL_BLOCK); }
 
-void launch_reset_batch(const BatchChunk& c, int blocks, cudaStream_t st) { k_reset_b<<<blocks, 256, 0, st>>>(c); }
 void launch_cell_prep_batch(const BatchChunk& c, int blocks, cudaStream_t st) {
-    k_cell_prep_b<<<blocks, 256, 0, st>>>(c);
+    k_cell_prep_b<<<blocks, CELL_BLOCK, 0, st>>>(c);
 }
 void launch_sample_count_batch(const BatchChunk& c, int blocks, cudaStream_t st) {
     k_sample_count_b<<<blocks, SCAN_BLOCK, 0, st>>>(c);
 }
 void launch_scan_batch(const BatchChunk& c, int blocks, cudaStream_t st) {
-    k_scan_bsum_b<<<c.n, SCAN_SUM_THREADS, 0, st>>>(c);
     k_scan_apply_b<<<blocks, SCAN_BLOCK, 0, st>>>(c);
 }
 void launch_cell_update_batch(const BatchChunk& c, int blocks, cudaStream_t st) {
-    k_cell_update_b<<<blocks, 256, 0, st>>>(c);
+    k_cell_update_b<<<blocks, CELL_BLOCK, 0, st>>>(c);
 }
 void launch_wave_update_batch(const BatchChunk& c, int blocks, cudaStream_t st) {
-    k_wave_update_b<<<blocks, 256, 0, st>>>(c);
+    k_wave_update_b<<<blocks, CELL_BLOCK, 0, st>>>(c);
 }
 void launch_rebuild_survivors(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& a,
                               cudaStream_t st) {

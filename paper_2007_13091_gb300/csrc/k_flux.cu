@@ -356,16 +356,24 @@ __global__ void __launch_bounds__(256) k_face_flux_b(const __grid_constant__ Bat
 
 }  // namespace
 
-static int wave_grid(int n, int blocks) {
-    const int need = (n + UGKWP_WAVE_THREADS - 1) / UGKWP_WAVE_THREADS;
-    return need < blocks ? need : blocks;
+// Block size of a persistent grid of at most `blocks` blocks of `threads`: where
+// n items do not fill one such block per SM, smaller blocks spread them over more
+// SMs, each of which has its own binary64 pipe.
+static int wave_block(long long n, int threads) {
+    const int sms = sm_count();
+    while (threads > 32 && n <= (long long)sms * (threads / 2)) threads /= 2;
+    return threads;
+}
+static int wave_grid(long long n, int threads, int blocks) {
+    const long long need = (n + threads - 1) / threads;
+    return need < blocks ? (int)need : blocks;
 }
 
 // A persistent grid of GRAD_BLOCKS_PER_SM blocks per SM, which leaves room
 // beside it for the first half of the tracking grid.
 void launch_gradients(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
-    const int need = (3 * m.nc + GRAD_THREADS - 1) / GRAD_THREADS, cap = GRAD_BLOCKS_PER_SM * sm_count();
-    k_gradients<<<need < cap ? need : cap, GRAD_THREADS, 0, st>>>(m, s, p);
+    const int t = wave_block(3LL * m.nc, GRAD_THREADS);
+    k_gradients<<<wave_grid(3LL * m.nc, t, GRAD_BLOCKS_PER_SM * sm_count() * (GRAD_THREADS / t)), t, 0, st>>>(m, s, p);
 }
 
 void launch_gp_coef(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
@@ -373,7 +381,8 @@ void launch_gp_coef(const DevMesh& m, const DevState& s, const DevParams& p, cud
 }
 
 void launch_face_flux_o2(const DevMesh& m, const DevState& s, const DevParams& p, int blocks, cudaStream_t st) {
-    k_face_flux_o2<<<wave_grid(m.nf, blocks), UGKWP_WAVE_THREADS, 0, st>>>(m, s, p);
+    const int t = wave_block(m.nf, UGKWP_WAVE_THREADS);
+    k_face_flux_o2<<<wave_grid(m.nf, t, blocks * (UGKWP_WAVE_THREADS / t)), t, 0, st>>>(m, s, p);
 }
 
 int wave_threads() { return UGKWP_WAVE_THREADS; }
@@ -398,8 +407,10 @@ cudaError_t configure_wave_kernels(int carveout) {
 // with the particle kernels launched beside it); 0: one thread per face.
 void launch_face_flux(const DevMesh& m, const DevState& s, const DevParams& p, int first, int blocks,
                       cudaStream_t st) {
-    const int need = (m.nf - first + 255) / 256;
-    k_face_flux<<<blocks > 0 && blocks < need ? blocks : need, 256, 0, st>>>(m, s, p, first);
+    const long long n = m.nf - first;
+    const int t = wave_block(n, 256);
+    const int need = (int)((n + t - 1) / t);
+    k_face_flux<<<blocks > 0 ? wave_grid(n, t, blocks * (256 / t)) : need, t, 0, st>>>(m, s, p, first);
 }
 
 int blocks_gp_coef(int nc) { return (nc + 127) / 128; }

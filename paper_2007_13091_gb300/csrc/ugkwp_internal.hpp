@@ -42,7 +42,7 @@ enum : int {
     CNT_WALL = 8,
     CNT_STEP = 9,       // step index of the next step
     CNT_TRACKED = 10,
-    CNT_DT_BITS = 11,   // min_i |Omega_i| / sum Lambda as ordered bits (positive double)
+    CNT_DT_BITS = 11,   // (between steps: DT_BITS_NONE) min_i |Omega_i| / sum Lambda as ordered bits (positive double)
     CNT_ERR = 12,       // error bits
     CNT_MOVES = 13,     // particle moves since init (never reset by a step)
     CNT_NSAM = 14,      // particles sampled this step (from the scan)
@@ -54,6 +54,9 @@ enum : int {
     CNT_CHECK = 56,     // the first failed self-check: (check << 48) | value
     CNT_SLOTS = 64,
 };
+
+// The time-step minimum's start value: the bits of +inf.
+constexpr int64_t DT_BITS_NONE = 0x7ff0000000000000LL;
 
 // Values of a cell's row in DevState::rec.
 constexpr int REC_N = 24;
@@ -192,7 +195,7 @@ struct DevState {
     double* F;            // [5][nf]
     double* rec;          // [nc][REC_N] order 2: what a face reads of a cell: W (5), rho^h, the limited
                           // gradients of W [3q + d] (15) and of rho^h (3)
-    int2* bsum;           // [n_scan_blocks] block sums of (count, N_sam)
+    int2* bsum;           // [scan_blocks] block sums of (bucket slots, N_sam)
     double* t;            // [1]
     double* dt;           // [1]
     int64_t* cnt64;       // [CNT_SLOTS]
@@ -235,14 +238,16 @@ constexpr int GP_NC = 14;
 constexpr int GP_ATTEMPTS = 64;
 
 // Kernel launchers (stream-ordered, no synchronisation).
-// cells per block of the counting and offset kernels (256: every SM takes
-// blocks on a ~1e5-cell mesh), and threads of the one-block scan of their
-// block sums
-constexpr int SCAN_BLOCK = 256;
-constexpr int SCAN_SUM_THREADS = 1024;
+// Cells per block of the per-cell kernels and of the counting and offset kernels.
+// Most are bound by the binary64 pipe or by the latency of its chains, so that
+// small blocks, which spread a small mesh over all SMs, are faster and cost a large
+// one nothing.  Two steps with 64 / 128 / 256 cells per block: tube of 1,992 tets
+// 59.0 / 63.7 / 70.6 us, 24^3 cavity 1.65 / 1.65 / 1.64 ms; 20 steps of a tube of
+// 9,600 tets in binary64 4.14 / 4.16 / 4.34 ms.
+constexpr int CELL_BLOCK = 64;
+constexpr int SCAN_BLOCK = 64;
 __host__ __device__ inline int scan_blocks(int nc) { return (nc + SCAN_BLOCK - 1) / SCAN_BLOCK; }
 
-void launch_reset(const DevMesh& m, const DevState& s, cudaStream_t st);
 void launch_cell_prep(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
 void launch_sample_count(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
 void launch_scan(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
@@ -311,19 +316,17 @@ void launch_kn_gll(const DevMesh& m, const DevState& s, const DevParams& p, doub
 // body its own launch would run; the particle kernels (sampling,
 // tracking) take every member in turn on the whole grid.
 constexpr int BATCH_CHUNK = 13;
-enum BatchClass { BCL_RESET, BCL_CELLS, BCL_SCAN, BCL_GRAD, BCL_GPC, BCL_FLUX_O2, BCL_FLUX, BCL_N };
+enum BatchClass { BCL_CELLS, BCL_SCAN, BCL_GRAD, BCL_GPC, BCL_FLUX_O2, BCL_FLUX, BCL_N };
 struct BatchChunk {
     int32_t n;
     int32_t off[BCL_N][BATCH_CHUNK + 1];
     BatchMember mem[BATCH_CHUNK];
 };
 static_assert(sizeof(BatchChunk) <= 32764, "a chunk must fit a launch's parameter space");
-int blocks_reset(int nc);        // grid of one simulation's reset launch
-int blocks_cells(int nc);        // one thread per cell, 256 per block
+int blocks_cells(int nc);        // one thread per cell, CELL_BLOCK per block
 int blocks_gp_coef(int nc);      // one thread per cell, 128 per block
 int gradient_threads();          // threads per block of the gradient kernel (one per cell)
 int gradient_blocks_per_sm();    // its persistent grid
-void launch_reset_batch(const BatchChunk& c, int blocks, cudaStream_t st);
 void launch_cell_prep_batch(const BatchChunk& c, int blocks, cudaStream_t st);
 void launch_sample_count_batch(const BatchChunk& c, int blocks, cudaStream_t st);
 void launch_scan_batch(const BatchChunk& c, int blocks, cudaStream_t st);
