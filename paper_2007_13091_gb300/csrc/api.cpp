@@ -165,7 +165,6 @@ void layout(const MeshHost& mh, int64_t cap, size_t rs, bool with_e, Carver& c, 
     S.tau = c.take<double>(nc);
     S.tauf = c.take<float>(nc);
     S.usig = c.take<float4>(nc);
-    S.sig = c.take<double>(nc);
     S.dtc = c.take<double>(nc);
     S.gpc = c.take<double>((size_t)GP_NC * nc);
     S.wsum = c.take<double>(5 * nc);
@@ -833,8 +832,8 @@ int enqueue_step(ugkwp_sim* s) {
         if (gp) CU(cudaStreamWaitEvent(q, s->gp_ready, 0));  // the sampler reads the g_p coefficients
         const bool matched = s->P.sampling == UGKWP_SAMPLE_ENERGY_MATCHED;
         timed(s, UGKWP_K_SAMPLE, matched ? 2 : 1, q, [&] {
-            if (matched) launch_sample_scale(s->M, s->S, s->P, q);
             launch_sample_write(s->M, s->S, s->P, s->A, s->lc.particle_blocks, q);
+            if (matched) launch_sample_scale(s->M, s->S, s->P, s->A, q);
         });
         // tracking in two launches that take tiles from one counter: the first
         // half of the grid starts now and leaves room on each SM for a block
@@ -1785,8 +1784,8 @@ int enqueue_chunk_step(FusedChunk& ch, const std::vector<ugkwp_sim*>& sims) {
     CU(cudaEventRecord(ch.waved, ch.wave));
     launch_scan_batch(c, blocks(BCL_SCAN), q);
     if (gp) CU(cudaStreamWaitEvent(q, ch.gp_ready, 0));
-    if (ch.sampling == UGKWP_SAMPLE_ENERGY_MATCHED) launch_sample_scale_batch(c, blocks(BCL_CELLS), ch.precision, q);
     launch_sample_write_batch(c, lc.particle_blocks, ch.precision, q);
+    if (ch.sampling == UGKWP_SAMPLE_ENERGY_MATCHED) launch_sample_scale_batch(c, blocks(BCL_CELLS), ch.precision, q);
     const int first_half = (lc.particle_blocks + 1) / 2;
     CU(cudaEventRecord(ch.sampled, q));
     launch_track_batch(c, ch.precision, ch.ke, lc.track, first_half, q);

@@ -52,29 +52,28 @@ template <class Real> __device__ __forceinline__ PartView<Real> view(const PartB
 
 // ------------------------------------------------------------------ sampling
 // The three normals X of the pair whose first member has id `ida`: Box-Muller
-// in the particle precision (binary32 in the mixed mode).
+// in the particle precision (binary32 in the mixed mode).  The pair's two members
+// sit in neighbouring lanes (side 0, 1) and each evaluates one of the two
+// Box-Muller pairs of the draw (the fourth normal is not used); every lane of the
+// warp takes part in the exchange.
 template <class Real>
-__device__ __forceinline__ void pair_normals(unsigned long long ida, long long step, unsigned long long seed, Real X[3]) {
+__device__ __forceinline__ void pair_normals(unsigned long long ida, long long step, unsigned long long seed, int side,
+                                             Real X[3]) {
     const dm::U4 r = dm::philox(ida, (unsigned long long)step, TAG_SVEL, 0ULL, seed, 0ULL);
+    const unsigned long long ru = side == 0 ? r.a : r.c, ra = side == 0 ? r.b : r.d;
+    Real rad, sn, cs;
     if constexpr (sizeof(Real) == 4) {
-        float sn, cs;
-        float rad = sqrtf(-2.0f * dm::f_log(dm::u01f(r.a)));
-        dm::f_sincos2pi(dm::u01f(r.b), &sn, &cs);
-        X[0] = rad * cs;
-        X[1] = rad * sn;
-        rad = sqrtf(-2.0f * dm::f_log(dm::u01f(r.c)));
-        dm::f_sincos2pi(dm::u01f(r.d), &sn, &cs);
-        X[2] = rad * cs;
+        rad = sqrtf(-2.0f * dm::f_log(dm::u01f(ru)));
+        dm::f_sincos2pi(dm::u01f(ra), &sn, &cs);
     } else {
-        double sn, cs;
-        double rad = sqrt(-2.0 * dm::d_log(dm::u01d(r.a)));
-        dm::d_sincos2pi(dm::u01d(r.b), &sn, &cs);
-        X[0] = rad * cs;
-        X[1] = rad * sn;
-        rad = sqrt(-2.0 * dm::d_log(dm::u01d(r.c)));
-        dm::d_sincos2pi(dm::u01d(r.d), &sn, &cs);
-        X[2] = rad * cs;
+        rad = sqrt(-2.0 * dm::d_log(dm::u01d(ru)));
+        dm::d_sincos2pi(dm::u01d(ra), &sn, &cs);
     }
+    const Real c = rad * cs, d = rad * sn;
+    const Real oc = __shfl_xor_sync(FULL, c, 1), od = __shfl_xor_sync(FULL, d, 1);
+    X[0] = side == 0 ? c : oc;
+    X[1] = side == 0 ? d : od;
+    X[2] = side == 0 ? oc : c;
 }
 
 // Internal energy of a particle with K internal degrees of freedom at spread
@@ -164,36 +163,6 @@ __device__ __forceinline__ void gp_normals(const double* gpc, int nc, int cell, 
     }
 }
 
-// Energy-matched sampling: one factor per cell, s^2 sum_j |X_j|^2 = 3 N_sam / 2,
-// so the pairs' thermal energy is exactly rho^hp |Omega| (3/2) R T.  The sum
-// runs over the cell's pairs in order in binary64; spread = s sqrt(RT).
-template <class Real>
-__device__ __forceinline__ void sample_scale_body(const DevMesh& m, const DevState& s, const DevParams& p,
-                                                  Blk bk) {
-    const int nc = m.nc;
-    const int cell = bk.id * blockDim.x + threadIdx.x;
-    if (cell >= nc) return;
-    const long long step = s.cnt64[CNT_STEP];
-    const int ns = s.nsam[cell];
-    double sig = sqrt(p.R * s.prim[4 * nc + cell]);
-    if (ns >= 2) {
-        double S = 0.0;
-        for (int j = 0; j < ns / 2; ++j) {
-            Real X[3];
-            pair_normals<Real>(make_id(step, cell, 2 * j), step, p.seed, X);
-            const double x0 = (double)X[0], x1 = (double)X[1], x2 = (double)X[2];
-            S = S + ((x0 * x0 + x1 * x1) + x2 * x2);
-        }
-        if (S > 0.0) sig = sig * sqrt((double)(3 * (ns / 2)) / S);
-    }
-    s.sig[cell] = sig;
-    if constexpr (sizeof(Real) == 4) s.usig[cell].w = (float)sig;
-}
-template <class Real>
-__global__ void __launch_bounds__(256) k_sample_scale(DevMesh m, DevState s, DevParams p) {
-    sample_scale_body<Real>(m, s, p, Blk{(int)blockIdx.x, (int)gridDim.x});
-}
-
 // a5 positions: a uniform point in the tet from three uniforms folded cube ->
 // prism -> tet (Rocchini & Cignoni, J. Graphics Tools 5(4), 2000).  The
 // uniforms are odd multiples of 2^-48 (47 bits of one Philox draw each) and
@@ -248,16 +217,28 @@ __device__ __forceinline__ float ff_position(const float* f, int nc, const float
     return s3 + lo;
 }
 
+// One lane per sample; cells sample even numbers, so that the two members of a
+// pair are lanes 2i and 2i + 1 and share the work of their normals (first-order
+// g_p: each particle on its own).  With energy-matched sampling a pair's
+// velocities hold its normals X until k_sample_scale has the cell's factor.  Bound
+// by the binary64 pipe in binary64 (logarithms, square roots, sines and cosines),
+// by the integer pipes (Philox4x64) in mixed mode.  20 binary64 steps of a tube of
+// 9,600 tets, energy-matched: 2.94 ms; with both members evaluating all of the
+// pair's normals, and the scale kernel all of them once more, 4.13 ms.
 template <class Real>
 __device__ __forceinline__ void sample_write_body(const DevMesh& m, const DevState& s, const DevParams& p,
                                                   const PartBufRaw& br, Blk bk) {
-    if (s.cnt64[CNT_ERR] & ERRB_CAPACITY) return;
+    if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
     const PartView<Real> b = view<Real>(br);
-    const int nc = m.nc;
+    const int nc = m.nc, lane = threadIdx.x & 31;
     const long long total = s.cnt64[CNT_NSAM];
     const long long step = s.cnt64[CNT_STEP];
+    const long long n_a = s.cnt64[CNT_N_A];
     const long long stride = (long long)bk.n * blockDim.x;
-    for (long long g = (long long)bk.id * blockDim.x + threadIdx.x; g < total; g += stride) {
+    const bool gp = p.sampling == UGKWP_SAMPLE_GP1, matched = p.sampling == UGKWP_SAMPLE_ENERGY_MATCHED;
+    // warp-uniform bounds: every lane takes part in the exchange of normals
+    for (long long base = (long long)bk.id * blockDim.x + (threadIdx.x & ~31); base < total; base += stride) {
+        const long long g = min(base + lane, total - 1);  // (a lane past the end repeats the last sample)
         // owning cell: the last c with soff[c] <= g (cells with N_sam = 0 share
         // the offset of the next cell and are never the last such c)
         int lo = 0, hi = nc;  // invariant: soff[lo] <= g < soff[hi] (soff[nc] = +inf)
@@ -267,46 +248,42 @@ __device__ __forceinline__ void sample_write_body(const DevMesh& m, const DevSta
         }
         const int cell = lo;
         const int k = (int)(g - s.soff[cell]);
-        const int side = k & 1;
+        const int side = lane & 1;  // = k & 1 for g < total
+        const unsigned long long ida = make_id(step, cell, k & ~1);
+        const unsigned long long id = ida + (unsigned long long)side;
+        Real X[3];
+        if (!gp) pair_normals<Real>(ida, step, p.seed, side, X);
         // the samples follow the current buffer's survivor slots, in cell order
-        const long long j = s.cnt64[CNT_N_A] + g;
+        const long long j = n_a + g;
+        if (base + lane >= total) continue;
         if (j >= p.capacity || cell < 0 || cell >= nc) {
             check_failed(s, 9, (unsigned long long)j);
             continue;
         }
-        const unsigned long long ida = make_id(step, cell, k - side);
-        const unsigned long long id = ida + (unsigned long long)side;
-        const bool gp = p.sampling == UGKWP_SAMPLE_GP1;
+        if (gp) gp_normals<Real>(s.gpc, nc, cell, id, step, p.seed, X);  // every particle on its own
+        Real U[3], sig;
+        if constexpr (sizeof(Real) == 4) {
+            // mixed mode: velocities in binary32 from U and the spread rounded to binary32
+            const float4 us = s.usig[cell];
+            U[0] = us.x; U[1] = us.y; U[2] = us.z;
+            sig = us.w;
+        } else {
+            for (int c = 0; c < 3; ++c) U[c] = s.prim[(size_t)(1 + c) * nc + cell];
+            sig = sqrt(p.R * s.prim[(size_t)4 * nc + cell]);
+        }
         long long N[3];
         tet_weights(dm::philox(id, (unsigned long long)step, TAG_SPOS, 0ULL, p.seed, 0ULL), N);
         if constexpr (sizeof(Real) == 4) {
-            // mixed mode: velocities in binary32 from U and the spread rounded
-            // to binary32; the position offset from the tet's anchor in
-            // binary32 pairs, rounded once
-            const float4 us = s.usig[cell];
-            float X[3];
-            if (gp) gp_normals<float>(s.gpc, nc, cell, id, step, p.seed, X);  // every particle on its own
-            else pair_normals<float>(ida, step, p.seed, X);
+            // the position offset from the tet's anchor in binary32 pairs, rounded once
             float wh[3], wl[3];
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 wh[q] = (float)(N[q] >> 24) * 0x1p-24f;
                 wl[q] = (float)(N[q] & 0xffffffLL) * 0x1p-48f;
             }
-            const float U[3] = {us.x, us.y, us.z};
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                b.x[c][j] = ff_position(m.smp_f + (size_t)(8 * c) * nc + cell, nc, wh, wl);
-                b.u[c][j] = (gp || side == 0) ? U[c] + us.w * X[c] : U[c] - us.w * X[c];
-            }
-            if (p.K > 0) b.e[j] = internal_energy<float>(id, step, TAG_SINT, 0ULL, p.K, us.w, p.seed);
+            for (int c = 0; c < 3; ++c) b.x[c][j] = ff_position(m.smp_f + (size_t)(8 * c) * nc + cell, nc, wh, wl);
         } else {
-            const double U[3] = {s.prim[nc + cell], s.prim[2 * nc + cell], s.prim[3 * nc + cell]};
-            const double sig =
-                p.sampling == UGKWP_SAMPLE_ENERGY_MATCHED ? s.sig[cell] : sqrt(p.R * s.prim[4 * nc + cell]);
-            double X[3];
-            if (gp) gp_normals<double>(s.gpc, nc, cell, id, step, p.seed, X);
-            else pair_normals<double>(ida, step, p.seed, X);
             const double a = (double)N[0] * 0x1p-48, bb = (double)N[1] * 0x1p-48, cc = (double)N[2] * 0x1p-48;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -315,10 +292,14 @@ __device__ __forceinline__ void sample_write_body(const DevMesh& m, const DevSta
                 const double E2 = m.vtx[(size_t)(6 + c) * nc + cell] - P0;
                 const double E3 = m.vtx[(size_t)(9 + c) * nc + cell] - P0;
                 b.x[c][j] = P0 + ((a * E1 + bb * E2) + cc * E3);
-                b.u[c][j] = (gp || side == 0) ? U[c] + sig * X[c] : U[c] - sig * X[c];
             }
-            if (p.K > 0) b.e[j] = internal_energy<double>(id, step, TAG_SINT, 0ULL, p.K, sig, p.seed);
         }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            if (matched) b.u[c][j] = X[c];
+            else b.u[c][j] = (gp || side == 0) ? U[c] + sig * X[c] : U[c] - sig * X[c];
+        }
+        if (p.K > 0) b.e[j] = internal_energy<Real>(id, step, TAG_SINT, 0ULL, p.K, sig, p.seed);
         b.m[j] = s.msam[cell];
         b.cell[j] = cell;
         b.id[j] = id;
@@ -327,6 +308,71 @@ __device__ __forceinline__ void sample_write_body(const DevMesh& m, const DevSta
 template <class Real>
 __global__ void __launch_bounds__(256) k_sample_write(DevMesh m, DevState s, DevParams p, PartBufRaw br) {
     sample_write_body<Real>(m, s, p, br, Blk{(int)blockIdx.x, (int)gridDim.x});
+}
+
+// Energy-matched sampling: one factor per cell, s^2 sum_j |X_j|^2 = 3 N_sam / 2,
+// so the pairs' thermal energy is exactly rho^hp |Omega| (3/2) R T.  The sum
+// runs over the cell's pairs in order in binary64; the velocities are
+// U +- s sqrt(RT) X.  A block takes CELL_BLOCK cells: a thread sums its cell's
+// normals, which k_sample_write left in the velocities, then the block goes over
+// its cells' samples, which lie in a row.
+template <class Real>
+__device__ __forceinline__ void sample_scale_body(const DevMesh& m, const DevState& s, const DevParams& p,
+                                                  const PartBufRaw& br, Blk bk) {
+    __shared__ int off[CELL_BLOCK + 1];
+    __shared__ Real spread[CELL_BLOCK];
+    if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
+    const PartView<Real> b = view<Real>(br);
+    const int nc = m.nc, t = threadIdx.x, cell = bk.id * CELL_BLOCK + t;
+    const long long n_a = s.cnt64[CNT_N_A];
+    int ns = 0, so = 0;
+    if (cell < nc) {
+        ns = s.nsam[cell];
+        so = s.soff[cell];
+        double sig = sqrt(p.R * s.prim[(size_t)4 * nc + cell]);
+        if (ns >= 2) {
+            double S = 0.0;
+            for (int j = 0; j < ns / 2; ++j) {
+                const long long at = n_a + so + 2 * j;
+                const double x0 = (double)b.u[0][at], x1 = (double)b.u[1][at], x2 = (double)b.u[2][at];
+                S = S + ((x0 * x0 + x1 * x1) + x2 * x2);
+            }
+            if (S > 0.0) sig = sig * sqrt((double)(3 * (ns / 2)) / S);
+        }
+        spread[t] = (Real)sig;
+    }
+    const int last = min(CELL_BLOCK, nc - bk.id * CELL_BLOCK) - 1;
+    off[t] = so;
+    __syncthreads();
+    if (t == last) off[last + 1] = so + ns;
+    __syncthreads();
+    const int first = off[0], end = off[last + 1];
+    for (int g = first + t; g < end; g += CELL_BLOCK) {
+        int lo = 0, hi = last + 1;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (off[mid] <= g) lo = mid; else hi = mid;
+        }
+        const int c0 = bk.id * CELL_BLOCK + lo;
+        const Real sg = spread[lo];
+        Real U[3];
+        if constexpr (sizeof(Real) == 4) {
+            const float4 us = s.usig[c0];
+            U[0] = us.x; U[1] = us.y; U[2] = us.z;
+        } else {
+            for (int c = 0; c < 3; ++c) U[c] = s.prim[(size_t)(1 + c) * nc + c0];
+        }
+        const long long j = n_a + g;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const Real X = b.u[c][j];
+            b.u[c][j] = ((g - off[lo]) & 1) == 0 ? U[c] + sg * X : U[c] - sg * X;
+        }
+    }
+}
+template <class Real>
+__global__ void __launch_bounds__(CELL_BLOCK) k_sample_scale(DevMesh m, DevState s, DevParams p, PartBufRaw br) {
+    sample_scale_body<Real>(m, s, p, br, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // ------------------------------------------------------------------ tracking
@@ -956,10 +1002,10 @@ __device__ __forceinline__ int member_of(const int32_t* off, int n) {
     return lo;
 }
 template <class Real>
-__global__ void __launch_bounds__(256) k_sample_scale_b(const __grid_constant__ BatchChunk c) {
+__global__ void __launch_bounds__(CELL_BLOCK) k_sample_scale_b(const __grid_constant__ BatchChunk c) {
     const int32_t* off = c.off[BCL_CELLS];
     const int i = member_of(off, c.n);
-    sample_scale_body<Real>(c.mem[i].m, c.mem[i].s, c.mem[i].p, Blk{(int)blockIdx.x - off[i], off[i + 1] - off[i]});
+    sample_scale_body<Real>(c.mem[i].m, c.mem[i].s, c.mem[i].p, c.mem[i].a, Blk{(int)blockIdx.x - off[i], off[i + 1] - off[i]});
 }
 // The particle kernels take every member of the chunk in turn on the whole grid.
 template <class Real>
@@ -986,9 +1032,9 @@ void launch_sample_write(const DevMesh& m, const DevState& s, const DevParams& p
     else k_sample_write<double><<<blocks, 256, 0, st>>>(m, s, p, b);
 }
 
-void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
-    if (p.precision == UGKWP_MIXED) k_sample_scale<float><<<(m.nc + 255) / 256, 256, 0, st>>>(m, s, p);
-    else k_sample_scale<double><<<(m.nc + 255) / 256, 256, 0, st>>>(m, s, p);
+void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b, cudaStream_t st) {
+    if (p.precision == UGKWP_MIXED) k_sample_scale<float><<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s, p, b);
+    else k_sample_scale<double><<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s, p, b);
 }
 
 namespace {
@@ -1036,8 +1082,8 @@ cudaError_t configure_particle_kernels(const DevParams& p, int carveout) {
 }
 
 void launch_sample_scale_batch(const BatchChunk& c, int blocks, int precision, cudaStream_t st) {
-    if (precision == UGKWP_MIXED) k_sample_scale_b<float><<<blocks, 256, 0, st>>>(c);
-    else k_sample_scale_b<double><<<blocks, 256, 0, st>>>(c);
+    if (precision == UGKWP_MIXED) k_sample_scale_b<float><<<blocks, CELL_BLOCK, 0, st>>>(c);
+    else k_sample_scale_b<double><<<blocks, CELL_BLOCK, 0, st>>>(c);
 }
 void launch_sample_write_batch(const BatchChunk& c, int blocks, int precision, cudaStream_t st) {
     if (precision == UGKWP_MIXED) k_sample_write_b<float><<<blocks, 256, 0, st>>>(c);

@@ -167,7 +167,6 @@ struct DevState {
     double* tau;          // [nc]
     float* tauf;          // [nc] binary32 rounding of tau (MIXED t_f draw)
     float4* usig;         // [nc] binary32 roundings of U and the sampling spread (MIXED sampling)
-    double* sig;          // [nc] sampling spread s sqrt(RT) of energy-matched sampling
     double* dtc;          // [nc] local time step CFL |Omega| / sum_d Lambda^d (GKS step, local steps)
     double* gpc;          // [GP_NC][nc] first-order g_p: acceptance polynomial and bound per cell
     double* wsum;         // [5][nc] time-average sums of dt^n W^n
@@ -266,8 +265,8 @@ struct LaunchCfg {
 
 void launch_sample_write(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b,
                          int blocks, cudaStream_t st);
-// Energy-matched sampling: the per-cell spread s sqrt(RT) (sig, usig.w).
-void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
+// Energy-matched sampling, after launch_sample_write: the samples' velocities.
+void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b, cudaStream_t st);
 // Tracking of buffer b (survivors, then this step's samples): the survivors go
 // into their end cells' buckets in nxt, the counting flux into pflux.
 void launch_track(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b,
