@@ -53,7 +53,7 @@ __device__ __forceinline__ void cell_prep_body(const DevMesh& m, const DevState&
         // the sums this step's tracking adds to
 #pragma unroll
         for (int q = 0; q < 5; ++q) s.pflux[(size_t)q * nc + i] = 0;
-        s.nleft_next[i] = 0;
+        s.fill[i] = 0;
         const double rho = s.W[i];
         const double Ux = s.W[nc + i] / rho, Uy = s.W[2 * nc + i] / rho, Uz = s.W[3 * nc + i] / rho;
         const double U2 = (Ux * Ux + Uy * Uy) + Uz * Uz;
@@ -152,7 +152,7 @@ __device__ __forceinline__ void sample_count_body(const DevMesh& m, const DevSta
         s.msam[i] = ms;
         nsam = (int)ns;
         const int count = s.nleft[i] + nsam;
-        s.cnt[i] = count;
+        s.nleft_next[i] = count;
         wcap = bucket_slots(count);
         s.wcap[i] = wcap;
     }
@@ -209,6 +209,14 @@ __device__ __forceinline__ void scan_apply_body(const DevMesh& m, const DevState
         s.cnt64[CNT_NSAM] = fits ? nsam : 0;
         s.cnt64[CNT_SAMPLED] = nsam;
         s.cnt64[CNT_WTOT] = wtot;
+        const long long live = s.cnt64[CNT_SURV] + nsam, cur = s.cnt64[CNT_CUR], age = s.cnt64[CNT_AGE] + 1;
+        // (past the capacity nothing is written and no particle is left)
+        const bool in_place = p.in_place && (!fits || (age < RESORT && total + 4 * nsam + 4LL * m.nc <= p.capacity &&
+                                        8 * nsam <= live && 4 * (total - live) <= live));
+        s.cnt64[CNT_SRC] = cur;
+        s.cnt64[CNT_IN_PLACE] = in_place ? 1 : 0;
+        s.cnt64[CNT_CUR] = in_place ? cur : 1 - cur;
+        s.cnt64[CNT_AGE] = in_place ? age : 0;
         s.cnt64[CNT_COLLIDED] = 0;
         s.cnt64[CNT_EXITED] = 0;
         s.cnt64[CNT_LOST] = 0;
@@ -227,7 +235,7 @@ __global__ void k_scan_apply(DevMesh m, DevState s, DevParams p) {
 
 // a10: W^{n+1} = W^n - 1/|Omega| sum_k (+-F_k |S_k|) + F^{fr,p}/|Omega|, faces
 // gathered in local order 0..3 (Eq. update_macro_variables).
-__device__ __forceinline__ void cell_update_body(const DevMesh& m, const DevState& s, const DevParams& p, int32_t* wcell, Blk bk) {
+__device__ __forceinline__ void cell_update_body(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& bufs, Blk bk) {
     const int nc = m.nc, nf = m.nf;
     const int i = bk.id * blockDim.x + threadIdx.x;
     if (p.gks) {
@@ -257,15 +265,19 @@ __device__ __forceinline__ void cell_update_body(const DevMesh& m, const DevStat
         if (p.averaging) s.tsum[0] += s.dt[0];
         s.cnt64[CNT_STEP] += 1;
         s.cnt64[CNT_DT_BITS] = DT_BITS_NONE;  // for the next step's minimum
-        // the survivor buckets and the overflow slots become the current buffer
+        // sorted: the survivor buckets and the overflow slots; in place: every slot
         const long long ovf = s.cnt64[CNT_OVF];
         const long long room = p.capacity - s.cnt64[CNT_WTOT];
-        s.cnt64[CNT_N_A] = s.cnt64[CNT_WTOT] + (ovf < room ? ovf : room);
+        s.cnt64[CNT_N_A] =
+            s.cnt64[CNT_IN_PLACE] ? s.cnt64[CNT_N_B] : s.cnt64[CNT_WTOT] + (ovf < room ? ovf : room);
     }
     if (i >= nc) return;
     // a11: the bucket slots no survivor took are holes
-    if (!(s.cnt64[CNT_ERR] & ERRB_CAPACITY)) {
-        const int cap = s.wcap[i], fill = s.nleft_next[i];
+    if (!s.cnt64[CNT_IN_PLACE] && !(s.cnt64[CNT_ERR] & ERRB_CAPACITY)) {
+        int32_t* wcell =
+            reinterpret_cast<int32_t*>(reinterpret_cast<char*>(bufs.b0.cell) + (bufs.dyn ? s.cnt64[CNT_CUR] : 1) * bufs.delta);
+        const int cap = s.wcap[i], fill = s.fill[i];
+        s.nleft_next[i] = fill;  // the bucket's survivors, those in overflow slots included
         if ((long long)s.woff[i] + cap <= p.capacity)
             for (int k = fill < cap ? fill : cap; k < cap; ++k) wcell[(size_t)s.woff[i] + k] = -1;
     }
@@ -311,8 +323,8 @@ __device__ __forceinline__ void wave_update_body(const DevMesh& m, const DevStat
 __global__ void k_wave_update(DevMesh m, DevState s) {
     wave_update_body(m, s, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
-__global__ void k_cell_update(DevMesh m, DevState s, DevParams p, int32_t* wcell) {
-    cell_update_body(m, s, p, wcell, Blk{(int)blockIdx.x, (int)gridDim.x});
+__global__ void k_cell_update(DevMesh m, DevState s, DevParams p, PartBufs bufs) {
+    cell_update_body(m, s, p, bufs, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // ---- fused batches: member i of the chunk runs on the blocks
@@ -344,7 +356,7 @@ __global__ void k_scan_apply_b(const __grid_constant__ BatchChunk c) {
 }
 __global__ void k_cell_update_b(const __grid_constant__ BatchChunk c) {
     const int i = member_of(c.off[BCL_CELLS], c.n);
-    cell_update_body(c.mem[i].m, c.mem[i].s, c.mem[i].p, c.mem[i].b.cell, member_blk(c.off[BCL_CELLS], i));
+    cell_update_body(c.mem[i].m, c.mem[i].s, c.mem[i].p, c.mem[i].bufs, member_blk(c.off[BCL_CELLS], i));
 }
 __global__ void k_wave_update_b(const __grid_constant__ BatchChunk c) {
     const int i = member_of(c.off[BCL_CELLS], c.n);
@@ -474,7 +486,15 @@ __global__ void k_import(int nc, long long n, const double* anc, const double* x
 // widening and the conversion to fixed point run on the integer pipes.  7.97e6
 // particles: 0.185 ms (one thread and five atomics per particle: 0.44 ms).
 template <class Real>
-__global__ void __launch_bounds__(256) k_wp_acc(DevMesh m, DevState s, DevParams p, PartBufRaw a) {
+__global__ void __launch_bounds__(256) k_wp_acc(DevMesh m, DevState s, DevParams p, PartBufs bufs) {
+    PartBufRaw a = bufs.b0;  // the buffer that holds the particles
+    {
+        const long long d = bufs.dyn ? s.cnt64[CNT_CUR] * bufs.delta : 0;
+        for (int k = 0; k < 3; ++k) a.u[k] = static_cast<char*>(a.u[k]) + d;
+        a.m = reinterpret_cast<double*>(reinterpret_cast<char*>(a.m) + d);
+        a.cell = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(a.cell) + d);
+        if (a.e) a.e = static_cast<char*>(a.e) + d;
+    }
     const unsigned n = (unsigned)s.cnt64[CNT_N_A];
     const int nc = m.nc, lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
@@ -616,8 +636,8 @@ void launch_sample_count(const DevMesh& m, const DevState& s, const DevParams& p
 void launch_scan(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
     k_scan_apply<<<scan_blocks(m.nc), SCAN_BLOCK, 0, st>>>(m, s, p);
 }
-void launch_cell_update(const DevMesh& m, const DevState& s, const DevParams& p, int32_t* wcell, cudaStream_t st) {
-    k_cell_update<<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s, p, wcell);
+void launch_cell_update(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, cudaStream_t st) {
+    k_cell_update<<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s, p, b);
 }
 void launch_wave_update(const DevMesh& m, const DevState& s, cudaStream_t st) {
     k_wave_update<<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s);
@@ -652,12 +672,10 @@ void launch_import(int nc, long long n, bool mixed, bool convert, const double* 
     else if (mixed) k_import<float, false><<<particle_grid(), 256, 0, st>>>(nc, n, anc, xs, us, es, b, err);
     else k_import<double, false><<<particle_grid(), 256, 0, st>>>(nc, n, anc, xs, us, es, b, err);
 }
-void launch_wp_moments(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& a,
-                       double* out, cudaStream_t st) {
+void launch_wp_moments(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, cudaStream_t st) {
     k_zero_wacc<<<cdiv(5LL * m.nc, 256), 256, 0, st>>>(m, s);
-    if (p.precision == UGKWP_MIXED) k_wp_acc<float><<<particle_grid(), 256, 0, st>>>(m, s, p, a);
-    else k_wp_acc<double><<<particle_grid(), 256, 0, st>>>(m, s, p, a);
-    (void)out;
+    if (p.precision == UGKWP_MIXED) k_wp_acc<float><<<particle_grid(), 256, 0, st>>>(m, s, p, b);
+    else k_wp_acc<double><<<particle_grid(), 256, 0, st>>>(m, s, p, b);
 }
 void launch_wbar(const DevMesh& m, const DevState& s, double* out, cudaStream_t st) {
     k_wbar<<<cdiv(5LL * m.nc, 256) < 4096 ? cdiv(5LL * m.nc, 256) : 4096, 256, 0, st>>>(m, s, out);

@@ -9,6 +9,8 @@
 //                   counting flux of the particles that left their cell or met a
 //                   wall, removal; each survivor is written into the bucket of
 //                   its end cell in the next buffer.
+#include <type_traits>
+
 #include "dmath.cuh"
 #include "fixed.cuh"
 #include "ugkwp_internal.hpp"
@@ -37,16 +39,18 @@ __device__ __forceinline__ unsigned long long make_id(long long step, int cell, 
     return ((unsigned long long)step << 40) | ((unsigned long long)cell << 16) | (unsigned long long)k;
 }
 
-template <class Real> __device__ __forceinline__ PartView<Real> view(const PartBufRaw& r) {
+// The arrays of buffer 0 shifted by `d` bytes (0 or the distance to buffer 1).
+template <class Real> __device__ __forceinline__ PartView<Real> view(const PartBufRaw& r, long long d) {
+    auto at = [d](void* q) { return static_cast<void*>(static_cast<char*>(q) + d); };
     PartView<Real> v;
     for (int c = 0; c < 3; ++c) {
-        v.x[c] = (Real*)r.x[c];
-        v.u[c] = (Real*)r.u[c];
+        v.x[c] = (Real*)at(r.x[c]);
+        v.u[c] = (Real*)at(r.u[c]);
     }
-    v.m = r.m;
-    v.cell = r.cell;
-    v.id = r.id;
-    v.e = (Real*)r.e;
+    v.m = (double*)at(r.m);
+    v.cell = (int32_t*)at(r.cell);
+    v.id = (uint64_t*)at(r.id);
+    v.e = r.e ? (Real*)at(r.e) : nullptr;
     return v;
 }
 
@@ -227,9 +231,9 @@ __device__ __forceinline__ float ff_position(const float* f, int nc, const float
 // pair's normals, and the scale kernel all of them once more, 4.13 ms.
 template <class Real>
 __device__ __forceinline__ void sample_write_body(const DevMesh& m, const DevState& s, const DevParams& p,
-                                                  const PartBufRaw& br, Blk bk) {
+                                                  const PartBufs& bufs, Blk bk) {
     if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
-    const PartView<Real> b = view<Real>(br);
+    const PartView<Real> b = view<Real>(bufs.b0, bufs.dyn ? s.cnt64[CNT_SRC] * bufs.delta : 0);
     const int nc = m.nc, lane = threadIdx.x & 31;
     const long long total = s.cnt64[CNT_NSAM];
     const long long step = s.cnt64[CNT_STEP];
@@ -306,8 +310,8 @@ __device__ __forceinline__ void sample_write_body(const DevMesh& m, const DevSta
     }
 }
 template <class Real>
-__global__ void __launch_bounds__(256) k_sample_write(DevMesh m, DevState s, DevParams p, PartBufRaw br) {
-    sample_write_body<Real>(m, s, p, br, Blk{(int)blockIdx.x, (int)gridDim.x});
+__global__ void __launch_bounds__(256) k_sample_write(DevMesh m, DevState s, DevParams p, PartBufs bufs) {
+    sample_write_body<Real>(m, s, p, bufs, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // Energy-matched sampling: one factor per cell, s^2 sum_j |X_j|^2 = 3 N_sam / 2,
@@ -318,11 +322,11 @@ __global__ void __launch_bounds__(256) k_sample_write(DevMesh m, DevState s, Dev
 // its cells' samples, which lie in a row.
 template <class Real>
 __device__ __forceinline__ void sample_scale_body(const DevMesh& m, const DevState& s, const DevParams& p,
-                                                  const PartBufRaw& br, Blk bk) {
+                                                  const PartBufs& bufs, Blk bk) {
     __shared__ int off[CELL_BLOCK + 1];
     __shared__ Real spread[CELL_BLOCK];
     if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
-    const PartView<Real> b = view<Real>(br);
+    const PartView<Real> b = view<Real>(bufs.b0, bufs.dyn ? s.cnt64[CNT_SRC] * bufs.delta : 0);
     const int nc = m.nc, t = threadIdx.x, cell = bk.id * CELL_BLOCK + t;
     const long long n_a = s.cnt64[CNT_N_A];
     int ns = 0, so = 0;
@@ -371,8 +375,8 @@ __device__ __forceinline__ void sample_scale_body(const DevMesh& m, const DevSta
     }
 }
 template <class Real>
-__global__ void __launch_bounds__(CELL_BLOCK) k_sample_scale(DevMesh m, DevState s, DevParams p, PartBufRaw br) {
-    sample_scale_body<Real>(m, s, p, br, Blk{(int)blockIdx.x, (int)gridDim.x});
+__global__ void __launch_bounds__(CELL_BLOCK) k_sample_scale(DevMesh m, DevState s, DevParams p, PartBufs bufs) {
+    sample_scale_body<Real>(m, s, p, bufs, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // ------------------------------------------------------------------ tracking
@@ -670,17 +674,26 @@ template <class Real> __device__ __forceinline__ const float4* test_planes(const
 // rounds and a mover list for a flux kernel of its own 2.20 and 7.33 ms, with
 // every exit face decided in binary64 and no prefetch of the next tile's lines
 // 1.78 and 2.99 ms.
-template <class Real, bool KE, int THREADS>
-__device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, const DevParams& p,
-                                           const PartBufRaw& br, const PartBufRaw& nr) {
+//
+// IN_PLACE (k_scan_apply chooses per step): a particle keeps its slot, a stayer
+// writes its position only, a removed one leaves a hole.  Otherwise each survivor
+// is written into the bucket of its end cell in the other buffer.
+template <class Real, int THREADS> struct TrackShared {
+    int q_slot[THREADS / 32][WALK_QUEUE];
+    Real q_end[THREADS / 32][WALK_QUEUE];  // t_f, or dt; -1: not drawn yet
+    unsigned red[THREADS / 32][8];
+};
+template <class Real, bool KE, int THREADS, bool IN_PLACE>
+__device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& bufs,
+                                           long long src, TrackShared<Real, THREADS>& sh) {
     constexpr int NW = THREADS / 32;
-    // (block-uniform: another block may set the bit while this one starts)
-    if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
-    __shared__ int q_slot[NW][WALK_QUEUE];
-    __shared__ Real q_end[NW][WALK_QUEUE];  // t_f, or dt; -1: not drawn yet
-    __shared__ unsigned sh_red[NW][8];
-    const PartView<Real> b = view<Real>(br);    // this step's particles, sorted by cell (holes: cell -1)
-    const PartView<Real> nxt = view<Real>(nr);  // the next step's survivors, in their end cells' buckets
+    auto& q_slot = sh.q_slot;
+    auto& q_end = sh.q_end;
+    auto& sh_red = sh.red;
+    const PartBufRaw& br = bufs.b0;
+    const PartView<Real> b = view<Real>(br, src);                 // this step's particles (holes: cell -1)
+    // sorting: the next step's (src is 0 or delta; without DYN always 0)
+    const PartView<Real> nxt = view<Real>(br, bufs.delta - src);
     const unsigned n = (unsigned)s.cnt64[CNT_N_B];
     const long long step = s.cnt64[CNT_STEP];
     const long long wtot = s.cnt64[CNT_WTOT];  // overflow slots start after the buckets
@@ -726,14 +739,14 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
         Walk<Real> w;
         Real us[3] = {(Real)0, (Real)0, (Real)0}, xe[3] = {(Real)0, (Real)0, (Real)0}, es = (Real)0, ee = (Real)0;
         double mm = 0.0;
-        int c0 = -1;
+        int c0 = -1, i = 0;
         unsigned long long id = 0;
         bool survivor = false, mover = false, exited = false;
         w.tet = -1;
         w.u[0] = w.u[1] = w.u[2] = (Real)0;
         w.nrefl = 0;
         if (act) {
-            const int i = q_slot[warp][k];
+            i = q_slot[warp][k];
             w.t_end = q_end[warp][k];
             c0 = b.cell[i];
             id = b.id[i];
@@ -798,15 +811,36 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
         // survivors' mass: out of the start cell, into the end cell
         const bool stays = survivor && w.tet == c0;
         if (act && !mover && !stays && !fixed_of_mass(mm, p.exps[0], q0[0])) set_err(s, ERRB_FIXED_OVERFLOW);
-        if (act && !stays) atomicAdd(&smass[c0], (unsigned long long)(-q0[0]));
-        if (survivor && !stays) atomicAdd(&smass[w.tet], (unsigned long long)q0[0]);
+        if (act && !stays) {
+            atomicAdd(&smass[c0], (unsigned long long)(-q0[0]));
+            if constexpr (IN_PLACE) atomicAdd(&s.nleft_next[c0], -1);
+        }
+        if (survivor && !stays) {
+            atomicAdd(&smass[w.tet], (unsigned long long)q0[0]);
+            if constexpr (IN_PLACE) atomicAdd(&s.nleft_next[w.tet], 1);
+        }
+        c_surv += __popc(__ballot_sync(FULL, survivor));
+        if constexpr (IN_PLACE) {
+            if (act) {
+                if (!stays) b.cell[i] = survivor ? w.tet : -1;
+                if (survivor) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) b.x[c][i] = xe[c];
+                    if (w.nrefl > 0) {
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) b.u[c][i] = w.u[c];
+                        if constexpr (KE) b.e[i] = ee;
+                    }
+                }
+            }
+            return;
+        }
         // a11: lanes with the same end cell take consecutive places of its bucket
         const int key = survivor ? w.tet : -1;
         const unsigned peers = __match_any_sync(FULL, key);
         const int leader = __ffs(peers) - 1;
         int first = 0;
-        if (lane == leader && key >= 0) first = atomicAdd(&s.nleft_next[key], __popc(peers));
-        c_surv += __popc(__ballot_sync(FULL, survivor));
+        if (lane == leader && key >= 0) first = atomicAdd(&s.fill[key], __popc(peers));
         first = __shfl_sync(FULL, first, leader);
         if (survivor) {
             const int j = slot_of(first + __popc(peers & lt), s.woff[key], s.wcap[key]);
@@ -840,13 +874,13 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
     unsigned pstr = 0;
     if (lane < 6 * XL) {
         const int a = lane / XL;
-        pptr = reinterpret_cast<const char*>(a < 3 ? br.x[a] : br.u[a - 3]) + (lane % XL) * 128;
+        pptr = reinterpret_cast<const char*>(a < 3 ? br.x[a] : br.u[a - 3]) + src + (lane % XL) * 128;
         pstr = sizeof(Real);
-    } else if (lane < 6 * XL + 2) {
-        pptr = reinterpret_cast<const char*>(br.m) + (lane - 6 * XL) * 128;
+    } else if (!IN_PLACE && lane < 6 * XL + 2) {
+        pptr = reinterpret_cast<const char*>(br.m) + src + (lane - 6 * XL) * 128;
         pstr = 8;
-    } else if (lane < 6 * XL + 4) {
-        pptr = reinterpret_cast<const char*>(br.id) + (lane - 6 * XL - 2) * 128;
+    } else if (lane >= 6 * XL + 2 && lane < 6 * XL + 4) {
+        pptr = reinterpret_cast<const char*>(br.id) + src + (lane - 6 * XL - 2) * 128;
         pstr = 8;
     }
     int cell_i = -1;
@@ -864,9 +898,12 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
             x0[c] = b.x[c][i];
             u[c] = b.u[c][i];
         }
-        const double mm = b.m[i];
+        double mm = 0.0;
         Real es = (Real)0;
-        if constexpr (KE) es = b.e[i];
+        if constexpr (!IN_PLACE) {
+            mm = b.m[i];
+            if constexpr (KE) es = b.e[i];
+        }
         const int cc = valid ? c0 : 0;
         const int4 info = s.cinfo[cc];
         const float4* pl = test_planes<Real>(m, cc);
@@ -919,16 +956,19 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
         inside = inside && !defer;
         const bool slow = valid && !inside;
         const bool surv = valid && inside && !coll, gone = valid && inside && coll;
-        // runs of equal cells
-        const int prev = __shfl_up_sync(FULL, c0, 1);
-        const unsigned heads = __ballot_sync(FULL, lane == 0 || prev != c0);
-        const int start = 31 - __clz(heads & upto);
-        const unsigned above = heads & ~upto;
-        const unsigned members = (above ? (above & (0u - above)) - 1u : FULL) & (FULL << start);
         const unsigned smask = __ballot_sync(FULL, surv), qmask = __ballot_sync(FULL, slow);
-        const unsigned mine = smask & members;
-        int first = 0;
-        if (lane == start && mine) first = atomicAdd(&s.nleft_next[c0], __popc(mine));
+        int first = 0, start = 0;
+        unsigned mine = 0;
+        if constexpr (!IN_PLACE) {
+            // runs of equal cells: one place in the bucket per survivor
+            const int prev = __shfl_up_sync(FULL, c0, 1);
+            const unsigned heads = __ballot_sync(FULL, lane == 0 || prev != c0);
+            start = 31 - __clz(heads & upto);
+            const unsigned above = heads & ~upto;
+            const unsigned members = (above ? (above & (0u - above)) - 1u : FULL) & (FULL << start);
+            mine = smask & members;
+            if (lane == start && mine) first = atomicAdd(&s.fill[c0], __popc(mine));
+        }
         c_valid += __popc(__ballot_sync(FULL, valid));
         c_surv += __popc(smask);
         if (slow) {
@@ -940,22 +980,34 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
         if (gone) {  // removed in its cell (a9)
             long long q = 0;
             c_coll += 1;
+            if constexpr (IN_PLACE) mm = b.m[i];
             if (!fixed_of_mass(mm, p.exps[0], q)) set_err(s, ERRB_FIXED_OVERFLOW);
             atomicAdd(&smass[c0], (unsigned long long)(-q));
+            if constexpr (IN_PLACE) {
+                atomicAdd(&s.nleft_next[c0], -1);
+                b.cell[i] = -1;
+            }
         }
-        first = __shfl_sync(FULL, first, start);
-        if (surv) {
-            const int j = slot_of(first + __popc(mine & lt), info.y, info.z);
-            if (j >= 0) {
+        if constexpr (IN_PLACE) {
+            if (surv) {
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    nxt.x[c][j] = xe[c];
-                    nxt.u[c][j] = u[c];
+                for (int c = 0; c < 3; ++c) b.x[c][i] = xe[c];
+            }
+        } else {
+            first = __shfl_sync(FULL, first, start);
+            if (surv) {
+                const int j = slot_of(first + __popc(mine & lt), info.y, info.z);
+                if (j >= 0) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        nxt.x[c][j] = xe[c];
+                        nxt.u[c][j] = u[c];
+                    }
+                    nxt.m[j] = mm;
+                    nxt.cell[j] = c0;
+                    nxt.id[j] = id;
+                    if constexpr (KE) nxt.e[j] = es;
                 }
-                nxt.m[j] = mm;
-                nxt.cell[j] = c0;
-                nxt.id[j] = id;
-                if constexpr (KE) nxt.e[j] = es;
             }
         }
         base = nbase;
@@ -985,10 +1037,24 @@ __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, 
         }
     }
 }
-template <class Real, bool KE, int THREADS>
-__global__ void __launch_bounds__(THREADS, TRACK_PER_SM<Real> / THREADS) k_track(DevMesh m, DevState s, DevParams p, PartBufRaw br,
-                                                                  PartBufRaw nr) {
-    track_body<Real, KE, THREADS>(m, s, p, br, nr);
+// DYN: the simulation may step in place.
+template <class Real, bool KE, int THREADS, bool DYN>
+__device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& bufs) {
+    __shared__ TrackShared<Real, THREADS> sh;
+    // (block-uniform: another block may set the bit while this one starts)
+    if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
+    if constexpr (DYN) {
+        const long long src = s.cnt64[CNT_SRC] * bufs.delta;
+        if (s.cnt64[CNT_IN_PLACE]) track_mode<Real, KE, THREADS, true>(m, s, p, bufs, src, sh);
+        else track_mode<Real, KE, THREADS, false>(m, s, p, bufs, src, sh);
+    } else {
+        track_mode<Real, KE, THREADS, false>(m, s, p, bufs, 0, sh);
+    }
+}
+template <class Real, bool KE, int THREADS, bool DYN>
+__global__ void __launch_bounds__(THREADS, TRACK_PER_SM<Real> / THREADS) k_track(DevMesh m, DevState s, DevParams p,
+                                                                                 PartBufs bufs) {
+    track_body<Real, KE, THREADS, DYN>(m, s, p, bufs);
 }
 
 // ---- fused batches
@@ -1005,56 +1071,68 @@ template <class Real>
 __global__ void __launch_bounds__(CELL_BLOCK) k_sample_scale_b(const __grid_constant__ BatchChunk c) {
     const int32_t* off = c.off[BCL_CELLS];
     const int i = member_of(off, c.n);
-    sample_scale_body<Real>(c.mem[i].m, c.mem[i].s, c.mem[i].p, c.mem[i].a, Blk{(int)blockIdx.x - off[i], off[i + 1] - off[i]});
+    sample_scale_body<Real>(c.mem[i].m, c.mem[i].s, c.mem[i].p, c.mem[i].bufs, Blk{(int)blockIdx.x - off[i], off[i + 1] - off[i]});
 }
 // The particle kernels take every member of the chunk in turn on the whole grid.
 template <class Real>
 __global__ void __launch_bounds__(256) k_sample_write_b(const __grid_constant__ BatchChunk c) {
     for (int k = 0; k < c.n; ++k)
-        sample_write_body<Real>(c.mem[k].m, c.mem[k].s, c.mem[k].p, c.mem[k].a, Blk{(int)blockIdx.x, (int)gridDim.x});
+        sample_write_body<Real>(c.mem[k].m, c.mem[k].s, c.mem[k].p, c.mem[k].bufs, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 // Tiles come from each member's own counter; a block starts at member
 // blockIdx.x mod n, so that the blocks spread over the members' counters.
+// A batch's members always sort (ugkwp_batch_create).
 template <class Real, bool KE, int THREADS>
 __global__ void __launch_bounds__(THREADS, TRACK_PER_SM<Real> / THREADS) k_track_b(const __grid_constant__ BatchChunk c) {
     for (int k = 0; k < c.n; ++k) {
         const BatchMember& e = c.mem[((int)blockIdx.x + k) % c.n];
-        track_body<Real, KE, THREADS>(e.m, e.s, e.p, e.a, e.b);
+        track_body<Real, KE, THREADS, false>(e.m, e.s, e.p, e.bufs);
         __syncthreads();
     }
 }
+
 }  // namespace
 
-void launch_sample_write(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b,
+void launch_sample_write(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b,
                          int blocks, cudaStream_t st) {
     (void)m;
     if (p.precision == UGKWP_MIXED) k_sample_write<float><<<blocks, 256, 0, st>>>(m, s, p, b);
     else k_sample_write<double><<<blocks, 256, 0, st>>>(m, s, p, b);
 }
 
-void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b, cudaStream_t st) {
+void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, cudaStream_t st) {
     if (p.precision == UGKWP_MIXED) k_sample_scale<float><<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s, p, b);
     else k_sample_scale<double><<<blocks_cells(m.nc), CELL_BLOCK, 0, st>>>(m, s, p, b);
 }
 
+// Calls f with (a value of) the particle type, K > 0, the block size and whether
+// the tracking may be in place (binary64 never is).
 namespace {
-template <class Real, bool KE>
-void track_shape(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b, const PartBufRaw& nxt,
-                 const TrackShape& sh, int blocks, cudaStream_t st) {
-    if (sh.threads == 256) k_track<Real, KE, 256><<<blocks, 256, 0, st>>>(m, s, p, b, nxt);
-    else k_track<Real, KE, 128><<<blocks, 128, 0, st>>>(m, s, p, b, nxt);
+template <class Real, bool KE, int THREADS, bool DYN> struct TrackKind {
+    using R = Real;
+    static constexpr bool ke = KE, dyn = DYN;
+    static constexpr int threads = THREADS;
+};
+template <class F> void track_kind(int precision, bool ke, bool dyn, int threads, F&& f) {
+    auto shape = [&](auto real, auto kev, auto dynv) {
+        using R = decltype(real);
+        if (threads == 256) f(TrackKind<R, decltype(kev)::value, 256, decltype(dynv)::value>{});
+        else f(TrackKind<R, decltype(kev)::value, 128, decltype(dynv)::value>{});
+    };
+    using T = std::true_type;
+    using N = std::false_type;
+    if (precision != UGKWP_MIXED) ke ? shape(0.0, T{}, N{}) : shape(0.0, N{}, N{});
+    else if (dyn) ke ? shape(0.0f, T{}, T{}) : shape(0.0f, N{}, T{});
+    else ke ? shape(0.0f, T{}, N{}) : shape(0.0f, N{}, N{});
 }
 }  // namespace
 
-void launch_track(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b, const PartBufRaw& nxt,
-                  const TrackShape& sh, int blocks, cudaStream_t st) {
-    if (p.precision == UGKWP_MIXED) {
-        if (p.K > 0) track_shape<float, true>(m, s, p, b, nxt, sh, blocks, st);
-        else track_shape<float, false>(m, s, p, b, nxt, sh, blocks, st);
-    } else {
-        if (p.K > 0) track_shape<double, true>(m, s, p, b, nxt, sh, blocks, st);
-        else track_shape<double, false>(m, s, p, b, nxt, sh, blocks, st);
-    }
+void launch_track(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, const TrackShape& sh,
+                  int blocks, cudaStream_t st) {
+    track_kind(p.precision, p.K > 0, b.dyn != 0, sh.threads, [&](auto k) {
+        using T = decltype(k);
+        k_track<typename T::R, T::ke, T::threads, T::dyn><<<blocks, T::threads, 0, st>>>(m, s, p, b);
+    });
 }
 
 namespace {
@@ -1064,12 +1142,15 @@ template <class Real, bool KE> cudaError_t configure_type(int carveout) {
     auto set = [&](auto f) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
     };
-    set(k_track<Real, KE, 128>);
-    set(k_track<Real, KE, 256>);
+    for (int threads : {128, 256})
+        for (bool dyn : {false, true})
+            track_kind(sizeof(Real) == 4 ? UGKWP_MIXED : UGKWP_FP64, KE, dyn, threads, [&](auto k) {
+                using T = decltype(k);
+                set(k_track<typename T::R, T::ke, T::threads, T::dyn>);
+                set(k_track_b<typename T::R, T::ke, T::threads>);
+            });
     set(k_sample_write<Real>);
     set(k_sample_scale<Real>);
-    set(k_track_b<Real, KE, 128>);
-    set(k_track_b<Real, KE, 256>);
     set(k_sample_write_b<Real>);
     set(k_sample_scale_b<Real>);
     return e;
@@ -1089,21 +1170,12 @@ void launch_sample_write_batch(const BatchChunk& c, int blocks, int precision, c
     if (precision == UGKWP_MIXED) k_sample_write_b<float><<<blocks, 256, 0, st>>>(c);
     else k_sample_write_b<double><<<blocks, 256, 0, st>>>(c);
 }
-namespace {
-template <class Real, bool KE>
-void track_batch_shape(const BatchChunk& c, const TrackShape& sh, int blocks, cudaStream_t st) {
-    if (sh.threads == 256) k_track_b<Real, KE, 256><<<blocks, 256, 0, st>>>(c);
-    else k_track_b<Real, KE, 128><<<blocks, 128, 0, st>>>(c);
-}
-}  // namespace
 void launch_track_batch(const BatchChunk& c, int precision, bool ke, const TrackShape& sh, int blocks,
                         cudaStream_t st) {
-    if (precision == UGKWP_MIXED) {
-        if (ke) track_batch_shape<float, true>(c, sh, blocks, st);
-        else track_batch_shape<float, false>(c, sh, blocks, st);
-    } else {
-        if (ke) track_batch_shape<double, true>(c, sh, blocks, st);
-        else track_batch_shape<double, false>(c, sh, blocks, st);
-    }
+    track_kind(precision, ke, false, sh.threads, [&](auto k) {
+        using T = decltype(k);
+        k_track_b<typename T::R, T::ke, T::threads><<<blocks, T::threads, 0, st>>>(c);
+    });
 }
+
 }  // namespace ugkwp

@@ -48,6 +48,11 @@ enum : int {
     CNT_NSAM = 14,      // particles sampled this step (from the scan)
     CNT_WTOT = 15,      // slots of the survivor buckets of the buffer written this step (from the scan)
     CNT_MOVERS = 16,    // particles of this step whose counting flux is not zero
+    CNT_CUR = 17,       // the buffer (0, 1) that holds the particles between steps; during a step, the
+                        // one that will hold them after it
+    CNT_SRC = 18,       // the buffer this step's particles are in
+    CNT_IN_PLACE = 19,  // this step leaves them there (1) or rewrites them sorted by cell (0)
+    CNT_AGE = 20,       // steps in place since the particles were last sorted
     CNT_TILE = 32,      // next run of tracking tiles
     CNT_IMPORT = 40,    // a state import's first failed particle: (index << 3) | problem
     CNT_OVF = 48,       // overflow slots (survivors whose bucket is full) taken this step
@@ -80,7 +85,7 @@ struct DevParams {
     int32_t averaging;     // add dt W^{n+1} to the time-average sums
     int32_t gks;           // 0: UGKWP step; 1: GKS step (no particles); 2: GKS step, local time steps
     int32_t K;             // internal degrees of freedom
-    int32_t kpad_;
+    int32_t in_place;      // the simulation may leave its particles in place (PartBufs::dyn)
     uint64_t seed;
     int64_t capacity;
     int32_t exps[5];
@@ -161,6 +166,35 @@ struct PartBufRaw {
     void* e;
 };
 
+// The two particle buffers as the kernels of a step get them: the arrays of one
+// and the signed distance in bytes to those of the other (the same for every
+// array).  A simulation that always sorts (dyn = 0) swaps them on the host, b0
+// holding the step's particles.  One that may leave its particles in place
+// (dyn = 1, see IN_PLACE_CAPACITY) passes buffer 0, and the device knows which one
+// holds them (CNT_CUR, CNT_SRC).
+struct PartBufs {
+    PartBufRaw b0;
+    int64_t delta;
+    int32_t dyn;
+    int32_t pad;
+};
+// In place or sorted by cell (a11; per step, k_scan_apply): in place a particle that
+// stays in its cell writes its position only (of 44 B read and 44 B written in mixed
+// mode, 36 and 12), and nothing takes a slot of a bucket; but neighbouring slots
+// drift into different cells (9% a step in a rarefied cavity), the removed
+// particles stay as holes and the samples follow in rows of their own.  The
+// particles are sorted every RESORT-th step, and whenever holes make up a fifth of
+// the slots, samples a ninth of the particles, or four times this step's samples
+// might not fit.  Two steps of a channel of 393,216 tets (6.7e7 particles): always
+// sorted 5.98 ms, sorted every 2nd / 3rd / 4th / 6th / 12th step 5.59 / 5.43 / 5.29 /
+// 5.21 / 5.19 ms.
+constexpr int RESORT = 6;
+// Mixed-mode simulations of at least this particle capacity may step in place: a
+// smaller one is bound by latencies, to which the extra indirection adds (tube of
+// 1,992 tets 62.4 against 60.5 us, 16^3 cavity of 3e6 particles 487 against 475 us
+// for two steps; 24^3 cavity of 1.9e7 1.60 against 1.64 ms), binary64 by its pipe.
+constexpr int64_t IN_PLACE_CAPACITY = (int64_t)1 << 25;
+
 struct DevState {
     double* W;            // [5][nc]
     double* prim;         // [5][nc] rho, Ux, Uy, Uz, T
@@ -176,18 +210,18 @@ struct DevState {
     int32_t* nsam;        // [nc]
     double* msam;         // [nc]
     int32_t* nleft;       // [nc] survivors at the start of the step
-    int32_t* nleft_next;  // [nc]
+    int32_t* nleft_next;  // [nc] (in place: the particles after sampling, less what leaves or is removed, plus
+                          // what arrives; sorting: fill)
     int64_t* smass;       // [nc] survivors' fixed-point mass
     int64_t* smass_next;  // [nc]
-    int32_t* cnt;         // [nc] particles per cell after sampling
+    int32_t* fill;        // [nc] slots of the cell's survivor bucket taken this step
     int32_t* soff;        // [nc] exclusive scan of N_sam (sampled-particle index)
     int32_t* wcap;        // [nc] slots of the cell's survivor bucket in the buffer written this step
     int4* cinfo;          // [nc] what the tracking reads per cell: collision threshold (a particle whose
                           // first random word is below it does not collide), woff, wcap, and the
                           // bits of the inside test's margin (binary32)
     uint32_t* cthr;       // [nc] the collision thresholds
-    int32_t* woff;        // [nc] first slot of that bucket (exclusive scan of wcap); the bucket's
-                          // fill count is nleft_next (the survivors that ended in the cell)
+    int32_t* woff;        // [nc] first slot of that bucket (exclusive scan of wcap)
     int64_t* pflux;       // [5][nc] fixed-point particle flux
     int64_t* wacc;        // [5][nc] fixed-point scratch for W^p
     double* mom;          // [5][nc] staging of moments copied to the host
@@ -200,14 +234,12 @@ struct DevState {
     int64_t* cnt64;       // [CNT_SLOTS]
 };
 
-// One member of a fused batch: a simulation's device structures for one step,
-// with its particle buffers in this step's roles.
+// One member of a fused batch: a simulation's device structures for one step.
 struct BatchMember {
     DevMesh m;
     DevState s;
     DevParams p;
-    PartBufRaw a;   // this step's particles
-    PartBufRaw b;   // the buffer the survivors are written to
+    PartBufs bufs;
 };
 
 // The block a kernel body runs as: its index among the blocks that work on
@@ -263,14 +295,14 @@ struct LaunchCfg {
     int carveout;         // preferred shared-memory carveout (percent) of the step's kernels, -1: driver default
 };
 
-void launch_sample_write(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b,
+void launch_sample_write(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b,
                          int blocks, cudaStream_t st);
 // Energy-matched sampling, after launch_sample_write: the samples' velocities.
-void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b, cudaStream_t st);
-// Tracking of buffer b (survivors, then this step's samples): the survivors go
-// into their end cells' buckets in nxt, the counting flux into pflux.
-void launch_track(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& b,
-                  const PartBufRaw& nxt, const TrackShape& sh, int blocks, cudaStream_t st);
+void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, cudaStream_t st);
+// Tracking of the particles and this step's samples, in place or into their end
+// cells' buckets in the other buffer; the counting flux goes into pflux.
+void launch_track(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, const TrackShape& sh,
+                  int blocks, cudaStream_t st);
 // The common preferred shared-memory carveout of the step's kernels (a
 // kernel attribute): set outside stream capture, before the configuration's
 // first launch.
@@ -284,9 +316,9 @@ void launch_face_flux(const DevMesh& m, const DevState& s, const DevParams& p, i
 void launch_face_flux_o2(const DevMesh& m, const DevState& s, const DevParams& p, int blocks, cudaStream_t st);
 void launch_gradients(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
 void launch_gp_coef(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
-// a10, and the end of a11: the unused slots of each survivor bucket of the
-// buffer written this step (cell array wcell) are marked as holes.
-void launch_cell_update(const DevMesh& m, const DevState& s, const DevParams& p, int32_t* wcell, cudaStream_t st);
+// a10, and the end of a11: in a step that sorted, the unused slots of each
+// survivor bucket are marked as holes.
+void launch_cell_update(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, cudaStream_t st);
 // the wave part of a step's update (before the particle part of launch_cell_update)
 void launch_wave_update(const DevMesh& m, const DevState& s, cudaStream_t st);
 // Survivor bucket of a cell that starts a step with `cnt` particles: the slots
@@ -300,8 +332,7 @@ void launch_rebuild_survivors(const DevMesh& m, const DevState& s, const DevPara
 void launch_import(int nc, long long n, bool mixed, bool convert, const double* anc, const double* xs,
                    const double* us, const double* es, const PartBufRaw& b, unsigned long long* err,
                    cudaStream_t st);
-void launch_wp_moments(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufRaw& a,
-                       double* out, cudaStream_t st);
+void launch_wp_moments(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, cudaStream_t st);
 void launch_prim_moments(const DevMesh& m, const DevState& s, const DevParams& p, int which,
                          double* out, cudaStream_t st);
 void launch_wbar(const DevMesh& m, const DevState& s, double* out, cudaStream_t st);

@@ -47,3 +47,57 @@ def test_particle_moments_after_steps(precision, K, n):
     WP = np.stack([np.bincount(st["cell"], p, len(tets)) for p in phi]) / vol
     np.testing.assert_allclose(s.moments(ugkwp.WP), WP, rtol=1e-12, atol=1e-12)
     np.testing.assert_allclose(s.moments(ugkwp.WH), st["W"] - WP, rtol=1e-11, atol=1e-11)
+
+
+def _by_id(st):
+    o = np.argsort(st["id"])
+    return [st["id"][o], st["cell"][o], st["m"][o], st["x"][:, o], st["u"][:, o], st["e"][o]]
+
+
+@pytest.mark.parametrize("flow,sampling,K", [("cavity", "maxwell", 0), ("cavity", "maxwell", 2),
+                                             ("channel", "energy_matched", 0), ("cavity", "gp1", 0)])
+def test_in_place_steps_equal_sorted_steps(flow, sampling, K):
+    """A mixed-mode simulation of a capacity from 2^25 on leaves its particles in
+    their slots in most steps; a smaller one sorts them in every step.  Both give
+    the same bits: fields, particles, counts, W^p, through single and replayed
+    steps, an import half-way and a batch."""
+    import torch
+    from paper_2007_13091_gb300 import ugkwp
+    if flow == "cavity":
+        cfg = wl.cavity(n=6, Kn=0.3, N_ref=80, precision="mixed", order=2, K=K)
+    else:
+        cfg = wl.wall_channel(n=(9, 4, 5), Kn=0.2, N_ref=70, precision="mixed")
+    cfg["params"]["sampling"] = sampling
+    sims = []
+    for cap in (1 << 25, 1 << 19):
+        p = dict(cfg["params"], particle_capacity=cap)
+        sims.append(ugkwp.Simulation(cfg["mesh"], cfg["W0"], p, stream=torch.cuda.Stream()))
+    big, small = sims
+    unsorted = 0
+
+    def same():
+        a, b = big.state_native(), small.state_native()
+        for x, y in zip(_by_id(a), _by_id(b)):
+            assert np.array_equal(x, y)
+        assert np.array_equal(a["W"], b["W"]) and a["t"] == b["t"]
+        for k in ("n_sam", "surv_count", "surv_mass", "pflux"):
+            assert np.array_equal(big.last(k), small.last(k)), k
+        assert np.array_equal(big.moments(ugkwp.WP), small.moments(ugkwp.WP))
+        return int((np.diff(a["cell"]) < 0).sum()) - int((np.diff(b["cell"]) < 0).sum())
+
+    for n in (1, 1, 2, 3, 4, 1, 6):
+        sa, sb = big.step(n, stats=True), small.step(n, stats=True)
+        assert {k: v for k, v in sa.items()} == {k: v for k, v in sb.items()}
+        unsorted = max(unsorted, same())
+    assert unsorted > 100  # steps in place did happen
+    st = big.state()
+    big.set_state(st)
+    small.set_state(st)
+    for s in sims:
+        s.step(5)
+    same()
+    batch = ugkwp.Batch(sims)
+    batch.step(5)
+    batch.sync()
+    batch.close()
+    same()
