@@ -63,6 +63,8 @@ struct ugkwp_sim {
     // the wave flux (binary64-bound) runs beside the particle kernels; the
     // second half of the tracking grid joins from `aux` once the wave is done
     cudaStream_t wave = nullptr, aux = nullptr;
+    cudaStream_t adj = nullptr;  // the adjoint's frozen forward (created by its first call)
+    cudaEvent_t recorded = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr, sampled = nullptr, tracked = nullptr, gp_ready = nullptr,
                 waved = nullptr;
     // grid sizes of the looping step kernels
@@ -97,6 +99,8 @@ struct ugkwp_sim {
         if (imp) cudaFree(imp);
         if (wave) cudaStreamDestroy(wave);
         if (aux) cudaStreamDestroy(aux);
+        if (adj) cudaStreamDestroy(adj);
+        if (recorded) cudaEventDestroy(recorded);
     }
 };
 
@@ -1529,29 +1533,39 @@ int ugkwp_adjoint_wave(ugkwp_sim* s, const ugkwp_adjoint_req* r, double* out) {
     cudaStream_t q = s->stream;
     const size_t nc = s->M.nc;
     CU(cudaMemcpyAsync(theta, th_h, sizeof(th_h), cudaMemcpyHostToDevice, q));
-    // 1. record K real steps
+    // 1. K real steps, each recorded; 2. the frozen forward at theta (checkpoints and
+    // the functional), step by step on a stream of its own behind the recording:
+    // its binary64 work runs beside the tracking of the next real steps (channel of
+    // 40,500 tets, first order, 10 steps: 7.35 -> 6.98 ms)
+    if (!s->adj) {
+        CU(cudaStreamCreateWithFlags(&s->adj, cudaStreamNonBlocking));
+        CU(cudaEventCreateWithFlags(&s->recorded, cudaEventDisableTiming));
+    }
+    struct Drain {  // the scratch is the caller's: no way out while the stream uses it
+        cudaStream_t q;
+        ~Drain() { cudaStreamSynchronize(q); }
+    } drain{s->adj};
     CU(cudaMemcpyAsync(ck, s->S.W, 5 * nc * sizeof(double), cudaMemcpyDeviceToDevice, q));
     for (int n = 0; n < K; ++n) {
         rc = ugkwp_step(s, 1, nullptr);
         if (rc) return rc;
         CU(cudaMemcpyAsync(dtv + n, s->S.dt, sizeof(double), cudaMemcpyDeviceToDevice, q));
         launch_adj_record(s->M, s->S, s->P, rp + (size_t)n * nc, pf + (size_t)n * 5 * nc, q);
+        CU(cudaEventRecord(s->recorded, q));
+        CU(cudaStreamWaitEvent(s->adj, s->recorded, 0));
+        launch_adj_forward(s->M, s->P, ap, ck + (size_t)n * 5 * nc, rp + (size_t)n * nc, pf + (size_t)n * 5 * nc, dtv + n,
+                           theta, step_o2(n), F, jf, sums + n, ck + (size_t)(n + 1) * 5 * nc, s->adj);
     }
+    CU(cudaEventRecord(s->recorded, s->adj));
     rc = read_error(s);
     if (rc) return rc;
-    std::vector<double> dth(K);
-    CU(cudaMemcpyAsync(dth.data(), dtv, K * sizeof(double), cudaMemcpyDeviceToHost, q));
-    CU(cudaStreamSynchronize(q));
-    // 2. frozen forward at theta: checkpoints and the functional
-    for (int n = 0; n < K; ++n)
-        launch_adj_forward(s->M, s->P, ap, ck + (size_t)n * 5 * nc, rp + (size_t)n * nc, pf + (size_t)n * 5 * nc, dth[n],
-                           theta, step_o2(n), F, jf, sums + n, ck + (size_t)(n + 1) * 5 * nc, q);
+    CU(cudaStreamWaitEvent(q, s->recorded, 0));
     // 3. reverse sweep
     CU(cudaMemsetAsync(lam1, 0, 5 * nc * sizeof(double), q));
     double* next = lam1;
     double* cur = lam0;
     for (int n = K - 1; n >= 0; --n) {
-        launch_adj_reverse(s->M, s->P, ap, ck + (size_t)n * 5 * nc, rp + (size_t)n * nc, dth[n], theta, step_o2(n), next,
+        launch_adj_reverse(s->M, s->P, ap, ck + (size_t)n * 5 * nc, rp + (size_t)n * nc, dtv + n, theta, step_o2(n), next,
                            cur, fb, thbar, sums + K + 3 * (size_t)n, q);
         std::swap(next, cur);
     }

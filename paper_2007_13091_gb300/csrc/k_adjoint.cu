@@ -227,11 +227,12 @@ __global__ void __launch_bounds__(128) k_adj_grad(DevMesh m, DevParams P, AdjPar
 // ---- forward: fluxes and the functional's terms (boundary faces) at theta
 template <bool O2>
 __global__ void __launch_bounds__(128) k_adj_fwd_flux(DevMesh m, DevParams P, AdjParams ap, const double* W,
-                                                      const double* rho_p, double dt, const double* theta,
+                                                      const double* rho_p, const double* dt_n, const double* theta,
                                                       const double* rec, double* F, double* jf) {
     const int nc = m.nc, nf = m.nf;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nf) return;
+    const double dt = dt_n[0];
     const int f = m.face_order[t];  // interior faces first
     const double n[3] = {m.f_n[f], m.f_n[nf + f], m.f_n[2 * nf + f]};
     const int o = m.f_own[f], nb = m.f_nbr[f];
@@ -416,13 +417,14 @@ constexpr int ROW1 = 6;
 // thbar[3][nbf].
 template <bool O2>
 __global__ void __launch_bounds__(128) k_adj_face(DevMesh m, DevParams P, AdjParams ap, const double* W,
-                                                  const double* rho_p, double dt, const double* theta,
+                                                  const double* rho_p, const double* dt_n, const double* theta,
                                                   const double* rec, const double* lam_next, double* fb,
                                                   double* thbar) {
     constexpr int ROW = O2 ? REC_N : ROW1;
     const int nc = m.nc, nf = m.nf;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nf) return;
+    const double dt = dt_n[0];
     const int f = m.face_order[t];  // interior faces first
     const int o = m.f_own[f], nb = m.f_nbr[f];
     const double n[3] = {m.f_n[f], m.f_n[nf + f], m.f_n[2 * nf + f]};
@@ -597,7 +599,7 @@ void launch_adj_record(const DevMesh& m, const DevState& s, const DevParams& p, 
 }
 
 void launch_adj_forward(const DevMesh& m, const DevParams& p, const AdjParams& ap, const double* W, const double* rho_p,
-                        const double* pf, double dt, const double* theta, const AdjO2& o2, double* F, double* jf,
+                        const double* pf, const double* dt, const double* theta, const AdjO2& o2, double* F, double* jf,
                         double* Jn, double* Wn, cudaStream_t st) {
     const int gf = (m.nf + 127) / 128, gc = (m.nc + 127) / 128;
     if (p.order == 2) {
@@ -611,7 +613,7 @@ void launch_adj_forward(const DevMesh& m, const DevParams& p, const AdjParams& a
 }
 
 void launch_adj_reverse(const DevMesh& m, const DevParams& p, const AdjParams& ap, const double* W,
-                        const double* rho_p, double dt, const double* theta, const AdjO2& o2, const double* lam_next,
+                        const double* rho_p, const double* dt, const double* theta, const AdjO2& o2, const double* lam_next,
                         double* lam, double* fb, double* thbar, double* th_out, cudaStream_t st) {
     const int gf = (m.nf + 127) / 128, gc = (m.nc + 127) / 128;
     if (p.order == 2) {

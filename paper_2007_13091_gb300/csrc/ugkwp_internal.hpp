@@ -399,13 +399,14 @@ struct AdjO2 {
 };
 // Values per side of a face in the reverse sweep's face rows.
 size_t adjoint_face_row(int order);
-// Fluxes at theta, the step's functional term Jn[0] and the next state Wn.
+// Fluxes at theta, the step's functional term Jn[0] and the next state Wn (dt: the
+// step's recorded time step, on the device).
 void launch_adj_forward(const DevMesh& m, const DevParams& p, const AdjParams& ap, const double* W, const double* rho_p,
-                        const double* pf, double dt, const double* theta, const AdjO2& o2, double* F, double* jf,
+                        const double* pf, const double* dt, const double* theta, const AdjO2& o2, double* F, double* jf,
                         double* Jn, double* Wn, cudaStream_t st);
 // lambda^n from lambda^{n+1} and this step's dJ/dtheta terms th_out[3].
 void launch_adj_reverse(const DevMesh& m, const DevParams& p, const AdjParams& ap, const double* W,
-                        const double* rho_p, double dt, const double* theta, const AdjO2& o2, const double* lam_next,
+                        const double* rho_p, const double* dt, const double* theta, const AdjO2& o2, const double* lam_next,
                         double* lam, double* fb, double* thbar, double* th_out, cudaStream_t st);
 
 int sm_count();       // multiprocessors of the current device
