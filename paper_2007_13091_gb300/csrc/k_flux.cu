@@ -43,7 +43,10 @@ namespace {
 // which then spreads evenly over the SMs and leaves each its room for a block
 // of the wave flux: two steps of the settled 24^3 cavity take 2.22 ms in a row
 // and 2.26 ms on their own, against 2.19 and 2.57 with three blocks per SM and
-// 2.24 and 2.57 with four.
+// 2.24 and 2.57 with four.  In the start-up steps and with
+// first-order g_p sampling, which waits for the gradients, nothing runs beside it:
+// four (four start-up steps of a channel of 96,000 tets 2.01 against 2.03 ms, two
+// g_p-sampled steps of the 16^3 cavity 478 -> 467 us).
 constexpr int GRAD_THREADS = 128, GRAD_BLOCKS_PER_SM = 2;
 
 // Constants of K internal degrees of freedom (rho E = rho |U|^2/2 + (3+K)/2 p,
@@ -373,7 +376,7 @@ static int wave_grid(long long n, int threads, int blocks) {
 // beside it for the first half of the tracking grid.
 void launch_gradients(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
     const int t = wave_block(3LL * m.nc, GRAD_THREADS);
-    k_gradients<<<wave_grid(3LL * m.nc, t, GRAD_BLOCKS_PER_SM * sm_count() * (GRAD_THREADS / t)), t, 0, st>>>(m, s, p);
+    k_gradients<<<wave_grid(3LL * m.nc, t, (p.gks || p.sampling == UGKWP_SAMPLE_GP1 ? 4 : GRAD_BLOCKS_PER_SM) * sm_count() * (GRAD_THREADS / t)), t, 0, st>>>(m, s, p);
 }
 
 void launch_gp_coef(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st) {
