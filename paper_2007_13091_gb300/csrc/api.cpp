@@ -205,6 +205,7 @@ void layout(const MeshHost& mh, int64_t cap, size_t rs, bool with_e, Carver& c, 
     S.F = c.take<double>(5 * nf);
     S.rec = c.take<double>(REC_N * nc);
     S.bsum = c.take<int2>((size_t)scan_blocks(mh.nc) + 1);
+    S.gsum = c.take<longlong2>((size_t)scan_groups(mh.nc));
     S.t = c.take<double>(1);
     S.dt = c.take<double>(1);
     S.cnt64 = c.take<int64_t>(CNT_SLOTS);

@@ -229,6 +229,7 @@ struct DevState {
     double* rec;          // [nc][REC_N] order 2: what a face reads of a cell: W (5), rho^h, the limited
                           // gradients of W [3q + d] (15) and of rho^h (3)
     int2* bsum;           // [scan_blocks] block sums of (bucket slots, N_sam)
+    longlong2* gsum;      // [scan_groups] their sums over groups of SCAN_GROUP blocks
     double* t;            // [1]
     double* dt;           // [1]
     int64_t* cnt64;       // [CNT_SLOTS]
@@ -277,14 +278,16 @@ constexpr int GP_ATTEMPTS = 64;
 // 9,600 tets in binary64 4.14 / 4.16 / 4.34 ms.
 constexpr int CELL_BLOCK = 64;
 constexpr int SCAN_BLOCK = 64;
+constexpr int SCAN_GROUP = 64;
 __host__ __device__ inline int scan_blocks(int nc) { return (nc + SCAN_BLOCK - 1) / SCAN_BLOCK; }
+__host__ __device__ inline int scan_groups(int nc) { return (scan_blocks(nc) + SCAN_GROUP - 1) / SCAN_GROUP; }
 
 void launch_cell_prep(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
 void launch_sample_count(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
 void launch_scan(const DevMesh& m, const DevState& s, const DevParams& p, cudaStream_t st);
 // Grid sizes of the step kernels that loop over their work (any positive
 // value gives the same results; chosen for speed, e.g. by the autotuner).
-// Shape of the tracking kernel: threads (= particles) per block and tile.
+// Shape of the tracking kernel: threads per block (its warps work on their own).
 struct TrackShape {
     int threads;  // 128 or 256
 };
@@ -355,7 +358,7 @@ struct BatchChunk {
 static_assert(sizeof(BatchChunk) <= 32764, "a chunk must fit a launch's parameter space");
 int blocks_cells(int nc);        // one thread per cell, CELL_BLOCK per block
 int blocks_gp_coef(int nc);      // one thread per cell, 128 per block
-int gradient_threads();          // threads per block of the gradient kernel (one per cell)
+int gradient_threads();          // threads per block of the gradient kernel (three per cell)
 int gradient_blocks_per_sm();    // its persistent grid
 void launch_cell_prep_batch(const BatchChunk& c, int blocks, cudaStream_t st);
 void launch_sample_count_batch(const BatchChunk& c, int blocks, cudaStream_t st);
