@@ -55,6 +55,7 @@ __device__ __forceinline__ void cell_prep_body(const DevMesh& m, const DevState&
         for (int q = 0; q < 5; ++q) s.pflux[(size_t)q * nc + i] = 0;
         s.fill[i] = 0;
         if (i < scan_groups(nc)) s.gsum[i] = make_longlong2(0, 0);
+        if (i == 0) s.cnt64[CNT_FLUX] = 0;
         const double rho = s.W[i];
         const double Ux = s.W[nc + i] / rho, Uy = s.W[2 * nc + i] / rho, Uz = s.W[3 * nc + i] / rho;
         const double U2 = (Ux * Ux + Uy * Uy) + Uz * Uz;

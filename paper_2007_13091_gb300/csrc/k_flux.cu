@@ -229,14 +229,55 @@ __global__ void __launch_bounds__(128) k_gp_coef(DevMesh m, DevState s, DevParam
 
 __device__ __forceinline__ void face_flux_o1(const DevMesh& m, const DevState& s, const DevParams& p, int t);
 
+// The faces face_order[first..nf) in tiles of 32, one warp each.  SHARED: a grid that
+// does not cover them takes the tiles from a counter, reserved one ahead, instead of
+// a fixed stride: the tracking's blocks can keep some flux blocks off the SMs until
+// the others are done, and with fixed shares those then start theirs.  Two steps of
+// a batch of 14 instances, second order, 7.33 -> 7.08 ms; of a channel of 393,216
+// tets, first order, 5.12 -> 5.07 ms.  Not SHARED: the second-order kernel of one
+// simulation, whose replayed steps place every block at once (24^3 cavity 1.59
+// against 1.61 ms, start-up steps 2.014 against 2.021).
+template <bool SHARED>
+struct FaceTiles {
+    unsigned long long* next_tile;
+    long long next;
+    int n;
+    int stride;
+    bool shared;
+    __device__ __forceinline__ FaceTiles(const DevState& s, int nf, int first, Blk bk) {
+        next_tile = reinterpret_cast<unsigned long long*>(s.cnt64 + CNT_FLUX);
+        n = nf;
+        stride = bk.n * blockDim.x;
+        shared = SHARED && stride < nf - first;
+        base = first;
+        next = first + (shared ? reserve() : (long long)bk.id * blockDim.x + (threadIdx.x & ~31u));
+    }
+    __device__ __forceinline__ bool take(int& t) {
+        const long long t0 = SHARED ? __shfl_sync(0xffffffffu, next, 0) : next;
+        if (t0 >= n) return false;
+        t = (int)t0 + (int)(threadIdx.x & 31);
+        next = shared ? base + reserve() : next + stride;
+        return true;
+    }
+
+   private:
+    int base;
+    __device__ __forceinline__ long long reserve() {  // (lane 0's counts)
+        return (threadIdx.x & 31) == 0 ? (long long)atomicAdd(next_tile, 32ull) : 0;
+    }
+};
+
 // Second-order flux of the interior faces (the first nif entries of face_order),
 // then the first-order flux of the boundary faces that follow them.
 // With local time steps (GKS step) each face is integrated over the smaller
 // step of its cells and stores the mean flux rate F / dt_f.
+template <bool SHARED>
 __device__ __forceinline__ void face_flux_o2_body(const DevMesh& m, const DevState& s, const DevParams& p, Blk bk) {
     const int nf = m.nf;
     const double dt = s.dt[0];
-    for (int t = bk.id * blockDim.x + threadIdx.x; t < nf; t += bk.n * blockDim.x) {
+    FaceTiles<SHARED> tiles(s, nf, 0, bk);
+    for (int t; tiles.take(t);) {
+        if (t >= nf) continue;
         if (t >= m.nif) {  // the boundary faces follow, at first order, in the same grid
             face_flux_o1(m, s, p, t);
             continue;
@@ -253,7 +294,7 @@ __device__ __forceinline__ void face_flux_o2_body(const DevMesh& m, const DevSta
     }
 }
 __global__ void __launch_bounds__(UGKWP_WAVE_THREADS, UGKWP_WAVE_MIN_BLOCKS) k_face_flux_o2(DevMesh m, DevState s, DevParams p) {
-    face_flux_o2_body(m, s, p, Blk{(int)blockIdx.x, (int)gridDim.x});
+    face_flux_o2_body<false>(m, s, p, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // First-order flux of face face_order[t].
@@ -316,10 +357,11 @@ __device__ __forceinline__ void face_flux_o1(const DevMesh& m, const DevState& s
     for (int q = 0; q < 5; ++q) s.F[(size_t)q * nf + f] = F[q];
 }
 
-// First-order flux of the faces face_order[first..nf), grid-stride.
+// First-order flux of the faces face_order[first..nf).
 __device__ __forceinline__ void face_flux_body(const DevMesh& m, const DevState& s, const DevParams& p, int first, Blk bk) {
-    for (int t = first + bk.id * blockDim.x + threadIdx.x; t < m.nf; t += bk.n * blockDim.x)
-        face_flux_o1(m, s, p, t);
+    FaceTiles<true> tiles(s, m.nf, first, bk);
+    for (int t; tiles.take(t);)
+        if (t < m.nf) face_flux_o1(m, s, p, t);
 }
 __global__ void __launch_bounds__(256) k_face_flux(DevMesh m, DevState s, DevParams p, int first) {
     face_flux_body(m, s, p, first, Blk{(int)blockIdx.x, (int)gridDim.x});
@@ -339,6 +381,13 @@ __device__ __forceinline__ int member_of(const int32_t* off, int n) {
 __device__ __forceinline__ Blk member_blk(const int32_t* off, int i) {
     return Blk{(int)blockIdx.x - off[i], off[i + 1] - off[i]};
 }
+// The flux of a block's own member i, then what is left of the others' tiles (a
+// member whose blocks cover its faces has none).
+template <class F> __device__ __forceinline__ void for_members(const BatchChunk& c, const int32_t* off, int i, F&& flux) {
+    for (int k = 0, j = i; k < c.n; ++k, j = j + 1 < c.n ? j + 1 : 0)
+        if (j == i || (long long)(off[j + 1] - off[j]) * blockDim.x < c.mem[j].m.nf)
+            flux(j, Blk{(int)blockIdx.x - off[j], off[j + 1] - off[j]});
+}
 __global__ void __launch_bounds__(GRAD_THREADS) k_gradients_b(const __grid_constant__ BatchChunk c) {
     const int i = member_of(c.off[BCL_GRAD], c.n);
     gradients_body(c.mem[i].m, c.mem[i].s, c.mem[i].p, member_blk(c.off[BCL_GRAD], i));
@@ -350,11 +399,11 @@ __global__ void __launch_bounds__(128) k_gp_coef_b(const __grid_constant__ Batch
 __global__ void __launch_bounds__(UGKWP_WAVE_THREADS, UGKWP_WAVE_MIN_BLOCKS)
     k_face_flux_o2_b(const __grid_constant__ BatchChunk c) {
     const int i = member_of(c.off[BCL_FLUX_O2], c.n);
-    face_flux_o2_body(c.mem[i].m, c.mem[i].s, c.mem[i].p, member_blk(c.off[BCL_FLUX_O2], i));
+    for_members(c, c.off[BCL_FLUX_O2], i, [&](int k, Blk bk) { face_flux_o2_body<true>(c.mem[k].m, c.mem[k].s, c.mem[k].p, bk); });
 }
 __global__ void __launch_bounds__(256) k_face_flux_b(const __grid_constant__ BatchChunk c) {
     const int i = member_of(c.off[BCL_FLUX], c.n);
-    face_flux_body(c.mem[i].m, c.mem[i].s, c.mem[i].p, 0, member_blk(c.off[BCL_FLUX], i));
+    for_members(c, c.off[BCL_FLUX], i, [&](int k, Blk bk) { face_flux_body(c.mem[k].m, c.mem[k].s, c.mem[k].p, 0, bk); });
 }
 
 }  // namespace

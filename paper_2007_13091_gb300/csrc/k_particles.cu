@@ -669,8 +669,8 @@ template <class Real> __device__ __forceinline__ const float4* test_planes(const
 // cavity).  Binary64 is bound by its pipe: what is left there per particle are the
 // end point (6 instructions), and per queued particle the logarithm, the last
 // segment, walls and the counting flux; the exit faces are decided in binary32
-// (exit_face32).  Two steps of the settled 24^3 cavity, mixed, 1.69 ms; of the 21^3
-// cavity in binary64 2.20 ms; with the walk of every first tet, block-wide output
+// (exit_face32).  Two steps of the settled 24^3 cavity, mixed, 1.60 ms; of the 21^3
+// cavity in binary64 2.17 ms; with the walk of every first tet, block-wide output
 // rounds and a mover list for a flux kernel of its own 2.20 and 7.33 ms, with
 // every exit face decided in binary64 and no prefetch of the next tile's lines
 // 1.78 and 2.99 ms.

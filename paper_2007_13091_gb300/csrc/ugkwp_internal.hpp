@@ -53,6 +53,7 @@ enum : int {
     CNT_SRC = 18,       // the buffer this step's particles are in
     CNT_IN_PLACE = 19,  // this step leaves them there (1) or rewrites them sorted by cell (0)
     CNT_AGE = 20,       // steps in place since the particles were last sorted
+    CNT_FLUX = 24,      // next tile of the wave flux's faces
     CNT_TILE = 32,      // next run of tracking tiles
     CNT_IMPORT = 40,    // a state import's first failed particle: (index << 3) | problem
     CNT_OVF = 48,       // overflow slots (survivors whose bucket is full) taken this step
