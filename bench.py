@@ -48,22 +48,14 @@ TRACK_BYTES_PER_CELL = {"mixed": 80 + 8, "fp64": 144 + 8}
 # launches) on this workload, from the ncu capture summarised in
 # profiles/k_track_cavity24_mixed.md; set to None whenever the
 # kernel changes until it is captured again
-TRACK_DRAM_BYTES = {"mixed": 1229627648 + 1073300224 + 48128, "fp64": None}
-# bytes the movers' flux kernel reads per mover (start and end velocity, mass,
-# start cell, end cell and exit flag), MIXED / FP64
-MOVER_BYTES = {"mixed": 12 + 12 + 8 + 4 + 8, "fp64": 24 + 24 + 8 + 4 + 8}
-# int64 atomic additions per mover: -phi at the start cell, +phi at the end cell
-MOVER_ATOMICS = 10
-# binary64 pipe operations of one phi = m (1, u, |u|^2/2): MIXED 3 widenings,
-# 7 products and 3 sums; FP64 the products and sums
-MOVER_FP64_OPS = {"mixed": 13, "fp64": 10}
+TRACK_DRAM_BYTES = {"mixed": 1297060096 + 1032955392 + 74752, "fp64": None}
 # Binary64 flops per interior face of k_face_flux_o2 (the second-order wave flux):
 # ncu's executed dadd + dmul + 2 dfma per launch divided by the interior faces, on
 # this workload (profiles/); None until captured for the current kernel.
 # (the kernel also takes the boundary faces' first-order flux after the
 # interior faces: their flops are included, counted per interior face)
-FLUX_O2_FLOPS_PER_FACE = (29934208 + 80965504 + 2 * 148104192) / 162432
-FLUX_O2_DRAM_BYTES = 31148800 + 512
+FLUX_O2_FLOPS_PER_FACE = (15.82e6 + 49.19e6 + 2 * 98.10e6) / 162432
+FLUX_O2_DRAM_BYTES = 31970000
 # FP64 peak: 2 FP64 FMA lanes per clock per SM (the nominal 1.25 TFLOP/s of this
 # part at 152 SMs and 2.07 GHz), 2 flops per FMA
 FP64_FMA_LANES_PER_SM = 2
@@ -938,7 +930,8 @@ def main():
     kmoves = kms.pop("_moves") / args.steps
     alg = TRACK_BYTES_PER_MOVE[args.precision] * kmoves + TRACK_BYTES_PER_CELL[args.precision] * nc
     achieved = alg / (track_ms * 1e-3) / 1e9
-    roof_track = {"kernel": "k_track (a6-a9, a11: t_f draw, tet walk, fixed-point flux, removal, compaction)", "bound": "hbm",
+    roof_track = {"kernel": "k_track (a6-a9, a11: t_f draw, tet walk, fixed-point flux of the particles that moved, "
+                            "removal, sort by cell)", "bound": "hbm",
                   "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                   "peak_kind": f"{peak_kind} HBM copy", "traffic": TRACK_DRAM_BYTES[args.precision],
                   "traffic_unit": "bytes per step, both k_track launches (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
@@ -949,29 +942,6 @@ def main():
                             "two k_track launches: the second starts when the wave flux is done) over "
                             f"{args.steps} further steps of the same run (direct launches, wave flux "
                             "overlapping on the second stream)"}
-    # the movers' flux pass (a8): bound by its arithmetic (binary64 pipe for
-    # phi, integer pipes for the fixed-point conversion); its binary64 work is
-    # one phi per mover and a second one per wall hit
-    movers_ms = kms.get("movers", 0.0) / args.steps
-    n_movers = int(st["n_movers"])
-    n_wall = int(st["n_wall_hits"])
-    fp64_meas = None
-    roof_movers = None
-    if movers_ms > 0.0:
-        fp64_meas = guarded(fp64_peak_measured)
-        ops = MOVER_FP64_OPS[args.precision] * (n_movers + n_wall)
-        ach_ops = ops / (movers_ms * 1e-3) / 1e9
-        peak_ops = fp64_meas * 1e3 / 2.0 if isinstance(fp64_meas, float) else None
-        mb = MOVER_BYTES[args.precision] * n_movers
-        roof_movers = {"kernel": "k_movers (a8: binary64 counting flux of the particles that changed cell, met a "
-                                 "wall or left)", "bound": "alu", "achieved": ach_ops, "peak": peak_ops,
-                       "unit": "Gop/s (binary64 pipe operations)", "frac": ach_ops / peak_ops if peak_ops else None,
-                       "peak_kind": "measured: cuBLAS DGEMM rate on this GPU / 2 (one FMA = 2 flops per pipe slot)",
-                       "traffic": None, "fp64_ops_per_phi": MOVER_FP64_OPS[args.precision],
-                       "movers_per_launch": n_movers, "wall_hits_per_launch": n_wall, "ms_per_launch": movers_ms,
-                       "bytes_read_per_launch": mb, "hbm_gbs": mb / (movers_ms * 1e-3) / 1e9,
-                       "int64_atomics_per_s": MOVER_ATOMICS * n_movers / (movers_ms * 1e-3),
-                       "timing": "CUDA events on the library's stream around each launch"}
     roof_flux = None
     if ORDER == 2 and kms.get("flux_o2", 0.0) > 0.0:
         props = torch.cuda.get_device_properties(local)
@@ -982,8 +952,7 @@ def main():
         except OSError:
             pass
         fp64_nominal = props.multi_processor_count * FP64_FMA_LANES_PER_SM * 2 * sm_mhz * 1e6 / 1e12
-        if fp64_meas is None:
-            fp64_meas = guarded(fp64_peak_measured)
+        fp64_meas = guarded(fp64_peak_measured)
         fp64_peak = fp64_meas if isinstance(fp64_meas, float) else fp64_nominal
         flux_ms = kms["flux_o2"] / args.steps
         n_if = sim.n_faces - sim.n_bfaces
@@ -1018,7 +987,7 @@ def main():
                       "parallelism": "replicas" if ws > 1 else "single GPU"},
            "cell_steps_per_s": cell_steps,
            "roofline": roof_track,
-           "roofline_track": roof_track, "roofline_movers": roof_movers, "roofline_flux_o2": roof_flux,
+           "roofline_track": roof_track, "roofline_flux_o2": roof_flux,
            "kernels_ms_per_step": {k: v / args.steps for k, v in kms.items()},
            "step_launch": "two-step CUDA graphs replayed on the caller's stream",
            "launch_cfg": launch_cfg,
