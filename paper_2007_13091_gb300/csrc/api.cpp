@@ -64,6 +64,7 @@ struct ugkwp_sim {
     // second half of the tracking grid joins from `aux` once the wave is done
     cudaStream_t wave = nullptr, aux = nullptr;
     cudaStream_t adj = nullptr;  // the adjoint's frozen forward (created by its first call)
+    bool recording = false;      // an adjoint call takes steps beside that forward
     cudaEvent_t recorded = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr, sampled = nullptr, tracked = nullptr, gp_ready = nullptr,
                 waved = nullptr;
@@ -858,17 +859,19 @@ int enqueue_step(ugkwp_sim* s) {
         // tracking in two launches that take tiles from one counter: the first
         // half of the grid starts now and leaves room on each SM for a block
         // of the wave flux; the second half starts once the wave flux is done
-        // and takes the tiles that are left
+        // and takes the tiles that are left.  Beside an adjoint's frozen forward
+        // the whole grid starts at once: there the flux shares the SMs with the
+        // forward anyway (first order, 40,500 tets, 10 steps: 6.96 -> 6.73 ms; second
+        // order, 21,168 tets, 4 steps: 3.57 -> 3.46)
         cudaError_t ce = cudaSuccess;
-        const int first_half = (s->lc.particle_blocks + 1) / 2;
+        const int first_half = s->recording ? s->lc.particle_blocks : (s->lc.particle_blocks + 1) / 2;
         timed(s, UGKWP_K_TRACK, s->lc.particle_blocks > first_half ? 2 : 1, q, [&] {
             ce = cudaEventRecord(s->sampled, q);
             launch_track(s->M, s->S, s->P, s->bufs(), s->lc.track, first_half, q);
+            if (s->lc.particle_blocks <= first_half) return;
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(s->aux, s->sampled, 0);
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(s->aux, s->join, 0);
-            if (s->lc.particle_blocks > first_half)
-                launch_track(s->M, s->S, s->P, s->bufs(), s->lc.track, s->lc.particle_blocks - first_half,
-                             s->aux);
+            launch_track(s->M, s->S, s->P, s->bufs(), s->lc.track, s->lc.particle_blocks - first_half, s->aux);
             if (ce == cudaSuccess) ce = cudaEventRecord(s->tracked, s->aux);
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(q, s->tracked, 0);
         });
@@ -1543,12 +1546,14 @@ int ugkwp_adjoint_wave(ugkwp_sim* s, const ugkwp_adjoint_req* r, double* out) {
         CU(cudaEventCreateWithFlags(&s->recorded, cudaEventDisableTiming));
     }
     struct Drain {  // the scratch is the caller's: no way out while the stream uses it
-        cudaStream_t q;
-        ~Drain() { cudaStreamSynchronize(q); }
-    } drain{s->adj};
+        ugkwp_sim* s;
+        ~Drain() { cudaStreamSynchronize(s->adj); }
+    } drain{s};
     CU(cudaMemcpyAsync(ck, s->S.W, 5 * nc * sizeof(double), cudaMemcpyDeviceToDevice, q));
     for (int n = 0; n < K; ++n) {
+        s->recording = true;
         rc = ugkwp_step(s, 1, nullptr);
+        s->recording = false;
         if (rc) return rc;
         CU(cudaMemcpyAsync(dtv + n, s->S.dt, sizeof(double), cudaMemcpyDeviceToDevice, q));
         launch_adj_record(s->M, s->S, s->P, rp + (size_t)n * nc, pf + (size_t)n * 5 * nc, q);
