@@ -701,7 +701,7 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u, upto = FULL >> (31 - lane);
     const int nc = m.nc;
-    unsigned long long* tile_ctr = reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_TILE]);
+    unsigned* tile_ctr = reinterpret_cast<unsigned*>(&s.cnt64[CNT_TILE]);  // (the low word)
     unsigned long long* smass = reinterpret_cast<unsigned long long*>(s.smass_next);
     unsigned long long* pf = reinterpret_cast<unsigned long long*>(s.pflux);
     // warp-uniform counters
@@ -861,12 +861,17 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
     // tiles per run: long enough that the counter is off the path, short enough
     // that a small simulation spreads over the whole grid
     const unsigned run = min(max(n / (32u * 8192u), 1u), 16u) * 32u;
-    unsigned long long ahead = 0;
-    unsigned base = 0, end = 0;
-    if (lane == 0) ahead = atomicAdd(tile_ctr, 1ULL);
-    base = (unsigned)__shfl_sync(FULL, ahead, 0) * run;
+    // (the largest grid hands out fewer than 2^27 runs, but their slots can pass 2^32:
+    // such a run starts at n)
+    auto first_of = [&](unsigned number) {
+        const unsigned k = __shfl_sync(FULL, number, 0);
+        return __umulhi(k, run) ? n : k * run;
+    };
+    unsigned ahead = 0, base = 0, end = 0;
+    if (lane == 0) ahead = atomicAdd(tile_ctr, 1u);
+    base = first_of(ahead);
     end = base + run;
-    if (lane == 0) ahead = atomicAdd(tile_ctr, 1ULL);
+    if (lane == 0) ahead = atomicAdd(tile_ctr, 1u);
     // the first lanes prefetch the lines of the next tile's x, u, m and id (its
     // cells are loaded), one line per lane, with one instruction per tile
     constexpr int XL = sizeof(Real) / 4;  // lines per coordinate array
@@ -913,9 +918,9 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
         // the next tile's cells (its other loads follow at the top of its turn)
         unsigned nbase = base + 32;
         if (nbase == end) {
-            nbase = (unsigned)__shfl_sync(FULL, ahead, 0) * run;
+            nbase = first_of(ahead);
             end = nbase + run;
-            if (lane == 0 && nbase < n) ahead = atomicAdd(tile_ctr, 1ULL);
+            if (lane == 0 && nbase < n) ahead = atomicAdd(tile_ctr, 1u);
         }
         if (nbase < n) {
             cell_i = b.cell[nbase + lane];

@@ -101,3 +101,24 @@ def test_in_place_steps_equal_sorted_steps(flow, sampling, K):
     batch.sync()
     batch.close()
     same()
+
+
+def test_largest_tracking_grid():
+    """2^20 blocks of 256 threads, the largest grid that is accepted, on some 2.6e6
+    particles: its 2^23 warps reserve two runs of 320 slots each, past 2^32 slots,
+    and every particle is tracked once all the same (fields and counts equal those
+    of the default grid, bit for bit)."""
+    import torch
+    from paper_2007_13091_gb300 import ugkwp
+    cfg = wl.cavity(n=14, Kn=0.5, N_ref=160, precision="mixed", order=1)
+    a, b = (ugkwp.Simulation(cfg["mesh"], cfg["W0"], cfg["params"], stream=torch.cuda.Stream()) for _ in range(2))
+    ugkwp.ugkwp_set_launch_cfg(a.handle, 1 << 20, 4, 256)
+    for k in range(3):
+        sa, sb = a.step(1, stats=True), b.step(1, stats=True)
+        assert sa == sb
+        assert k > 0 or sa["n_tracked"] >= 10 * (32 * 8192)  # runs of ten tiles
+    assert 2 * (1 << 20) * 8 * 320 > 1 << 32
+    assert np.array_equal(a.moments(ugkwp.WP), b.moments(ugkwp.WP))
+    assert np.array_equal(a.state_native()["W"], b.state_native()["W"])
+    for k in ("pflux", "surv_count", "surv_mass"):
+        assert np.array_equal(a.last(k), b.last(k)), k
