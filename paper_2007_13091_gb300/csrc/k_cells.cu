@@ -225,9 +225,8 @@ __device__ __forceinline__ void scan_apply_body(const DevMesh& m, const DevState
         s.cnt64[CNT_SAMPLED] = nsam;
         s.cnt64[CNT_WTOT] = wtot;
         const long long live = s.cnt64[CNT_SURV] + nsam, cur = s.cnt64[CNT_CUR], age = s.cnt64[CNT_AGE] + 1;
-        // (past the capacity nothing is written and no particle is left)
-        const bool in_place = p.in_place && (!fits || (age < RESORT && total + 4 * nsam + 4LL * m.nc <= p.capacity &&
-                                        8 * nsam <= live && 4 * (total - live) <= live));
+        const bool in_place = p.in_place && fits && age < RESORT && total + 4 * nsam + 4LL * m.nc <= p.capacity &&
+                              8 * nsam <= live && 4 * (total - live) <= live;
         s.cnt64[CNT_SRC] = cur;
         s.cnt64[CNT_IN_PLACE] = in_place ? 1 : 0;
         s.cnt64[CNT_CUR] = in_place ? cur : 1 - cur;
@@ -275,6 +274,8 @@ __device__ __forceinline__ void cell_update_body(const DevMesh& m, const DevStat
         }
         return;
     }
+    // past the capacity the slots of this step were not all written: no particle is left
+    const bool lost = s.cnt64[CNT_ERR] & ERRB_CAPACITY;
     if (i == 0) {
         s.t[0] = s.t[0] + s.dt[0];
         if (p.averaging) s.tsum[0] += s.dt[0];
@@ -284,11 +285,14 @@ __device__ __forceinline__ void cell_update_body(const DevMesh& m, const DevStat
         const long long ovf = s.cnt64[CNT_OVF];
         const long long room = p.capacity - s.cnt64[CNT_WTOT];
         s.cnt64[CNT_N_A] =
-            s.cnt64[CNT_IN_PLACE] ? s.cnt64[CNT_N_B] : s.cnt64[CNT_WTOT] + (ovf < room ? ovf : room);
+            lost ? 0 : s.cnt64[CNT_IN_PLACE] ? s.cnt64[CNT_N_B] : s.cnt64[CNT_WTOT] + (ovf < room ? ovf : room);
+        if (lost) s.cnt64[CNT_SURV] = 0;
     }
     if (i >= nc) return;
-    // a11: the bucket slots no survivor took are holes
-    if (!s.cnt64[CNT_IN_PLACE] && !(s.cnt64[CNT_ERR] & ERRB_CAPACITY)) {
+    if (lost) {
+        s.nleft_next[i] = 0;
+        s.smass_next[i] = 0;
+    } else if (!s.cnt64[CNT_IN_PLACE]) {  // a11: the bucket slots no survivor took are holes
         int32_t* wcell =
             reinterpret_cast<int32_t*>(reinterpret_cast<char*>(bufs.b0.cell) + (bufs.dyn ? s.cnt64[CNT_CUR] : 1) * bufs.delta);
         const int cap = s.wcap[i], fill = s.fill[i];

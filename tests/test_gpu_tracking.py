@@ -122,3 +122,22 @@ def test_largest_tracking_grid():
     assert np.array_equal(a.state_native()["W"], b.state_native()["W"])
     for k in ("pflux", "surv_count", "surv_mass"):
         assert np.array_equal(a.last(k), b.last(k)), k
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_past_the_capacity_no_particle_is_left(precision):
+    """A step that does not fit the capacity writes no particle; none of the slots
+    it left unwritten is read afterwards: the simulation has no particles until a
+    step fits, and says so in the image, in W^p and in the sums per cell."""
+    from paper_2007_13091_gb300 import ugkwp
+    cfg = wl.shock_tube(nx=20, ny=2, nz=2, precision=precision)
+    cfg["params"]["particle_capacity"] = 1000  # far below the 480 x 50 sampled particles
+    s = ugkwp.Simulation(cfg["mesh"], cfg["W0"], cfg["params"])
+    for n in (1, 2, 1):
+        s.step(n)
+        with pytest.raises(ugkwp.UgkwpError) as e:
+            s.moments(ugkwp.WP)
+        assert e.value.code == ugkwp.E_CAPACITY
+        assert not s.moments(ugkwp.WP).any()
+        assert s.state()["id"].size == 0 and s.state_native()["id"].size == 0
+        assert not s.last("surv_count").any() and not s.last("surv_mass").any()
