@@ -217,19 +217,27 @@ __device__ __forceinline__ void scan_apply_body(const DevMesh& m, const DevState
         s.cinfo[i] = make_int4((int)s.cthr[i], woff, v.x, __float_as_int(m.margin[i]));
     }
     if (bk.id == bk.n - 1 && threadIdx.x == blockDim.x - 1) {
-        const long long wtot = px + incl.x, nsam = py + incl.y, total = s.cnt64[CNT_N_A] + nsam;
+        const long long wtot = px + incl.x, nsam = py + incl.y, slots = s.cnt64[CNT_N_A], left = s.cnt64[CNT_SURV];
+        const long long live = left + nsam, cur = s.cnt64[CNT_CUR], age = s.cnt64[CNT_AGE] + 1;
+        // steps in place leave holes: where the samples do not fit behind the slots,
+        // but behind the particles, these are packed into the other buffer first
+        const bool pack = p.in_place && slots + nsam > p.capacity && live <= p.capacity;
+        const long long total = pack ? live : slots + nsam;
         const bool fits = total <= p.capacity && wtot <= p.capacity;
         if (!fits) set_err(s, ERRB_CAPACITY);
         s.cnt64[CNT_N_B] = fits ? total : 0;
         s.cnt64[CNT_NSAM] = fits ? nsam : 0;
         s.cnt64[CNT_SAMPLED] = nsam;
         s.cnt64[CNT_WTOT] = wtot;
-        const long long live = s.cnt64[CNT_SURV] + nsam, cur = s.cnt64[CNT_CUR], age = s.cnt64[CNT_AGE] + 1;
-        const bool in_place = p.in_place && fits && age < RESORT && total + 4 * nsam + 4LL * m.nc <= p.capacity &&
-                              8 * nsam <= live && 4 * (total - live) <= live;
-        s.cnt64[CNT_SRC] = cur;
+        const bool in_place = p.in_place && fits && !pack && age < RESORT &&
+                              total + 4 * nsam + 4LL * m.nc <= p.capacity && 8 * nsam <= live && 4 * (total - live) <= live;
+        const long long src = pack ? 1 - cur : cur;
+        s.cnt64[CNT_PACK] = pack && fits ? slots : 0;
+        s.cnt64[CNT_PACKED] = 0;
+        if (pack) s.cnt64[CNT_N_A] = left;
+        s.cnt64[CNT_SRC] = src;
         s.cnt64[CNT_IN_PLACE] = in_place ? 1 : 0;
-        s.cnt64[CNT_CUR] = in_place ? cur : 1 - cur;
+        s.cnt64[CNT_CUR] = in_place ? src : 1 - src;
         s.cnt64[CNT_AGE] = in_place ? age : 0;
         s.cnt64[CNT_COLLIDED] = 0;
         s.cnt64[CNT_EXITED] = 0;

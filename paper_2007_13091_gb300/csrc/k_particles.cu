@@ -221,6 +221,54 @@ __device__ __forceinline__ float ff_position(const float* f, int nc, const float
     return s3 + lo;
 }
 
+// The live slots of the buffer that holds the particles (CNT_PACK slots, holes among
+// them) go to the start of the other one (their order changes no result): the rare
+// step in place too many, see CNT_PACK.  The samples' slots follow theirs, so that one
+// kernel writes both.
+template <class Real>
+__device__ __forceinline__ void pack_slots(const DevState& s, const PartBufs& bufs, Blk bk) {
+    const long long n = s.cnt64[CNT_PACK], left = s.cnt64[CNT_N_A];
+    if (n == 0) return;
+    // (one address per buffer, the arrays at their distances from the first one:
+    // the kernel takes 64 registers, the sampling alone 60; with an address per array 80)
+    char* const to = static_cast<char*>(bufs.b0.x[0]) + s.cnt64[CNT_SRC] * bufs.delta;
+    char* const from = static_cast<char*>(bufs.b0.x[0]) + s.cnt64[CNT_CUR] * bufs.delta;
+    auto at = [&](char* buffer, const void* array) {
+        return buffer + (static_cast<const char*>(array) - static_cast<const char*>(bufs.b0.x[0]));
+    };
+    auto move = [&](const void* array, auto type, long long i, long long j) {
+        using T = decltype(type);
+        reinterpret_cast<T*>(at(to, array))[j] = reinterpret_cast<const T*>(at(from, array))[i];
+    };
+    const int32_t* cells = reinterpret_cast<const int32_t*>(at(from, bufs.b0.cell));
+    const int lane = threadIdx.x & 31;
+    const long long stride = (long long)bk.n * blockDim.x;
+#pragma unroll 1
+    for (long long base = (long long)bk.id * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
+        const long long i = base + lane;
+        const bool live = i < n && cells[i] >= 0;
+        const unsigned mask = __ballot_sync(FULL, live);
+        unsigned long long first = 0;
+        if (lane == 0 && mask)
+            first = atomicAdd(reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_PACKED]), (unsigned long long)__popc(mask));
+        const long long j = (long long)__shfl_sync(FULL, first, 0) + __popc(mask & ((1u << lane) - 1u));
+        if (!live) continue;
+        if (j >= left) {
+            check_failed(s, 10, (unsigned long long)j);
+            continue;
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            move(bufs.b0.x[c], Real(), i, j);
+            move(bufs.b0.u[c], Real(), i, j);
+        }
+        move(bufs.b0.m, double(), i, j);
+        move(bufs.b0.cell, int32_t(), i, j);
+        move(bufs.b0.id, uint64_t(), i, j);
+        if (bufs.b0.e) move(bufs.b0.e, Real(), i, j);
+    }
+}
+
 // One lane per sample; cells sample even numbers, so that the two members of a
 // pair are lanes 2i and 2i + 1 and share the work of their normals (first-order
 // g_p: each particle on its own).  With energy-matched sampling a pair's
@@ -309,9 +357,12 @@ __device__ __forceinline__ void sample_write_body(const DevMesh& m, const DevSta
         b.id[j] = id;
     }
 }
-template <class Real>
+// DYN: the simulation may step in place.
+template <class Real, bool DYN>
 __global__ void __launch_bounds__(256) k_sample_write(DevMesh m, DevState s, DevParams p, PartBufs bufs) {
-    sample_write_body<Real>(m, s, p, bufs, Blk{(int)blockIdx.x, (int)gridDim.x});
+    const Blk bk{(int)blockIdx.x, (int)gridDim.x};
+    if constexpr (DYN) pack_slots<Real>(s, bufs, bk);
+    sample_write_body<Real>(m, s, p, bufs, bk);
 }
 
 // Energy-matched sampling: one factor per cell, s^2 sum_j |X_j|^2 = 3 N_sam / 2,
@@ -1101,8 +1152,9 @@ __global__ void __launch_bounds__(THREADS, TRACK_PER_SM<Real> / THREADS) k_track
 void launch_sample_write(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b,
                          int blocks, cudaStream_t st) {
     (void)m;
-    if (p.precision == UGKWP_MIXED) k_sample_write<float><<<blocks, 256, 0, st>>>(m, s, p, b);
-    else k_sample_write<double><<<blocks, 256, 0, st>>>(m, s, p, b);
+    if (p.precision != UGKWP_MIXED) k_sample_write<double, false><<<blocks, 256, 0, st>>>(m, s, p, b);
+    else if (b.dyn) k_sample_write<float, true><<<blocks, 256, 0, st>>>(m, s, p, b);
+    else k_sample_write<float, false><<<blocks, 256, 0, st>>>(m, s, p, b);
 }
 
 void launch_sample_scale(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, cudaStream_t st) {
@@ -1154,7 +1206,8 @@ template <class Real, bool KE> cudaError_t configure_type(int carveout) {
                 set(k_track<typename T::R, T::ke, T::threads, T::dyn>);
                 set(k_track_b<typename T::R, T::ke, T::threads>);
             });
-    set(k_sample_write<Real>);
+    set(k_sample_write<Real, false>);
+    if constexpr (sizeof(Real) == 4) set(k_sample_write<Real, true>);
     set(k_sample_scale<Real>);
     set(k_sample_write_b<Real>);
     set(k_sample_scale_b<Real>);

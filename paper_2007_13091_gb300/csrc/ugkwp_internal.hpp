@@ -53,7 +53,9 @@ enum : int {
     CNT_SRC = 18,       // the buffer this step's particles are in
     CNT_IN_PLACE = 19,  // this step leaves them there (1) or rewrites them sorted by cell (0)
     CNT_AGE = 20,       // steps in place since the particles were last sorted
+    CNT_PACK = 21,      // slots that this step packs into the other buffer before it samples (0: it does not pack)
     CNT_FLUX = 24,      // next tile of the wave flux's faces
+    CNT_PACKED = 28,    // slots packed
     CNT_TILE = 32,      // next run of tracking tiles
     CNT_IMPORT = 40,    // a state import's first failed particle: (index << 3) | problem
     CNT_OVF = 48,       // overflow slots (survivors whose bucket is full) taken this step
@@ -185,8 +187,10 @@ struct PartBufs {
 // drift into different cells (9% a step in a rarefied cavity), the removed
 // particles stay as holes and the samples follow in rows of their own.  The
 // particles are sorted every RESORT-th step, and whenever holes make up a fifth of
-// the slots, samples a ninth of the particles, or four times this step's samples
-// might not fit.  Two steps of a channel of 393,216 tets (6.7e7 particles): always
+// the slots, samples an eighth of the particles, or four times this step's samples
+// might not fit behind the slots.  Should the next step sample still more, it packs
+// the particles first (k_sample_write) and sorts, so that steps in place need no more
+// capacity than sorted ones.  Two steps of a channel of 393,216 tets (6.7e7 particles): always
 // sorted 5.98 ms, sorted every 2nd / 3rd / 4th / 6th / 12th step 5.59 / 5.43 / 5.29 /
 // 5.21 / 5.19 ms.
 constexpr int RESORT = 6;
