@@ -371,8 +371,13 @@ int ugkwp_autotune(ugkwp_sim* s, int32_t steps_per_trial, ugkwp_launch_cfg* best
  * launched on cuda_stream (NULL: the legacy default stream).  Each member
  * keeps its own state, random streams and results, bit for bit the same as
  * when stepped alone.  Members must be distinct; while stepped through a batch
- * a member is read or stepped on its own only after ugkwp_batch_sync.  The
- * batch does not own its members (free it before them). */
+ * a member is read or stepped on its own only after ugkwp_batch_sync, and the
+ * batch is stepped only once the member's own steps are done (ugkwp_sync).  The
+ * batch does not own its members (free it before them).  While it is in a
+ * batch, a mixed-precision member of a capacity of 2^25 particles or more sorts
+ * its particles in every step (otherwise it leaves them in place in most steps,
+ * which is faster and gives the same results); ugkwp_batch_create waits for
+ * such a member's stream. */
 typedef struct ugkwp_batch ugkwp_batch;
 
 int ugkwp_batch_create(ugkwp_sim* const* sims, int32_t n_sims, void* cuda_stream, ugkwp_batch** out);

@@ -3,6 +3,7 @@
 // kernel launches of one step, and state import/export.
 // This file is compiled with floating-point contraction disabled.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -34,6 +35,9 @@ struct ugkwp_sim {
     DevState S;
     PartBufRaw buf[2];  // the particle buffers
     int cur = 0;        // the one that holds the particles between steps, unless the device knows (P.in_place)
+    bool may_in_place = false;  // steps in place, except while it is in a batch
+    // the batches it is in (shared with them: they may outlive it)
+    std::shared_ptr<std::atomic<int>> batches = std::make_shared<std::atomic<int>>(0);
     // the buffers as the kernels of the next step take them
     PartBufs bufs() const {
         const int k = P.in_place ? 0 : cur;
@@ -434,7 +438,8 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
     P.N_ref = p->N_ref; P.N_min = p->N_min; P.max_crossings = p->max_crossings; P.precision = p->precision;
     P.order = p->order;
     P.sampling = p->sampling;
-    P.in_place = p->precision == UGKWP_MIXED && p->particle_capacity >= IN_PLACE_CAPACITY;
+    s->may_in_place = p->precision == UGKWP_MIXED && p->particle_capacity >= IN_PLACE_CAPACITY;
+    P.in_place = s->may_in_place;
     P.K = p->K;
     P.seed = p->seed; P.capacity = p->particle_capacity; P.n_bc = p->n_bc;
     for (int b = 0; b < p->n_bc; ++b) {
@@ -958,6 +963,11 @@ extern "C" {
 int ugkwp_step(ugkwp_sim* s, int32_t n_steps, ugkwp_stats* st) {
     if (!s || n_steps < 0) return fail(UGKWP_E_ARG, "invalid argument");
     cudaStream_t q = s->stream;
+    if (s->may_in_place && !s->P.in_place && s->batches->load() == 0) {
+        // out of its last batch (CNT_CUR has followed the steps that sorted)
+        s->P.in_place = 1;
+        s->drop_graphs();
+    }
     for (int32_t k = 0; k < n_steps;) {
         if (s->step >= ((int64_t)1 << 24) - 2) return fail(UGKWP_E_STATE, "step counter exhausted (2^24 steps)");
         if (n_steps - k >= 2) {
@@ -1734,6 +1744,7 @@ struct ugkwp_batch {
     std::vector<ugkwp_sim*> sims;
     cudaStream_t stream = nullptr;
     std::vector<cudaStream_t> lanes;
+    std::vector<std::shared_ptr<std::atomic<int>>> joined;  // the members' counts of their batches
     cudaEvent_t fork = nullptr;
     std::vector<cudaEvent_t> join;
     std::vector<std::unique_ptr<FusedChunk>> chunks;
@@ -1752,6 +1763,7 @@ struct ugkwp_batch {
     ~ugkwp_batch() {
         if (stream) cudaStreamSynchronize(stream);
         drop_graphs();
+        for (auto& n : joined) n->fetch_sub(1);
         for (auto e : join) if (e) cudaEventDestroy(e);
         if (fork) cudaEventDestroy(fork);
         for (auto l : lanes) if (l) cudaStreamDestroy(l);
@@ -1958,18 +1970,6 @@ int ugkwp_batch_create(ugkwp_sim* const* sims, int32_t n_sims, void* cuda_stream
     std::sort(sorted.begin(), sorted.end());
     if (std::adjacent_find(sorted.begin(), sorted.end()) != sorted.end())
         return fail(UGKWP_E_ARG, "a simulation appears twice in the batch");
-    // the fused tracking has no registers to spare for steps in place (a batch of
-    // 14 members 8.02 against 7.35 ms): from here on every member sorts, with the
-    // buffer that holds its particles known on the host
-    for (auto* s : v) {
-        if (!s->P.in_place) continue;
-        int spare = 0;
-        int rc = spare_buffer(s, spare);
-        if (rc) return rc;
-        s->cur = 1 - spare;
-        s->P.in_place = 0;
-        s->drop_graphs();
-    }
     ugkwp_batch* b = new ugkwp_batch;
     b->sims = v;
     b->stream = (cudaStream_t)cuda_stream;
@@ -2010,6 +2010,27 @@ int ugkwp_batch_create(ugkwp_sim* const* sims, int32_t n_sims, void* cuda_stream
     if (ce != cudaSuccess) {
         delete b;
         return cuda_fail(ce, "ugkwp_batch_create");
+    }
+    // the fused tracking has no registers to spare for steps in place (a batch of
+    // 14 members 8.02 against 7.35 ms): while it is in a batch a member sorts, with
+    // the buffer that holds its particles known on the host
+    std::vector<int> spare(v.size(), 0);
+    for (size_t i = 0; i < v.size(); ++i) {
+        if (!v[i]->P.in_place) continue;
+        int rc = spare_buffer(v[i], spare[i]);
+        if (rc) {
+            delete b;
+            return rc;
+        }
+    }
+    for (size_t i = 0; i < v.size(); ++i) {
+        ugkwp_sim* s = v[i];
+        b->joined.push_back(s->batches);
+        s->batches->fetch_add(1);
+        if (!s->P.in_place) continue;
+        s->cur = 1 - spare[i];
+        s->P.in_place = 0;
+        s->drop_graphs();
     }
     *out = b;
     return UGKWP_OK;

@@ -73,3 +73,52 @@ def test_samples_past_the_slots(sampling, K):
         assert np.array_equal(a[k][oa], b[k][ob]), k
     for k in ("x", "u"):
         assert np.array_equal(a[k][:, oa], b[k][:, ob]), k
+
+
+def test_members_step_in_place_again_after_their_batches():
+    """A member sorts while it is in a batch, and steps in place as before once its
+    last batch is freed: the particles of its image then lie out of cell order.
+    Everything equals, bit for bit, a simulation that was in no batch."""
+    import torch
+    from paper_2007_13091_gb300 import ugkwp
+    cfg = wl.cavity(n=6, Kn=0.3, N_ref=80, precision="mixed", order=2)
+    cfg["params"]["particle_capacity"] = 1 << 25
+    a, b = (ugkwp.Simulation(cfg["mesh"], cfg["W0"], cfg["params"], stream=torch.cuda.Stream()) for _ in range(2))
+
+    def backward_steps():  # in cell order from slot to slot; only overflow slots when sorted
+        x, y = a.state_native(), b.state_native()
+        ox, oy = np.argsort(x["id"]), np.argsort(y["id"])
+        for k in ("id", "cell", "m"):
+            assert np.array_equal(x[k][ox], y[k][oy]), k
+        for k in ("x", "u"):
+            assert np.array_equal(x[k][:, ox], y[k][:, oy]), k
+        assert np.array_equal(x["W"], y["W"])
+        assert np.array_equal(a.moments(ugkwp.WP), b.moments(ugkwp.WP))
+        return [int((np.diff(s["cell"]) < 0).sum()) for s in (x, y)]
+
+    a.step(5)
+    b.step(5)
+    inplace = backward_steps()[1]
+    assert inplace > 1000
+    one = ugkwp.Batch([a])
+    two = ugkwp.Batch([a])
+    one.step(3)
+    one.sync()
+    one.close()
+    a.step(2)  # alone, but still in the second batch
+    a.sync()
+    two.step(2)
+    two.sync()
+    b.step(7)
+    assert backward_steps()[0] < 100
+    two.close()
+    for n in (1, 2, 2):
+        a.step(n)
+        b.step(n)
+        got = backward_steps()
+    assert got[0] > 1000
+    never = ugkwp.Batch([a])  # created and freed between steps in place
+    never.close()
+    a.step(3)
+    b.step(3)
+    backward_steps()
