@@ -343,7 +343,8 @@ enum {
  * speed does. */
 typedef struct {
     int32_t particle_blocks;     /* blocks of the sampling and tracking kernels (> 0) */
-    int32_t wave_blocks;         /* blocks of the persistent second-order wave kernels (> 0) */
+    int32_t wave_blocks;         /* blocks of the second-order wave flux kernel (> 0; default one per
+                                  * SM, for which second-order start-up steps take two per SM) */
     int32_t track_threads;       /* threads per block of the tracking kernel: 128 or 256 */
     int32_t smem_carveout;       /* preferred shared-memory carveout of the step's kernels, percent of
                                   * the largest (0..100), or -1 for the driver's choice (default 58).

@@ -49,3 +49,22 @@ def test_batch_members_share_the_blocks(order):
         y.step(3)
         _assert_same(x, y)
     b.close()
+
+
+def test_wave_blocks_hold_in_start_up_steps():
+    """Second-order start-up steps take the grid the caller chose: four blocks, on
+    four of the chip's SMs, take far longer (some 38 times, bound by the binary64
+    pipe; at least 5 is asked) than the default, with the same bits."""
+    import torch
+    cfg = _cfg(24, 2, 5)
+    few, default = _sim(cfg, torch.cuda.Stream()), _sim(cfg, torch.cuda.Stream())
+    d = ugkwp.ugkwp_get_launch_cfg(few.handle)
+    ugkwp.ugkwp_set_launch_cfg(few.handle, d["particle_blocks"], 4, d["track_threads"], d["smem_carveout"])
+    ms = []
+    for s in (few, default):
+        s.gks_steps(3)
+        ugkwp.ugkwp_timing_enable(s.handle, True)
+        s.gks_steps(5)
+        ms.append(ugkwp.ugkwp_timing_read(s.handle)[0]["flux_o2"])
+    _assert_same(few, default)
+    assert ms[0] > 5 * ms[1]
