@@ -172,7 +172,6 @@ void layout(const MeshHost& mh, int64_t cap, size_t rs, bool with_e, Carver& c, 
     M.lsq_dxf = c.take<double>(12 * nc);
     M.f_dx = c.take<double>(6 * nf);
     M.eps2 = c.take<double>(nc);
-    M.f_lk = c.take<int32_t>(nf);
     M.f_own = c.take<int32_t>(nf);
     M.f_nbr = c.take<int32_t>(nf);
     M.f_n = c.take<double>(3 * nf);
@@ -342,8 +341,6 @@ int read_error(ugkwp_sim* s) {
     if (e & ERRB_TRACK_LIMIT) return fail(UGKWP_E_TRACK_LIMIT, std::to_string(h[CNT_LOST]) + " particles exceeded max_crossings");
     if (e & ERRB_FIXED_OVERFLOW) return fail(UGKWP_E_FIXED_OVERFLOW, "fixed-point particle flux overflow");
     if (e & ERRB_SAMPLE_LIMIT) return fail(UGKWP_E_CAPACITY, "more than 65534 particles sampled in one cell");
-    if (e & ERRB_SORT)
-        return fail(UGKWP_E_STATE, "survivor counts per cell disagree with the survivors: the particle state is not valid");
     if (e & ERRB_CHECK)
         return fail(UGKWP_E_STATE, "a kernel's bounds or alignment check failed (check " + std::to_string(h[CNT_CHECK] >> 48) +
                                    ", value " + std::to_string(h[CNT_CHECK] & 0xffffffffffffLL) + "); the access was skipped");
@@ -478,7 +475,6 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
     // c_k = A^-1 w_k dx_k, A = sum_k w_k dx_k dx_k^T.  Also the centroid-to-face
     // vectors and epsilon^2 = (K |Omega|^(1/3))^3 of Venkatakrishnan's limiter.
     std::vector<double> lsq_c(12 * (size_t)nc), lsq_dxf(12 * (size_t)nc), eps2(nc), fdx(6 * (size_t)nf, 0.0);
-    std::vector<int32_t> flk(nf, 0);
     for (int i = 0; i < nc; ++i) {
         double xi[3] = {0.0, 0.0, 0.0};
         for (int k = 0; k < 4; ++k)
@@ -508,8 +504,6 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
             w[k] = 1.0 / (dx[k][0] * dx[k][0] + dx[k][1] * dx[k][1] + dx[k][2] * dx[k][2]);
             for (int r = 0; r < 3; ++r)
                 for (int cc = 0; cc < 3; ++cc) A[r][cc] += w[k] * dx[k][r] * dx[k][cc];
-            if (own) flk[f] |= k;
-            else flk[f] |= k << 2;
         }
         // inverse of the symmetric 3x3 matrix by cofactors
         double C[3][3];
@@ -706,7 +700,6 @@ int ugkwp_init(const ugkwp_mesh* m, const ugkwp_params* p, const double* W0, voi
     UP(s->M.lsq_dxf, lsq_dxf.data(), lsq_dxf.size() * sizeof(double));
     UP(s->M.f_dx, fdx.data(), fdx.size() * sizeof(double));
     UP(s->M.eps2, eps2.data(), eps2.size() * sizeof(double));
-    UP(s->M.f_lk, flk.data(), flk.size() * sizeof(int32_t));
     UP(s->M.f_own, mh.f_own.data(), nf * sizeof(int32_t));
     UP(s->M.f_nbr, fnb.data(), nf * sizeof(int32_t));
     UP(s->M.f_n, fn.data(), fn.size() * sizeof(double));

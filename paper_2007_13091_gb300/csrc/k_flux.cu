@@ -50,22 +50,14 @@ namespace {
 constexpr int GRAD_THREADS = 128, GRAD_BLOCKS_PER_SM = 2;
 
 // Constants of K internal degrees of freedom (rho E = rho |U|^2/2 + (3+K)/2 p,
-// <|xi|^2> = K theta, <|xi|^4> = K (K+2) theta^2, theta = 1/(2 lambda)); for
-// K = 0 each is the monatomic literal (2/3, 4/3, 1/3, 3, 5/2, 5, 7) exactly.
+// <|xi|^2> = K theta, theta = 1/(2 lambda)); for K = 0 each is the monatomic
+// literal (4/3, 1/3, 3, 5/2) exactly.
 struct KC {
-    double K, c23, c43, c13, e3, e5h, e5, e7;
+    double c43, c13, e3, e5h;
 };
 __device__ __forceinline__ KC kconst(int K) {
-    KC k;
-    k.K = (double)K;
-    k.c23 = 2.0 / (3.0 + k.K);
-    k.c43 = 4.0 / (3.0 + k.K);
-    k.c13 = 1.0 / (3.0 + k.K);
-    k.e3 = 3.0 + k.K;
-    k.e5h = 0.5 * (5.0 + k.K);
-    k.e5 = 5.0 + k.K;
-    k.e7 = 7.0 + k.K;
-    return k;
+    const double e3 = 3.0 + (double)K;
+    return KC{4.0 / e3, 1.0 / e3, e3, 0.5 * (5.0 + (double)K)};
 }
 
 __device__ __forceinline__ double dot3(const double* a, const double* b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; }

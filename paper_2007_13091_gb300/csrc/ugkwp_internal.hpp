@@ -18,7 +18,6 @@ enum : int32_t {
     ERRB_FIXED_OVERFLOW = 4,
     ERRB_NONFINITE = 8,
     ERRB_SAMPLE_LIMIT = 16,
-    ERRB_SORT = 64,         // a cell holds more survivors than its count (sort skipped them)
     ERRB_CHECK = 128,       // a kernel's own bounds or alignment check failed (the access was skipped;
                             // CNT_CHECK holds the check and the value)
 };
@@ -139,7 +138,6 @@ struct DevMesh {
     const double* lsq_dxf;   // [12][nc]: face centroid minus cell centroid for local face k
     const double* f_dx;      // [6][nf] face centroid minus the owner's, the neighbour's centroid
     const double* eps2;      // [nc] Venkatakrishnan epsilon^2 = (K h)^3
-    const int32_t* f_lk;     // [nf] owner's local face | neighbour's local face << 2
     const int32_t* face_order;  // [nf] interior faces, then boundary faces grouped by type
     const int32_t* f_own;    // [nf]
     const int32_t* f_nbr;    // [nf] >= 0 tet, else -1 - boundary index
