@@ -1,7 +1,8 @@
-// Second-order wave flux of one interior face (Sec. 2.1, 2.3) in the lab frame,
-// and the product of its Jacobian's transpose with a given face vector
-// (hand-written reverse pass): plain functions of scalars, used by the step's
-// flux kernel and by the adjoint kernels.
+// The wave flux of a face in the lab frame (Sec. 2.1, 2.3): second order for an
+// interior face, first order for a boundary face or a first-order step, and for each
+// the product of its Jacobian's transpose with a given face vector (hand-written
+// reverse pass).  Plain functions of scalars, used by the step's flux kernels and by
+// the adjoint kernels; they compile for the host as well.
 //
 // Every slope moment of the flux is the derivative of a Maxwellian moment
 // along the gradient of the primitive state (rho, U, theta = RT): for a
@@ -171,8 +172,12 @@ UGKWP_HD SideFlux side_flux(const Prim& s, const PrimGrad& pg, double rh, const 
     return o;
 }
 
-// q1..q5, a4, a5 (time integrals of Sec. 2.1) from one expm1; their absolute
-// errors stay at rounding level of dt and dt^2, the scales at which they enter.
+// q1..q5, a4, a5 (time integrals of Sec. 2.1) from one expm1.  q1, q4 and a4 are
+// differences of terms of size dt, and carry absolute errors of some 2^-52 dt; q2, q3,
+// q5 and a5 are differences of terms of size tau dt, with errors of some
+// 2^-52 dt max(tau, dt): far below dt^2, the scale at which they enter the flux, as long as
+// tau/dt is far below 2^52 (1e-12 dt^2 at dt/tau = 1e-4, 1e-8 dt^2 at 1e-8), but not
+// relative to their own values, which fall as dt^3/tau.
 struct QC {
     double q1, q2, q3, q4, q5, a4, a5, e;
 };
@@ -526,7 +531,9 @@ UGKWP_HD void flux_o1_adj(const Prim& L, double rhL, const Prim& R, double rhR, 
     }
 }
 
-// d/dtau of the time coefficients, contracted with their adjoints.
+// d/dtau of the time coefficients, contracted with their adjoints.  Absolute errors of
+// some 2^-52 dt in the derivatives of q2, q3 and a5, of 2^-52 dt/tau in those of q1, q4
+// and a4, by the same differences.
 UGKWP_HD double time_coeffs_adj(const QC& c, double dt, double tau, double q1b, double q2b, double q3b, double q4b,
                                 double a4b, double a5b) {
     const double x = dt / tau, xe = x * c.e, dq4 = c.a4 / tau;
@@ -535,8 +542,8 @@ UGKWP_HD double time_coeffs_adj(const QC& c, double dt, double tau, double q1b, 
            q3b * (c.q4 + tau * dq4 - dt) + a4b * (dq4 - x * xe) + a5b * (dq5 + 0.5 * dt * x * xe);
 }
 
-// Adjoint of equilibrium_flux: W0b += , Bb (of B itself) += , qb = adjoints of
-// q1, q2, q3 (+=); s_b the state's adjoints that stem from other uses of W0.
+// Adjoint of equilibrium_flux: a += (the adjoint of the primitive state), E_b += (of the
+// energy W0[4]), Bb += (of B itself), qb += (of q1, q2, q3).
 UGKWP_HD void equilibrium_flux_adj(const double* W0, const Prim& s, const double B[5][3], double scale,
                                    const double n[3], const QC& c, double pr_fix, const Gas& gas, const double Fb[5],
                                    PrimAdj& a, double& E_b, double Bb[5][3], double qb[3]) {
