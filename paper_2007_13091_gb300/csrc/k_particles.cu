@@ -686,8 +686,9 @@ constexpr int WALK_QUEUE = 64;
 constexpr int DEFER_LOG = 8;
 // Threads per SM the tracking kernel is compiled for: 64 registers in mixed mode
 // (80: 1.82 ms against 1.69 ms for two steps of the 24^3 cavity, whose wave flux
-// leaves room for four such blocks per SM), 96 in binary64 (a 20-step run of a tube
-// of 9,600 tets 4.43 ms against 4.71 ms with 64).
+// leaves room for four such blocks per SM); in binary64 five blocks of 128 threads
+// with 96 registers (a 20-step run of a tube of 9,600 tets 4.43 ms against 4.71 ms
+// with 64), or two of 256 with up to 128.
 template <class Real> constexpr int TRACK_PER_SM = sizeof(Real) == 4 ? 1024 : 640;
 
 // The planes of a tet in binary32, for the inside test: in mixed mode those of

@@ -192,10 +192,14 @@ struct PartBufs {
 // sorted 5.98 ms, sorted every 2nd / 3rd / 4th / 6th / 12th step 5.59 / 5.43 / 5.29 /
 // 5.21 / 5.19 ms.
 constexpr int RESORT = 6;
-// Mixed-mode simulations of at least this particle capacity may step in place: a
-// smaller one is bound by latencies, to which the extra indirection adds (tube of
-// 1,992 tets 62.4 against 60.5 us, 16^3 cavity of 3e6 particles 487 against 475 us
-// for two steps; 24^3 cavity of 1.9e7 1.60 against 1.64 ms), binary64 by its pipe.
+// Mixed-mode simulations of at least this particle capacity may step in place.  The
+// host chooses the kernels before there are any particles, and the capacity is what it
+// knows of their number.  In place pays where the tracking is bound by what it moves
+// (two steps of the 24^3 cavity, 1.7e7 particles in a capacity of 4.7e7, 1.60 against
+// 1.64 ms); a simulation of few particles is bound by latencies, to which the
+// indirection adds, whatever its buffer (tube of 1,992 tets 62.4 against 60.5 us, 16^3
+// cavity of 3e6 particles 487 against 475 us).  Binary64 is bound by its pipe and
+// always sorts.
 constexpr int64_t IN_PLACE_CAPACITY = (int64_t)1 << 25;
 
 struct DevState {
