@@ -9,6 +9,7 @@
 //                   counting flux of the particles that left their cell or met a
 //                   wall, removal; each survivor is written into the bucket of
 //                   its end cell in the next buffer.
+#include <algorithm>
 #include <type_traits>
 
 #include "dmath.cuh"
@@ -684,6 +685,8 @@ constexpr int WALK_QUEUE = 64;
 // logarithm to the queue: two steps of the 21^3 cavity in binary64 2.22 ms with 4,
 // 8 or 16 against 2.52 ms with none.
 constexpr int DEFER_LOG = 8;
+// Slots of a run of tiles at most.
+constexpr unsigned TRACK_RUN_MAX = 512;
 // Threads per SM the tracking kernel is compiled for: 64 registers in mixed mode
 // (80: 1.82 ms against 1.69 ms for two steps of the 24^3 cavity, whose wave flux
 // leaves room for four such blocks per SM); in binary64 five blocks of 128 threads
@@ -753,7 +756,7 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u, upto = FULL >> (31 - lane);
     const int nc = m.nc;
-    unsigned* tile_ctr = reinterpret_cast<unsigned*>(&s.cnt64[CNT_TILE]);  // (the low word)
+    unsigned long long* tile_ctr = reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_TILE]);
     unsigned long long* smass = reinterpret_cast<unsigned long long*>(s.smass_next);
     unsigned long long* pf = reinterpret_cast<unsigned long long*>(s.pflux);
     // warp-uniform counters
@@ -912,18 +915,14 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
 
     // tiles per run: long enough that the counter is off the path, short enough
     // that a small simulation spreads over the whole grid
-    const unsigned run = min(max(n / (32u * 8192u), 1u), 16u) * 32u;
-    // (the largest grid hands out fewer than 2^27 runs, but their slots can pass 2^32:
-    // such a run starts at n)
-    auto first_of = [&](unsigned number) {
-        const unsigned k = __shfl_sync(FULL, number, 0);
-        return __umulhi(k, run) ? n : k * run;
-    };
-    unsigned ahead = 0, base = 0, end = 0;
-    if (lane == 0) ahead = atomicAdd(tile_ctr, 1u);
-    base = first_of(ahead);
+    const unsigned run = min(max(n / (32u * 8192u), 1u), TRACK_RUN_MAX / 32u) * 32u;
+    // (slots in 32 bits: see track_blocks)
+    unsigned long long ahead = 0;
+    unsigned base = 0, end = 0;
+    if (lane == 0) ahead = atomicAdd(tile_ctr, 1ULL);
+    base = (unsigned)__shfl_sync(FULL, ahead, 0) * run;
     end = base + run;
-    if (lane == 0) ahead = atomicAdd(tile_ctr, 1u);
+    if (lane == 0) ahead = atomicAdd(tile_ctr, 1ULL);
     // the first lanes prefetch the lines of the next tile's x, u, m and id (its
     // cells are loaded), one line per lane, with one instruction per tile
     constexpr int XL = sizeof(Real) / 4;  // lines per coordinate array
@@ -970,9 +969,9 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
         // the next tile's cells (its other loads follow at the top of its turn)
         unsigned nbase = base + 32;
         if (nbase == end) {
-            nbase = first_of(ahead);
+            nbase = (unsigned)__shfl_sync(FULL, ahead, 0) * run;
             end = nbase + run;
-            if (lane == 0 && nbase < n) ahead = atomicAdd(tile_ctr, 1u);
+            if (lane == 0 && nbase < n) ahead = atomicAdd(tile_ctr, 1ULL);
         }
         if (nbase < n) {
             cell_i = b.cell[nbase + lane];
@@ -1183,13 +1182,22 @@ template <class F> void track_kind(int precision, bool ke, bool dyn, int threads
     else if (dyn) ke ? shape(0.0f, T{}, T{}) : shape(0.0f, N{}, T{});
     else ke ? shape(0.0f, T{}, N{}) : shape(0.0f, N{}, N{});
 }
+// Blocks of one of a step's two tracking launches.  A warp reserves up to two runs
+// past the end, so that the slots of all runs stay below n + 2 TRACK_RUN_MAX per warp
+// (n < 2^31): two launches of fewer than 2^20 warps keep them below 2^32, in which the
+// kernel counts.  (With a check in the kernel a step pair of the batch of 14 members
+// took 7.20 ms instead of 7.11, of the 16^3 cavity with g_p sampling 564 us instead of 561.)
+int track_blocks(int blocks, int threads) {
+    constexpr int WARPS = int((1u << 31) / (4 * TRACK_RUN_MAX));
+    return std::min(blocks, (WARPS - 1) / (threads / 32));
+}
 }  // namespace
 
 void launch_track(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& b, const TrackShape& sh,
                   int blocks, cudaStream_t st) {
     track_kind(p.precision, p.K > 0, b.dyn != 0, sh.threads, [&](auto k) {
         using T = decltype(k);
-        k_track<typename T::R, T::ke, T::threads, T::dyn><<<blocks, T::threads, 0, st>>>(m, s, p, b);
+        k_track<typename T::R, T::ke, T::threads, T::dyn><<<track_blocks(blocks, T::threads), T::threads, 0, st>>>(m, s, p, b);
     });
 }
 
@@ -1233,7 +1241,7 @@ void launch_track_batch(const BatchChunk& c, int precision, bool ke, const Track
                         cudaStream_t st) {
     track_kind(precision, ke, false, sh.threads, [&](auto k) {
         using T = decltype(k);
-        k_track_b<typename T::R, T::ke, T::threads><<<blocks, T::threads, 0, st>>>(c);
+        k_track_b<typename T::R, T::ke, T::threads><<<track_blocks(blocks, T::threads), T::threads, 0, st>>>(c);
     });
 }
 
