@@ -738,7 +738,11 @@ template <class Real, int THREADS> struct TrackShared {
     Real q_end[THREADS / 32][WALK_QUEUE];  // t_f, or dt; -1: not drawn yet
     unsigned red[THREADS / 32][8];
 };
-template <class Real, bool KE, int THREADS, bool IN_PLACE>
+// Number: the type of the runs' numbers (fewer than 2^27, see track_blocks).  32 bits in
+// the kernel of one simulation (20 binary64 steps of a tube of 9,600 tets 1% faster than
+// with 64), 64 in the fused one, which then spills less (a batch of 14 members 7.08
+// against 7.18 ms).
+template <class Real, bool KE, int THREADS, bool IN_PLACE, class Number>
 __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& bufs,
                                            long long src, TrackShared<Real, THREADS>& sh) {
     constexpr int NW = THREADS / 32;
@@ -756,7 +760,7 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u, upto = FULL >> (31 - lane);
     const int nc = m.nc;
-    unsigned long long* tile_ctr = reinterpret_cast<unsigned long long*>(&s.cnt64[CNT_TILE]);
+    Number* tile_ctr = reinterpret_cast<Number*>(&s.cnt64[CNT_TILE]);  // (or its low word)
     unsigned long long* smass = reinterpret_cast<unsigned long long*>(s.smass_next);
     unsigned long long* pf = reinterpret_cast<unsigned long long*>(s.pflux);
     // warp-uniform counters
@@ -916,13 +920,12 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
     // tiles per run: long enough that the counter is off the path, short enough
     // that a small simulation spreads over the whole grid
     const unsigned run = min(max(n / (32u * 8192u), 1u), TRACK_RUN_MAX / 32u) * 32u;
-    // (slots in 32 bits: see track_blocks)
-    unsigned long long ahead = 0;
+    Number ahead = 0;
     unsigned base = 0, end = 0;
-    if (lane == 0) ahead = atomicAdd(tile_ctr, 1ULL);
+    if (lane == 0) ahead = atomicAdd(tile_ctr, Number(1));
     base = (unsigned)__shfl_sync(FULL, ahead, 0) * run;
     end = base + run;
-    if (lane == 0) ahead = atomicAdd(tile_ctr, 1ULL);
+    if (lane == 0) ahead = atomicAdd(tile_ctr, Number(1));
     // the first lanes prefetch the lines of the next tile's x, u, m and id (its
     // cells are loaded), one line per lane, with one instruction per tile
     constexpr int XL = sizeof(Real) / 4;  // lines per coordinate array
@@ -971,7 +974,7 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
         if (nbase == end) {
             nbase = (unsigned)__shfl_sync(FULL, ahead, 0) * run;
             end = nbase + run;
-            if (lane == 0 && nbase < n) ahead = atomicAdd(tile_ctr, 1ULL);
+            if (lane == 0 && nbase < n) ahead = atomicAdd(tile_ctr, Number(1));
         }
         if (nbase < n) {
             cell_i = b.cell[nbase + lane];
@@ -1094,23 +1097,23 @@ __device__ __forceinline__ void track_mode(const DevMesh& m, const DevState& s, 
     }
 }
 // DYN: the simulation may step in place.
-template <class Real, bool KE, int THREADS, bool DYN>
+template <class Real, bool KE, int THREADS, bool DYN, class Number>
 __device__ __forceinline__ void track_body(const DevMesh& m, const DevState& s, const DevParams& p, const PartBufs& bufs) {
     __shared__ TrackShared<Real, THREADS> sh;
     // (block-uniform: another block may set the bit while this one starts)
     if (__syncthreads_or(threadIdx.x == 0 && (s.cnt64[CNT_ERR] & ERRB_CAPACITY))) return;
     if constexpr (DYN) {
         const long long src = s.cnt64[CNT_SRC] * bufs.delta;
-        if (s.cnt64[CNT_IN_PLACE]) track_mode<Real, KE, THREADS, true>(m, s, p, bufs, src, sh);
-        else track_mode<Real, KE, THREADS, false>(m, s, p, bufs, src, sh);
+        if (s.cnt64[CNT_IN_PLACE]) track_mode<Real, KE, THREADS, true, Number>(m, s, p, bufs, src, sh);
+        else track_mode<Real, KE, THREADS, false, Number>(m, s, p, bufs, src, sh);
     } else {
-        track_mode<Real, KE, THREADS, false>(m, s, p, bufs, 0, sh);
+        track_mode<Real, KE, THREADS, false, Number>(m, s, p, bufs, 0, sh);
     }
 }
 template <class Real, bool KE, int THREADS, bool DYN>
 __global__ void __launch_bounds__(THREADS, TRACK_PER_SM<Real> / THREADS) k_track(DevMesh m, DevState s, DevParams p,
                                                                                  PartBufs bufs) {
-    track_body<Real, KE, THREADS, DYN>(m, s, p, bufs);
+    track_body<Real, KE, THREADS, DYN, unsigned>(m, s, p, bufs);
 }
 
 // ---- fused batches
@@ -1142,7 +1145,7 @@ template <class Real, bool KE, int THREADS>
 __global__ void __launch_bounds__(THREADS, TRACK_PER_SM<Real> / THREADS) k_track_b(const __grid_constant__ BatchChunk c) {
     for (int k = 0; k < c.n; ++k) {
         const BatchMember& e = c.mem[((int)blockIdx.x + k) % c.n];
-        track_body<Real, KE, THREADS, false>(e.m, e.s, e.p, e.bufs);
+        track_body<Real, KE, THREADS, false, unsigned long long>(e.m, e.s, e.p, e.bufs);
         __syncthreads();
     }
 }
